@@ -142,8 +142,8 @@ luna_status make_plan(const luna_attn_desc *ad, const luna_phi_desc *pd, Plan &p
         }
         p.ws_fwd = w.n;
         // per-head partial slots: generic splits, or (tensor-core path) runs of work items, never more
-        // than the forward split count
-        const size_t nslot = (size_t)std::max(p.nsplit, p.nsplit_b);
+        // than the forward split count; the generic kernels' partials are pairs
+        const size_t nslot = (size_t)std::max(p.nsplit, 2 * p.nsplit_b);
         p.o_dSpart = w.take((size_t)BH * nslot * SD * f);
         p.o_dzpart = w.take((size_t)BH * nslot * D * f);
         p.o_dSfin = w.take((size_t)BH * SD * f);
@@ -175,7 +175,7 @@ luna_status make_plan(const luna_attn_desc *ad, const luna_phi_desc *pd, Plan &p
         p.o_dzpart = w.take((size_t)BH * ns * D * f);
         p.o_segdS = w.take((size_t)BH * ns * SD * f);
         p.o_segdz = w.take((size_t)BH * ns * D * f);
-        p.o_rowstat = w.take((size_t)BH * n * 2 * f);
+        p.o_rowstat = w.take((size_t)BH * n * 4 * f);
         p.o_gpart = w.take((2 * (size_t)BH * ns + (p.ch_target > 0.0f ? 2 * kChKBlocks : 0)) * p.gsize *
                            sizeof(double));
         p.o_hist = w.take((size_t)p.gsize * sizeof(double));

@@ -1,4 +1,4 @@
-// Streaming (causal) form on CUDA cores (fp32 arithmetic).
+// Streaming (causal) form on CUDA cores (fp32 arithmetic, sums as pairs of floats).
 //
 // The paper names the associative streaming form of kernel attention (abstract,
 // Sec. 3.2, Conclusion) without writing it out; it is the prefix recurrence
@@ -6,195 +6,260 @@
 //     O_i = phi(q_i)^T S_i / (phi(q_i)^T z_i + eps).
 // Rows are cut into state segments.  The prefix statistics at every segment
 // start come from an exclusive scan of per-segment sums (key-statistics kernel
-// in scan mode); inside a segment the rows are processed in sub-chunks of kCs
-// rows: a masked intra-chunk term tril(phi(Q) phi(K)^T) V plus the carried
-// state, then the state advances by the chunk's phi(K)^T V.
+// in scan mode); inside a segment the rows are processed in tiles of up to 64
+// rows: a masked intra-tile term tril(phi(Q) phi(K)^T) V plus the carried
+// state, then the state advances by the tile's phi(K)^T V.
 //
 // Backward (derived from the same recurrence):
 //   dnum_i = do_i / den_i, dden_i = -(do_i . o_i)/den_i
 //   dphi(q_i) = S_i dnum_i + z_i dden_i
 //   G_j = sum_{i>=j} phi(q_i) dnum_i^T, g_j = sum_{i>=j} phi(q_i) dden_i
 //   dv_j = G_j^T phi(k_j),  dphi(k_j) = G_j v_j + g_j
-// A forward sweep per segment records (den_i, dden_i) and the segment sums of
-// G; a reverse exclusive scan gives G after every segment; then one forward
-// sweep produces dQ and one reverse sweep produces dK and dV.
+// A forward sweep per segment records (den_i, dden_i), produces dQ and the
+// segment sums of G; a reverse exclusive scan gives G after every segment; then
+// a reverse sweep produces dK and dV.
 #include <math.h>
 
 #include "luna_prof.cuh"
-#include "luna_simt_dev.cuh"
+#include "luna_tile.cuh"
 
 namespace luna {
 namespace {
 using namespace simt;
 
-constexpr int kCs = 16;  // rows per sub-chunk
+// Measured at 8 x 12 heads of 1024 bf16 rows, d = D = 64 (us; before: fp64 sums, tiles of 16 rows, and separate
+// sweeps for the segment sums and dQ): outputs 5918 -> 326, backward queries 16081 -> 937, backward keys
+// 6861 -> 606, with the key statistics 2715 -> 177.
+//
+// Each kernel walks its segment in tiles of `cap` rows (luna_tile.cuh).  The running state is held in fp32 in
+// shared memory and advances once per tile from pairs of floats, so a tile of 64 rows rounds it a quarter as
+// often as one of 16.
 
-struct ChunkBufs {
-    float *Q, *K, *V, *dO, *Pq, *Pk, *A, *P, *den, *dden;
-};
-
-template <typename IO>
-__device__ void load_chunk(const AttnArgs &a, int bh, int t0, int nr, float *sQ, float *sK, float *sV, float *sdO) {
-    const size_t r0 = head_rows(a, bh) + t0;
-    load_rows(sQ, static_cast<const IO *>(a.Q) + r0 * a.d, nr * a.d);
-    load_rows(sK, static_cast<const IO *>(a.K) + r0 * a.d, nr * a.d);
-    load_rows(sV, static_cast<const IO *>(a.V) + r0 * a.dv, nr * a.dv);
-    if (sdO) load_rows(sdO, static_cast<const IO *>(a.dO) + r0 * a.dv, nr * a.dv);
-}
-
-// sA[r][j] = phi(q_r) . phi(k_j) for j <= r (0 above the diagonal)
-__device__ void masked_scores(const float *sPq, const float *sPk, int nr, int D, float *sA) {
-    for (int e = threadIdx.x; e < nr * kCs; e += blockDim.x) {
-        const int r = e / kCs, j = e - r * kCs;
-        float acc = 0.0f;
-        if (j <= r && j < nr)
-            for (int f = 0; f < D; ++f) acc = fmaf(sPq[r * D + f], sPk[j * D + f], acc);
-        sA[e] = acc;
-    }
-}
-
-// state update S += phi(K)^T V, z += sum phi(K) over the chunk rows (fp64, one rounding per chunk: the
-// running state is shared by every later row, so its rounding does not average out in the gradients)
-__device__ void advance_state(float *S, float *z, const float *sPk, const float *sV, int nr, int D, int dv) {
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) {
-        const int f = e / dv, c = e - f * dv;
-        double acc = S[e];
-        for (int r = 0; r < nr; ++r) acc = fma((double)sPk[r * D + f], (double)sV[r * dv + c], acc);
-        S[e] = (float)acc;
-    }
-    for (int f = threadIdx.x; f < D; f += blockDim.x) {
-        double acc = z[f];
-        for (int r = 0; r < nr; ++r) acc += (double)sPk[r * D + f];
-        z[f] = (float)acc;
-    }
-}
-
-// den_r = eps + phi(q_r).z + sum_{j<=r} A[r][j];  O_r = (phi(q_r) S + sum_{j<=r} A[r][j] v_j) / den_r,
-// both formed in fp64 and rounded once (the backward's gradients cancel to a small part of their terms
-// under the scale invariance of each row, so a row's rounding must stay at half an ulp)
-__device__ void chunk_outputs(const AttnArgs &a, const float *S, const float *z, const float *sPq, const float *sA,
-                              const float *sV, int nr, float *sden, float *sO) {
-    const int D = a.D, dv = a.dv;
-    for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-        double den = a.eps;
-        for (int f = 0; f < D; ++f) den = fma((double)sPq[r * D + f], (double)z[f], den);
-        for (int j = 0; j <= r; ++j) den += (double)sA[r * kCs + j];
-        sden[r] = (float)den;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-        const int r = e / dv, c = e - r * dv;
-        float o = 0.0f;
-        if (sden[r] != 0.0f) {
-            double num = 0.0;
-            for (int f = 0; f < D; ++f) num = fma((double)sPq[r * D + f], (double)S[f * dv + c], num);
-            for (int j = 0; j <= r; ++j) num = fma((double)sA[r * kCs + j], (double)sV[j * dv + c], num);
-            o = (float)(num / (double)sden[r]);
-        }
-        sO[e] = o;
-    }
+// den_r = eps + phi(q_r) . z + sum_{j<=r} A[r][j], rounded once
+__device__ __forceinline__ void tile_dens(const Rows &Pq, int nr, int D, const float *z, const Rows &A, float eps,
+                                          float *sden, float *sinv) {
+    row_dots(Pq, nr, D, [&](int, int f) { return z[f]; }, A, [](int r) { return r + 1; },
+             [&](int r, float h, float l) {
+                 pair_mac_any(h, l, eps, 1.0f);
+                 const float den = pair_value(h, l);
+                 sden[r] = den;
+                 sinv[r] = 1.0f / den;
+             });
 }
 
 // ---------------------------------------------------------------------------
 
 template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_causal_out(AttnArgs a) {
+__global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    const int D = a.D, dv = a.dv, d = a.d;
-    SmemPhi s = carve_phi(cv, lay);
-    float *S = cv.take(D * dv), *z = cv.take(D);
-    float *sQ = cv.take(kCs * d), *sK = cv.take(kCs * d), *sV = cv.take(kCs * dv);
-    float *sPq = cv.take(kCs * D), *sPk = cv.take(kCs * D), *sA = cv.take(kCs * kCs);
-    float *sden = cv.take(kCs), *sO = cv.take(kCs * dv);
+    const int D = a.D, dv = a.dv, d = a.d, Dp = (D + 3) & ~3;
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    float *tiles = cv.p;
+    const Rows S = take_rows(cv, Dp, dv);
+    float *z = cv.take(Dp);
+    const Rows sQ = take_rows(cv, cap, d), sK = take_rows(cv, cap, d), sV = take_rows(cv, cap, dv);
+    const Rows sPq = take_rows(cv, cap, D), sPk = take_rows(cv, cap, D), sA = take_rows(cv, cap, cap);
+    float *sden = cv.take(cap), *sinv = cv.take(cap);
+    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(4));  // largest |phi(k)|, |V|
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = seg * a.seg_len, rend = min(a.n, r0 + a.seg_len), r1 = min(len, rend);
     IO *O = static_cast<IO *>(a.O) + head_rows(a, bh) * dv;
-    for (int e = threadIdx.x + max(r0, len) * dv; e < rend * dv; e += blockDim.x) io_store(O + e, 0.0f);
+    zero_rows(O, max(r0, len), rend, dv);
     if (r0 >= r1) return;
-    load_phi(s, lay, a.table);
+    zero_words(tiles, (int)(cv.p - tiles));
+    load_phi_tile(s, lay, a.table);
     const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) S[e] = a.seg_S[so * D * dv + e];
-    for (int e = threadIdx.x; e < D; e += blockDim.x) z[e] = a.seg_z[so * D + e];
-    for (int t0 = r0; t0 < r1; t0 += kCs) {
-        const int nr = min(kCs, r1 - t0);
+    __syncthreads();
+    load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv);
+    const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
+    const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
+    const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
+    const bool vec = vec_store(O, dv);
+    for (int t0 = r0; t0 < r1; t0 += cap) {
+        const int nr = min(cap, r1 - t0);
         __syncthreads();
-        load_chunk<IO>(a, bh, t0, nr, sQ, sK, sV, nullptr);
+        if (threadIdx.x < 2) mx[threadIdx.x] = 0u;
+        load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
+        load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_tile(lay, s, sQ, nr, sPq, nullptr, nullptr);
-        phi_tile(lay, s, sK, nr, sPk, nullptr, nullptr);
+        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, nullptr);
+        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx);
+        tile_max(sV.p, cap * sV.ld, mx + 1);
         __syncthreads();
-        masked_scores(sPq, sPk, nr, D, sA);
+        scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int) { return 0.0f; }, [](int, float &, float &) {});
         __syncthreads();
-        chunk_outputs(a, S, z, sPq, sA, sV, nr, sden, sO);
+        tile_dens(sPq, nr, D, z, sA, a.eps, sden, sinv);
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) io_store(O + (size_t)t0 * dv + e, sO[e]);
-        advance_state(S, z, sPk, sV, nr, D, dv);
+        // O_r = (phi(q_r) S + sum_{j<=r} A[r][j] v_j) / den_r from the pair of the numerator
+        prod_nn(sPq, nr, S, Dp, dv, sA, sV, [](int) { return 0.0f; },
+                [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        if (q0 + i >= nr) continue;
+                        const float den = sden[q0 + i], inv = sinv[q0 + i];
+                        float o[4];
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) o[m] = den != 0.0f ? pair_div(h[i][m], l[i][m], den, inv) : 0.0f;
+                        store4(O + (size_t)(t0 + q0 + i) * dv + c0, o, dv - c0, vec);
+                    }
+                });
+        if (t0 + cap >= r1) break;
+        __syncthreads();
+        const float zbound = (float)nr * __uint_as_float(mx[0]);
+        advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base(zbound * __uint_as_float(mx[1])), pair_base(zbound));
     }
 }
 
-// forward sweep of the backward pass: records (den_i, dden_i), sums G over the segment
-template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_causal_bwd_seg(AttnArgs a) {
+// Query side of the backward pass, one forward sweep per segment: den_i and dden_i of every row as pairs (kept for the
+// key side), dQ, and the segment's sums of G and g.
+//   dphi(q_i) = S_{before tile} dnum_i + z dden_i + sum_{j<=i in tile} dP_ij phi(k_j),  dP_ij = dnum_i . v_j + dden_i
+// den_i, dnum_i . num_i and dden_i are pairs (RowPairs); dP and dphi are pairs rounded once.
+template <typename IO, int TF, int TC>
+__global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int cap, int nbuf, int finish) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    const int D = a.D, dv = a.dv, d = a.d;
-    SmemPhi s = carve_phi(cv, lay);
-    float *S = cv.take(D * dv), *z = cv.take(D);
-    float *sQ = cv.take(kCs * d), *sK = cv.take(kCs * d), *sV = cv.take(kCs * dv), *sdO = cv.take(kCs * dv);
-    float *sPq = cv.take(kCs * D), *sPk = cv.take(kCs * D), *sA = cv.take(kCs * kCs);
-    float *sden = cv.take(kCs), *sdden = cv.take(kCs), *sO = cv.take(kCs * dv);
+    const int D = a.D, dv = a.dv, d = a.d, M = a.M, Dp = (D + 3) & ~3, dvp = (dv + 3) & ~3;
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    float *tiles = cv.p;
+    const Rows S = take_rows(cv, Dp, dv);
+    float *z = cv.take(Dp);
+    const Rows sQ = take_rows(cv, cap, d), sV = take_rows(cv, cap, dv), sdO = take_rows(cv, cap, dv);
+    const Rows sPq = take_rows(cv, cap, D), sPk = take_rows(cv, cap, D), sA = take_rows(cv, cap, cap);
+    // one buffer holds k_j, then the parts of dnum_i . num_i, then dphi(q_i)
+    float *shared = cv.take(cap * max(row_stride(d), max(row_stride(dv), row_stride(D))));
+    const Rows sK{shared, row_stride(d)}, sR{shared, row_stride(dv)}, sdPhi{shared, row_stride(D)};
+    const RowPairs rp = take_row_pairs(cv, cap);
+    float *sU = cv.take(cap * M);
+    int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
+    float *sdU = cv.take(cap * du_stride(M));
+    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(8));  // |S|, |V|, |dO|, |phi(q)|, |phi(k)|, |z|, |dnum|, |dden|
+    cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
+    __shared__ double sT[kMaxL];  // channel normalisation: the block's sums of phi . dphi per channel
+    if ((int)threadIdx.x < kMaxL) sT[threadIdx.x] = 0.0;
+    const size_t slot = (size_t)bh * a.nseg + seg;
+    double *gp = reinterpret_cast<double *>(a.gpart) + (slot % nbuf) * a.gsize;
+    double *hist = gp + M * d + M;
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = seg * a.seg_len, rend = min(a.n, r0 + a.seg_len), r1 = min(len, rend);
-    load_phi(s, lay, a.table);
-    const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) S[e] = a.seg_S[so * D * dv + e];
-    for (int e = threadIdx.x; e < D; e += blockDim.x) z[e] = a.seg_z[so * D + e];
-    const int nc = (dv + 7) / 8, nf = (D + 7) / 8;
-    const bool active = threadIdx.x < nf * nc;
-    const int tf = active ? threadIdx.x / nc : 0, tc = active ? threadIdx.x % nc : 0;
-    const int f0 = tf * 8, c0 = tc * 8;
-    double acc[8][8] = {}, zacc[8] = {};
-    for (int t0 = r0; t0 < r1; t0 += kCs) {
-        const int nr = min(kCs, r1 - t0);
+    IO *dQ = static_cast<IO *>(a.dQ) + head_rows(a, bh) * d;
+    zero_rows(dQ, max(r0, len), rend, d);
+    OuterAcc<TF, TC> acc;
+    acc.zero();
+    GradTile g;
+    grad_zero(g);
+    if (r0 < r1) {
+        zero_words(tiles, (int)(cv.p - tiles));
+        load_phi_tile(s, lay, a.table);
+        const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
         __syncthreads();
-        load_chunk<IO>(a, bh, t0, nr, sQ, sK, sV, sdO);
+        load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv);
+    }
+    const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
+    const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
+    const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
+    const IO *dO = static_cast<const IO *>(a.dO) + head_rows(a, bh) * dv;
+    const Rows none{};
+    for (int t0 = r0; t0 < r1; t0 += cap) {
+        const int nr = min(cap, r1 - t0);
         __syncthreads();
-        phi_tile(lay, s, sQ, nr, sPq, nullptr, nullptr);
-        phi_tile(lay, s, sK, nr, sPk, nullptr, nullptr);
+        if (threadIdx.x < 8) mx[threadIdx.x] = 0u;
+        load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
+        load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
+        load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        masked_scores(sPq, sPk, nr, D, sA);
+        phi_rows(lay, s, sQ, nr, cap, sPq, sU, sJ, mx + 3);
+        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx + 4);
+        tile_max(S.p, Dp * S.ld, mx);
+        tile_max(z, Dp, mx + 5);
+        tile_max(sV.p, cap * sV.ld, mx + 1);
+        tile_max(sdO.p, cap * sdO.ld, mx + 2);
         __syncthreads();
-        chunk_outputs(a, S, z, sPq, sA, sV, nr, sden, sO);
+        const float mS = __uint_as_float(mx[0]), mV = __uint_as_float(mx[1]), mdO = __uint_as_float(mx[2]);
+        const float mq = __uint_as_float(mx[3]), mk = __uint_as_float(mx[4]), mz = __uint_as_float(mx[5]);
+        // pairs too: o and den are formed from A, and a common rounding error of theirs does not cancel in dphi
+        const float bA = pair_base((float)D * mq * mk);
+        scores_lower<true>(sPq, sPk, nr, Dp, sA, [&](int) { return bA; }, [](int, float &, float &) {});
         __syncthreads();
-        for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-            double dot = 0.0;  // dden and dphi are formed in fp64 and rounded once: they cancel
-            for (int c = 0; c < dv; ++c) dot = fma((double)sdO[r * dv + c], (double)sO[r * dv + c], dot);
-            const float dd = (sden[r] != 0.0f) ? (float)(-dot / (double)sden[r]) : 0.0f;
-            sdden[r] = dd;
-            float *rs = a.rowstat + ((size_t)bh * a.n + t0 + r) * 2;
-            rs[0] = sden[r];
-            rs[1] = dd;
+        row_dots(sPq, nr, D, [&](int, int f) { return z[f]; }, sA, [](int r) { return r + 1; },
+                 [&](int r, float h, float l) { rp.set_den(r, h, l, a.eps); });
+        __syncthreads();
+        {
+            float m = 0.0f;
+            for (int e = threadIdx.x; e < nr * dvp; e += blockDim.x) {  // dnum in place
+                const int r = e / dvp, c = e - r * dvp;
+                const float v = rp.over_den(r, sdO[r][c]);
+                sdO[r][c] = v;
+                m = fmaxf(m, fabsf(v));
+            }
+            block_max(m, mx + 6);
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-            const int r = e / dv;
-            sO[e] = (sden[r] != 0.0f) ? sdO[e] / sden[r] : 0.0f;  // dnum
-        }
+        const float bnum = pair_base((float)D * mq * fmaf((float)nr * mk, mV, mS));
+        prod_nn(sPq, nr, S, Dp, dv, sA, sV, [&](int) { return bnum; },
+                [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
+                    unit_dots(sdO, sR, nr, q0, c0, h, l, bnum);
+                });
         __syncthreads();
-        if (active) outer_accumulate(acc, zacc, true, sPq, D, sO, dv, sdden, nr, f0, c0);
-        advance_state(S, z, sPk, sV, nr, D, dv);
+        sum_unit_dots(sR, nr, dvp / 4, [&](int r, float h, float l) {
+            rp.set_dden(r, h, l);
+            atomicMax(mx + 7, __float_as_uint(fabsf(rp.gh[r])));
+            *reinterpret_cast<float4 *>(a.rowstat + ((size_t)bh * a.n + t0 + r) * 4) =
+                make_float4(rp.dh[r], rp.dl[r], rp.gh[r], rp.gl[r]);
+        });
+        __syncthreads();
+        // starts of row r's sums: |dP[r][.]| and the terms of dphi(q_r) stay below these bounds
+        auto bound_p = [&](int r) {
+            return r < nr && rp.dh[r] != 0.0f ? fmaf(2.0f * (float)dv * mV * mdO, fabsf(rp.inv[r]), fabsf(rp.gh[r])) : 0.0f;
+        };
+        auto base_p = [&](int r) { return pair_base(bound_p(r)); };
+        auto base_q = [&](int r) {
+            return r < nr && rp.dh[r] != 0.0f
+                       ? pair_base(fmaf(2.0f * (float)dv * mS * mdO, fabsf(rp.inv[r]), mz * fabsf(rp.gh[r])) +
+                                   (float)nr * mk * bound_p(r))
+                       : 0.0f;
+        };
+        scores_lower<true>(sdO, sV, nr, dvp, sA, base_p, [&](int r, float &h, float &l) {
+            pair_mac(h, l, rp.gh[r], 1.0f);
+            l = __fadd_rn(l, rp.gl[r]);
+        });
+        acc.add(sPq, D, sdO, dv, rp.gh, rp.gl, nr, pair_base((float)nr * mq * __uint_as_float(mx[6])),
+                pair_base((float)nr * mq * __uint_as_float(mx[7])));
+        __syncthreads();
+        prod_nt<kLower>(sdO, nr, S, D, dvp, sA, sPk, nr,
+                        [&](int r, int f, float &h, float &l) {
+                            h = base_q(r);
+                            l = 0.0f;
+                            if (r < nr) {
+                                l = z[f] * rp.gl[r];
+                                pair_mac(h, l, z[f], rp.gh[r]);
+                            }
+                        },
+                        [&](int r, int f, float h, float l) {
+                            if (r >= nr) return;
+                            h -= base_q(r);
+                            sdPhi[r][f] = pair_value(h, l);
+                            if (a.ch_T) atomicAdd(sT + f % a.L, (double)sPq[r][f] * ((double)h + (double)l));
+                        });
+        __syncthreads();
+        if (t0 + cap < r1)
+            advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base((float)nr * mk * mV), pair_base((float)nr * mk));
+        phi_backward_rows(lay, s, sQ, nr, cap, sPq, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
+        store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
     __syncthreads();
-    const size_t slot = (size_t)bh * a.nseg + seg;
-    store_tile(acc, zacc, active, tc, f0, c0, D, dv, a.dS_part + slot * D * dv, a.dz_part + slot * D);
-    if (last_arrival(a.counters + a.B * a.H + bh, a.nseg)) {
+    acc.store(D, dv, a.dS_part, a.dz_part, slot, false);
+    if (r0 < r1) add_grad_tile(lay, g, gp);
+    if (a.ch_T && (int)threadIdx.x < a.L) a.ch_T[slot * a.L + threadIdx.x] = sT[threadIdx.x];
+    if (finish && last_arrival(a.counters + a.B * a.H + bh, a.nseg)) {
         exclusive_scan(a.dS_part + (size_t)bh * a.nseg * D * dv, a.nseg, D * dv, a.seg_dS + (size_t)bh * a.nseg * D * dv,
                        true);
         exclusive_scan(a.dz_part + (size_t)bh * a.nseg * D, a.nseg, D, a.seg_dz + (size_t)bh * a.nseg * D, true);
@@ -202,200 +267,151 @@ __global__ void __launch_bounds__(kThreads) k_causal_bwd_seg(AttnArgs a) {
     }
 }
 
-// dQ: forward sweep.  dphi(q_i) = S_{before chunk} dnum_i + z dden_i + sum_{j<=i in chunk} dP_ij phi(k_j),
-// dP_ij = dnum_i . v_j + dden_i
+// dK, dV: reverse sweep with the suffix state G (after the current tile).
+//   dv_j = G^T phi(k_j) + sum_{i>=j in tile} A_ij dnum_i
+//   dphi(k_j) = G v_j + g + sum_{i>=j in tile} dP_ij phi(q_i)
 template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_causal_dq(AttnArgs a) {
+__global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap, int nbuf) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    const int D = a.D, dv = a.dv, d = a.d, M = a.M;
-    SmemPhi s = carve_phi(cv, lay);
-    float *S = cv.take(D * dv), *z = cv.take(D);
-    float *sQ = cv.take(kCs * d), *sK = cv.take(kCs * d), *sV = cv.take(kCs * dv), *sdO = cv.take(kCs * dv);
-    float *sPq = cv.take(kCs * D), *sPk = cv.take(kCs * D), *sdPq = cv.take(kCs * D), *sP = cv.take(kCs * kCs);
-    float *sden = cv.take(kCs), *sdden = cv.take(kCs);
-    float *sU = cv.take(kCs * M);
-    int *sJ = reinterpret_cast<int *>(cv.take(kCs * M));
-    float *sdU = cv.take(kCs * M);
+    const int D = a.D, dv = a.dv, d = a.d, M = a.M, Dp = (D + 3) & ~3, dvp = (dv + 3) & ~3;
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    float *tiles = cv.p;
+    const Rows G = take_rows(cv, Dp, dv);
+    float *gz = cv.take(Dp);
+    const Rows sK = take_rows(cv, cap, d), sV = take_rows(cv, cap, dv), sdO = take_rows(cv, cap, dv);
+    const Rows sPq = take_rows(cv, cap, D), sPk = take_rows(cv, cap, D);
+    const Rows sA = take_rows(cv, cap, cap), sP = take_rows(cv, cap, cap);
+    // one buffer holds q_i, then dphi(k_j)
+    float *shared = cv.take(cap * max(row_stride(d), row_stride(D)));
+    const Rows sQ{shared, row_stride(d)}, sdPhi{shared, row_stride(D)};
+    const RowPairs rp = take_row_pairs(cv, cap);
+    float *sU = cv.take(cap * M);
+    int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
+    float *sdU = cv.take(cap * du_stride(M));
+    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(8));  // largest |V|, |dden|, |dnum|, |phi(q)|, |G|, |g|
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
-    __shared__ double sT[kMaxL];  // channel normalisation: the block's sums of phi . dphi per channel
-    if ((int)threadIdx.x < kMaxL) sT[threadIdx.x] = 0.0;
-    double *gp = reinterpret_cast<double *>(a.gpart) + ((size_t)bh * a.nseg + seg) * a.gsize;
-    double *shist = gp + M * d + M;  // the block's fp64 histogram, accumulated in place by L2 atomics
-    const int len = head_length(a.lengths, bh / a.H, a.n);
-    const int r0 = seg * a.seg_len, rend = min(a.n, r0 + a.seg_len), r1 = min(len, rend);
-    IO *dQ = static_cast<IO *>(a.dQ) + head_rows(a, bh) * d;
-    for (int e = threadIdx.x + max(r0, len) * d; e < rend * d; e += blockDim.x) io_store(dQ + e, 0.0f);
-    load_phi(s, lay, a.table);
-    const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) S[e] = a.seg_S[so * D * dv + e];
-    for (int e = threadIdx.x; e < D; e += blockDim.x) z[e] = a.seg_z[so * D + e];
-    for (int e = threadIdx.x; e < mlp_words(lay) + var_words(lay); e += blockDim.x) shist[e] = 0.0;
-    GradAcc g = {};
-    for (int t0 = r0; t0 < r1; t0 += kCs) {
-        const int nr = min(kCs, r1 - t0);
-        __syncthreads();
-        load_chunk<IO>(a, bh, t0, nr, sQ, sK, sV, sdO);
-        for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-            const float *rs = a.rowstat + ((size_t)bh * a.n + t0 + r) * 2;
-            sden[r] = rs[0];
-            sdden[r] = rs[1];
-        }
-        __syncthreads();
-        phi_tile(lay, s, sQ, nr, sPq, sU, sJ);
-        phi_tile(lay, s, sK, nr, sPk, nullptr, nullptr);
-        for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-            const int r = e / dv;
-            sdO[e] = (sden[r] != 0.0f) ? sdO[e] / sden[r] : 0.0f;  // dnum in place
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < nr * kCs; e += blockDim.x) {
-            const int r = e / kCs, j = e - r * kCs;
-            double acc = 0.0;
-            if (j <= r && j < nr) {
-                for (int c = 0; c < dv; ++c) acc = fma((double)sdO[r * dv + c], (double)sV[j * dv + c], acc);
-                acc += (double)sdden[r];
-            }
-            sP[e] = (float)acc;
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < nr * D; e += blockDim.x) {
-            const int r = e / D, f = e - r * D;
-            double acc = (double)z[f] * (double)sdden[r];
-            for (int c = 0; c < dv; ++c) acc = fma((double)S[f * dv + c], (double)sdO[r * dv + c], acc);
-            for (int j = 0; j <= r; ++j) acc = fma((double)sP[r * kCs + j], (double)sPk[j * D + f], acc);
-            sdPq[e] = (float)acc;
-            if (a.ch_T) atomicAdd(sT + f % a.L, (double)sPq[e] * acc);
-        }
-        __syncthreads();
-        advance_state(S, z, sPk, sV, nr, D, dv);
-        phi_backward_tile(lay, s, sQ, nr, sPq, sdPq, sU, sJ, sdU, shist, shist + mlp_words(lay), g);
-        store_dx(lay, s, sdU, nr, dQ + (size_t)t0 * d);
-    }
-    __syncthreads();
-    store_grad_partial(lay, g, gp);
-    if (a.ch_T && (int)threadIdx.x < a.L) a.ch_T[((size_t)bh * a.nseg + seg) * a.L + threadIdx.x] = sT[threadIdx.x];
-}
-
-// dK, dV: reverse sweep with the suffix state G (after the current chunk).
-//   dv_j = G^T phi(k_j) + sum_{i>=j in chunk} A_ij dnum_i
-//   dphi(k_j) = G v_j + g + sum_{i>=j in chunk} dP_ij phi(q_i)
-template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_causal_dkv(AttnArgs a) {
-    extern __shared__ __align__(16) float smem[];
-    Carve cv{smem};
-    const TableLayout &lay = a.lay;
-    const int D = a.D, dv = a.dv, d = a.d, M = a.M;
-    SmemPhi s = carve_phi(cv, lay);
-    float *G = cv.take(D * dv), *gz = cv.take(D);
-    float *sQ = cv.take(kCs * d), *sK = cv.take(kCs * d), *sV = cv.take(kCs * dv), *sdO = cv.take(kCs * dv);
-    float *sPq = cv.take(kCs * D), *sPk = cv.take(kCs * D), *sdPk = cv.take(kCs * D);
-    float *sA = cv.take(kCs * kCs), *sP = cv.take(kCs * kCs);
-    float *sden = cv.take(kCs), *sdden = cv.take(kCs);
-    float *sU = cv.take(kCs * M);
-    int *sJ = reinterpret_cast<int *>(cv.take(kCs * M));
-    float *sdU = cv.take(kCs * M);
-    if (!carve_fits(cv, smem)) return;
-    const int bh = blockIdx.y, seg = blockIdx.x;
-    double *gp = reinterpret_cast<double *>(a.gpart) + ((size_t)a.B * a.H * a.nseg + (size_t)bh * a.nseg + seg) * a.gsize;
-    double *shist = gp + M * d + M;  // the block's fp64 histogram, accumulated in place by L2 atomics
+    double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nseg + seg) % nbuf) * a.gsize;
+    double *hist = gp + M * d + M;
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = seg * a.seg_len, rend = min(a.n, r0 + a.seg_len), r1 = min(len, rend);
     IO *dK = static_cast<IO *>(a.dK) + head_rows(a, bh) * d;
     IO *dV = static_cast<IO *>(a.dV) + head_rows(a, bh) * dv;
-    for (int e = threadIdx.x + max(r0, len) * d; e < rend * d; e += blockDim.x) io_store(dK + e, 0.0f);
-    for (int e = threadIdx.x + max(r0, len) * dv; e < rend * dv; e += blockDim.x) io_store(dV + e, 0.0f);
-    load_phi(s, lay, a.table);
+    zero_rows(dK, max(r0, len), rend, d);
+    zero_rows(dV, max(r0, len), rend, dv);
+    if (r1 <= r0) return;
+    zero_words(tiles, (int)(cv.p - tiles));
+    load_phi_tile(s, lay, a.table);
     const size_t so = (size_t)bh * a.nseg + seg;
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) G[e] = a.seg_dS[so * D * dv + e];
-    for (int e = threadIdx.x; e < D; e += blockDim.x) gz[e] = a.seg_dz[so * D + e];
-    for (int e = threadIdx.x; e < mlp_words(lay) + var_words(lay); e += blockDim.x) shist[e] = 0.0;
-    GradAcc g = {};
-    if (r1 > r0) {
-        for (int t0 = r0 + ((r1 - 1 - r0) / kCs) * kCs; t0 >= r0; t0 -= kCs) {
-            const int nr = min(kCs, r1 - t0);
-            __syncthreads();
-            load_chunk<IO>(a, bh, t0, nr, sQ, sK, sV, sdO);
-            for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-                const float *rs = a.rowstat + ((size_t)bh * a.n + t0 + r) * 2;
-                sden[r] = rs[0];
-                sdden[r] = rs[1];
-            }
-            __syncthreads();
-            phi_tile(lay, s, sQ, nr, sPq, nullptr, nullptr);
-            phi_tile(lay, s, sK, nr, sPk, sU, sJ);
-            for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-                const int r = e / dv;
-                sdO[e] = (sden[r] != 0.0f) ? sdO[e] / sden[r] : 0.0f;  // dnum in place
-            }
-            __syncthreads();
-            masked_scores(sPq, sPk, nr, D, sA);
-            for (int e = threadIdx.x; e < nr * kCs; e += blockDim.x) {
-                const int r = e / kCs, j = e - r * kCs;
-                double acc = 0.0;
-                if (j <= r && j < nr) {
-                    for (int c = 0; c < dv; ++c) acc = fma((double)sdO[r * dv + c], (double)sV[j * dv + c], acc);
-                    acc += (double)sdden[r];
-                }
-                sP[e] = (float)acc;
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-                const int j = e / dv, c = e - j * dv;
-                float acc = 0.0f;
-                for (int f = 0; f < D; ++f) acc = fmaf(G[f * dv + c], sPk[j * D + f], acc);
-                for (int r = j; r < nr; ++r) acc = fmaf(sA[r * kCs + j], sdO[r * dv + c], acc);
-                io_store(dV + (size_t)t0 * dv + e, acc);
-            }
-            for (int e = threadIdx.x; e < nr * D; e += blockDim.x) {
-                const int j = e / D, f = e - j * D;
-                double acc = gz[f];
-                for (int c = 0; c < dv; ++c) acc = fma((double)G[f * dv + c], (double)sV[j * dv + c], acc);
-                for (int r = j; r < nr; ++r) acc = fma((double)sP[r * kCs + j], (double)sPq[r * D + f], acc);
-                sdPk[e] = (float)acc;
-            }
-            __syncthreads();
-            // G += phi(Q_chunk)^T dnum, g += phi(Q_chunk)^T dden
-            for (int e = threadIdx.x; e < D * dv; e += blockDim.x) {
-                const int f = e / dv, c = e - f * dv;
-                double acc = G[e];
-                for (int r = 0; r < nr; ++r) acc = fma((double)sPq[r * D + f], (double)sdO[r * dv + c], acc);
-                G[e] = (float)acc;
-            }
-            for (int f = threadIdx.x; f < D; f += blockDim.x) {
-                double acc = gz[f];
-                for (int r = 0; r < nr; ++r) acc = fma((double)sPq[r * D + f], (double)sdden[r], acc);
-                gz[f] = (float)acc;
-            }
-            phi_backward_tile(lay, s, sK, nr, sPk, sdPk, sU, sJ, sdU, shist, shist + mlp_words(lay), g);
-            store_dx(lay, s, sdU, nr, dK + (size_t)t0 * d);
-        }
-    }
     __syncthreads();
-    store_grad_partial(lay, g, gp);
+    load_state(G, gz, a.seg_dS + so * D * dv, a.seg_dz + so * D, D, dv);
+    const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
+    const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
+    const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
+    const IO *dO = static_cast<const IO *>(a.dO) + head_rows(a, bh) * dv;
+    const bool vec = vec_store(dV, dv);
+    GradTile g;
+    grad_zero(g);
+    for (int t0 = r0 + ((r1 - 1 - r0) / cap) * cap; t0 >= r0; t0 -= cap) {
+        const int nr = min(cap, r1 - t0);
+        __syncthreads();
+        if (threadIdx.x < 8) mx[threadIdx.x] = 0u;
+        load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
+        load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
+        load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
+        for (int r = threadIdx.x; r < cap; r += blockDim.x) {
+            const float4 v = r < nr ? ld4(a.rowstat + ((size_t)bh * a.n + t0 + r) * 4) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            rp.dh[r] = v.x; rp.dl[r] = v.y; rp.inv[r] = 1.0f / v.x;
+            rp.gh[r] = v.z; rp.gl[r] = v.w;
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < nr * dvp; e += blockDim.x) {  // dnum in place
+            const int r = e / dvp, c = e - r * dvp;
+            sdO[r][c] = rp.over_den(r, sdO[r][c]);
+        }
+        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, mx + 3);
+        phi_rows(lay, s, sK, nr, cap, sPk, sU, sJ, nullptr);
+        tile_max(G.p, Dp * G.ld, mx + 4);
+        tile_max(gz, Dp, mx + 5);
+        tile_max(sV.p, cap * sV.ld, mx);
+        tile_max(rp.gh, cap, mx + 1);
+        __syncthreads();
+        tile_max(sdO.p, cap * sdO.ld, mx + 2);
+        scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int) { return 0.0f; }, [](int, float &, float &) {});
+        __syncthreads();
+        const float mV = __uint_as_float(mx[0]), mdd = __uint_as_float(mx[1]), mdn = __uint_as_float(mx[2]);
+        const float mq = __uint_as_float(mx[3]), mG = __uint_as_float(mx[4]), mg = __uint_as_float(mx[5]);
+        const float bound_p = fmaf((float)dv * mdn, mV, mdd), bp = pair_base(bound_p);
+        const float bk = pair_base(fmaf((float)dv * mG, mV, mg) + (float)nr * mq * bound_p);
+        scores_lower<true>(sdO, sV, nr, dvp, sP, [&](int) { return bp; }, [&](int r, float &h, float &l) {
+            pair_mac(h, l, rp.gh[r], 1.0f);
+            l = __fadd_rn(l, rp.gl[r]);
+        });
+        prod_nn_plain(sPk, nr, G, Dp, dv, sA, sdO, nr, [&](int q0, int c0, const float (&h)[2][4]) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);
+        });
+        __syncthreads();
+        prod_nt<kUpper>(sV, nr, G, D, dvp, sP, sPq, nr,
+                        [&](int, int f, float &h, float &l) {
+                            h = bk;
+                            l = 0.0f;
+                            pair_mac(h, l, gz[f], 1.0f);
+                        },
+                        [&](int r, int f, float h, float l) {
+                            if (r < nr) sdPhi[r][f] = pair_value(h - bk, l);
+                        });
+        __syncthreads();
+        if (t0 > r0)
+            advance_rows(G, gz, sPq, D, sdO, dv, rp.gh, rp.gl, nr, pair_base((float)nr * mq * mdn),
+                         pair_base((float)nr * mq * mdd));
+        phi_backward_rows(lay, s, sK, nr, cap, sPk, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
+        store_dx_rows(lay, s, sdU, nr, dK + (size_t)t0 * d);
+    }
+    add_grad_tile(lay, g, gp);
 }
 
 // ---------------------------------------------------------------------------
 
-size_t smem_out(const AttnArgs &a) {
-    HostCarve cv; carve_phi_host(cv, a.lay);
-    cv.take(a.D * a.dv); cv.take(a.D); cv.take(kCs * a.d); cv.take(kCs * a.d); cv.take(kCs * a.dv);
-    cv.take(kCs * a.D); cv.take(kCs * a.D); cv.take(kCs * kCs); cv.take(kCs); cv.take(kCs * a.dv);
+size_t smem_out(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
+    take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv);
+    take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, cap);
+    cv.take(cap); cv.take(cap); cv.take(4);
     return cv.bytes();
 }
-size_t smem_bwd_seg(const AttnArgs &a) {
-    return smem_out(a) + 4 * (size_t)(r4(kCs * a.dv) + r4(kCs));
-}
-size_t smem_dq(const AttnArgs &a) {
-    HostCarve cv; carve_phi_host(cv, a.lay);
-    cv.take(a.D * a.dv); cv.take(a.D); cv.take(kCs * a.d); cv.take(kCs * a.d); cv.take(kCs * a.dv);
-    cv.take(kCs * a.dv); cv.take(kCs * a.D); cv.take(kCs * a.D); cv.take(kCs * a.D); cv.take(kCs * kCs);
-    cv.take(kCs); cv.take(kCs); cv.take(kCs * a.M); cv.take(kCs * a.M); cv.take(kCs * a.M);
+size_t smem_bwd_query(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
+    take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.dv);
+    take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, cap);
+    cv.take(cap * std::max(row_stride(a.d), std::max(row_stride(a.dv), row_stride(a.D))));
+    take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
+    cv.take(8); cv.take(kSlack);
     return cv.bytes();
 }
-size_t smem_dkv(const AttnArgs &a) { return smem_dq(a) + 4 * (size_t)r4(kCs * kCs); }
+size_t smem_bwd_key(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
+    take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.dv);
+    take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D);
+    take_rows_host(cv, cap, cap); take_rows_host(cv, cap, cap);
+    cv.take(cap * std::max(row_stride(a.d), row_stride(a.D)));
+    take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
+    cv.take(8);
+    return cv.bytes();
+}
+
+// Rows per tile: a segment is walked tile by tile by one block, so the largest that fits.
+template <typename Smem>
+int seg_cap(const AttnArgs &a, Smem smem) {
+    return pick_cap((int64_t)kSMs * kMaxC, std::min(a.n, a.seg_len), smem);
+}
 
 template <typename IO>
 cudaError_t seg_stats(const AttnArgs &a, cudaStream_t s) {
@@ -409,32 +425,45 @@ template <typename IO>
 cudaError_t causal_fwd_impl(const AttnArgs &a, cudaStream_t s) {
     cudaError_t e = seg_stats<IO>(a, s);
     if (e != cudaSuccess) return e;
-    const size_t sm = smem_out(a);
+    const int cap = seg_cap(a, [&](int c) { return smem_out(a, c); });
+    const size_t sm = smem_out(a, cap);
     if ((e = set_smem(k_causal_out<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("causal_out", k_causal_out<IO>, dim3(a.nseg, a.B * a.H), kThreads, sm, s, a);
+    LUNA_LAUNCH("causal_out", k_causal_out<IO>, dim3(a.nseg, a.B * a.H), kThr, sm, s, a, cap);
     return cudaGetLastError();
 }
 
 template <typename IO>
 cudaError_t causal_bwd_impl(const AttnArgs &a0, bool have_state, cudaStream_t s) {
     AttnArgs a = a0;
-    a.gpart64 = 1;  // the generic kernels write fp64 parameter-gradient partials
+    a.gpart64 = 1;  // the generic kernels write fp64 parameter-gradient sums
     cudaError_t e;
     if (!have_state && (e = seg_stats<IO>(a, s)) != cudaSuccess) return e;
+    const int64_t blocks = (int64_t)a.B * a.H * a.nseg;
+    const int nbuf = grad_buffers(blocks, 2 * blocks);
+    if ((e = cudaMemsetAsync(a.gpart, 0, (size_t)nbuf * a.gsize * sizeof(double), s)) != cudaSuccess) return e;
     const dim3 grid(a.nseg, a.B * a.H);
-    size_t sm = smem_bwd_seg(a);
-    if ((e = set_smem(k_causal_bwd_seg<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("causal_bwd_seg", k_causal_bwd_seg<IO>, grid, kThreads, sm, s, a);
+    int cap = seg_cap(a, [&](int c) { return smem_bwd_query(a, c); });
+    size_t sm = smem_bwd_query(a, cap);
+    outer_dispatch(a.D, a.dv, [&](auto tf, auto tc) {
+        auto k = k_causal_bwd_query<IO, decltype(tf)::value, decltype(tc)::value>;
+        if ((e = set_smem(k, sm)) != cudaSuccess) return;
+        LUNA_LAUNCH("causal_bwd_query", k, grid, kThr, sm, s, a, cap, nbuf, a.nseg <= kFinishParts);
+        e = cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
+    if (a.nseg > kFinishParts) {
+        AttnArgs b = a;
+        b.hs_mul = 1;  // the suffixes are indexed by the sub-problem's own heads
+        if ((e = launch_part_reduce(kScanDown, b, a.nseg, a.dS_part, a.dz_part, a.seg_dS, a.seg_dz,
+                                    (size_t)a.nseg * a.D * a.dv, (size_t)a.nseg * a.D, s)) != cudaSuccess)
+            return e;
+    }
+    cap = seg_cap(a, [&](int c) { return smem_bwd_key(a, c); });
+    sm = smem_bwd_key(a, cap);
+    if ((e = set_smem(k_causal_bwd_key<IO>, sm)) != cudaSuccess) return e;
+    LUNA_LAUNCH("causal_bwd_key", k_causal_bwd_key<IO>, grid, kThr, sm, s, a, cap, nbuf);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    sm = smem_dq(a);
-    if ((e = set_smem(k_causal_dq<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("causal_dq", k_causal_dq<IO>, grid, kThreads, sm, s, a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    sm = smem_dkv(a);
-    if ((e = set_smem(k_causal_dkv<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("causal_dkv", k_causal_dkv<IO>, grid, kThreads, sm, s, a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int nparts = 2 * a.B * a.H * a.nseg;
+    int nparts = nbuf;
     if (a.ch_sigma) {  // the scale term of the channel normalisation (kappa from the queries' T rows)
         a.ch_T_rows = a.B * a.H * a.nseg;
         if ((e = launch_chrms_backward(a, nparts, &nparts, s)) != cudaSuccess) return e;
@@ -445,11 +474,7 @@ cudaError_t causal_bwd_impl(const AttnArgs &a0, bool have_state, cudaStream_t s)
 }  // namespace
 
 size_t causal_max_smem(const AttnArgs &a) {
-    size_t m = smem_out(a);
-    if (smem_bwd_seg(a) > m) m = smem_bwd_seg(a);
-    if (smem_dq(a) > m) m = smem_dq(a);
-    if (smem_dkv(a) > m) m = smem_dkv(a);
-    return m;
+    return std::max(smem_out(a, kMinC), std::max(smem_bwd_query(a, kMinC), smem_bwd_key(a, kMinC)));
 }
 
 cudaError_t launch_causal_fwd(const AttnArgs &a, luna_dtype io, bool, cudaStream_t s) {

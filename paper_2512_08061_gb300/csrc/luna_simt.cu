@@ -1,16 +1,23 @@
-// Generic CUDA-core kernels of the LUNA attention path (fp32 arithmetic).
+// Generic CUDA-core kernels of the LUNA attention path.
 //
 // They serve the fp32 I/O path (the parity bar there is 1e-4 relative, which
 // rules out bf16 tensor-core operands) and every shape the tensor-core path
-// does not specialise.  One thread block owns a (head, row range); all
-// statistics are fp32 and every cross-block reduction is performed in a fixed
-// order by the last block to arrive, so results are reproducible run to run
-// except for the order of shared-memory atomic adds in the gradient
-// histograms of the channel-MLP parameters.
+// does not specialise.  A block owns a range of rows of one head and walks it
+// in tiles of up to 64 rows (luna_tile.cuh); the statistics, normalisers and
+// feature gradients are pairs of floats rounded once.  Every cross-block sum of
+// S, z, dS, dz runs in a fixed order; the parameter gradients are fp64 sums by
+// L2 reductions, whose order varies in the last bits of the fp64 sum.
+//
+// Measured at 8 x 12 heads of 512 fp32 rows, d = D = 64 (us; before: fp64 sums in
+// tiles of 16 or 32 rows, 64 of 256 threads in the outer products):
+//   key statistics 1402 -> 121, queries 161 -> 54, backward queries 3848 -> 300,
+//   backward keys 1451 -> 151, gradient sum 30 -> 8.
+// The fma pipe is 30 to 35 % busy and the issue slots about half: what is left is
+// barriers between a tile's phases, the feature map's gathers and the histogram.
 #include <math.h>
 
 #include "luna_prof.cuh"
-#include "luna_simt_dev.cuh"
+#include "luna_tile.cuh"
 
 namespace luna {
 namespace {
@@ -23,23 +30,21 @@ template <typename IO>
 __global__ void __launch_bounds__(kThreads) k_featmap(TableLayout lay, const char *table, const IO *X, int64_t rows,
                                                       float *Phi) {
     extern __shared__ __align__(16) float smem[];
-    __shared__ __align__(16) float sS[kEytzinger];  // the interval search block (the tensor-core kernels' lookup)
     Carve cv{smem};
-    SmemPhi s = carve_phi(cv, lay);
+    SmemPhi s = carve_phi_tile(cv, lay, 0);
     if (!carve_fits(cv, smem)) return;
-    load_phi(s, lay, table);
-    for (int e = threadIdx.x; e < kEytzinger; e += blockDim.x) sS[e] = reinterpret_cast<const float *>(table + lay.off_Te)[e];
+    load_phi_tile(s, lay, table);
     __syncthreads();
-    const unsigned short *sB = reinterpret_cast<const unsigned short *>(sS + kSearchT);
-    const int M = lay.M, L = lay.L, d = lay.d, D = lay.D;
+    const unsigned short *sB = reinterpret_cast<const unsigned short *>(s.T + kSearchT);
+    const int M = lay.M, L = lay.L, d = lay.d, D = lay.D, ldw = row_stride(d);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < rows * M; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = e / M;
         const int i = (int)(e - r * M);
         const IO *x = X + r * d;
-        const float *w = s.W + i * d;
+        const float *w = s.W + i * ldw;
         float u = s.b[i];
         for (int c = 0; c < d; ++c) u = fmaf(w[c], io_load(x + c), u);
-        const int j = interval_bucketed(sS, sB, u);
+        const int j = interval_bucketed(s.T, sB, u);
         const float *ab = s.AB + j * ab_stride(lay);
         float *out = Phi + r * D + i * L;
         for (int l = 0; l < L; ++l) {
@@ -56,36 +61,39 @@ __global__ void __launch_bounds__(kThreads) k_featmap_var(TableLayout lay, const
                                                           int64_t rows, float *Phi) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
-    SmemPhi s = carve_phi(cv, lay);
-    float *sX = cv.take(kPhiRows * lay.d);
-    float *sPhi = cv.take(kPhiRows * lay.D);
+    SmemPhi s = carve_phi_tile(cv, lay, kPhiRows);
+    const Rows sX = take_rows(cv, kPhiRows, lay.d), sPhi = take_rows(cv, kPhiRows, lay.D);
     if (!carve_fits(cv, smem)) return;
-    load_phi(s, lay, table);
+    load_phi_tile(s, lay, table);
     for (int64_t t0 = (int64_t)blockIdx.x * kPhiRows; t0 < rows; t0 += (int64_t)gridDim.x * kPhiRows) {
         const int nr = (int)(rows - t0 < kPhiRows ? rows - t0 : kPhiRows);
         __syncthreads();
-        load_rows(sX, X + t0 * lay.d, nr * lay.d);
+        load_tile(sX, X + t0 * lay.d, nr, lay.d, kPhiRows);
         __syncthreads();
-        phi_tile(lay, s, sX, nr, sPhi, nullptr, nullptr);
+        phi_rows(lay, s, sX, nr, kPhiRows, sPhi, nullptr, nullptr, nullptr);
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * lay.D; e += blockDim.x) Phi[t0 * lay.D + e] = sPhi[e];
+        for (int e = threadIdx.x; e < nr * lay.D; e += blockDim.x) Phi[t0 * lay.D + e] = sPhi[e / lay.D][e % lay.D];
     }
 }
 
 // ---------------------------------------------------------------------------
+// The attention kernels.  Shared memory of each: the same arrays on the device (Carve) and on the host (HostCarve).
+
+// ---------------------------------------------------------------------------
 // key statistics S = sum_j phi(k_j) v_j^T, z = sum_j phi(k_j)   (Sec. 4: S_KV, S_K1)
 
-template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_keystats(AttnArgs a) {
+template <typename IO, int TF, int TC>
+__global__ void __launch_bounds__(kThr, 1) k_keystats(AttnArgs a, int cap, int pairs, int finish) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    SmemPhi s = carve_phi(cv, lay);
-    float *sK = cv.take(kTileK * a.d);
-    float *sV = cv.take(kTileK * a.dv);
-    float *sPhi = cv.take(kTileK * a.D);
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    const Rows sK = take_rows(cv, cap, a.d), sV = take_rows(cv, cap, a.dv), sPhi = take_rows(cv, cap, a.D);
+    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(4));  // largest |phi|, |V|
+    cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
-    load_phi(s, lay, a.table);
+    zero_words(sV.p, cap * sV.ld);
+    load_phi_tile(s, lay, a.table);
 
     const int bh = blockIdx.y, split = blockIdx.x;
     const int len = head_length(a.lengths, bh / a.H, a.n);
@@ -93,34 +101,34 @@ __global__ void __launch_bounds__(kThreads) k_keystats(AttnArgs a) {
     const int r1 = min(len, r0 + a.rows_per_split);
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * a.d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * a.dv;
-
-    const int nc = (a.dv + 7) / 8, nf = (a.D + 7) / 8;
-    const bool active = threadIdx.x < nf * nc;
-    const int tf = active ? threadIdx.x / nc : 0, tc = active ? threadIdx.x % nc : 0;
-    const int f0 = tf * 8, c0 = tc * 8;
-    double acc[8][8] = {}, zacc[8] = {};
-    for (int t0 = r0; t0 < r1; t0 += kTileK) {
-        const int nr = min(kTileK, r1 - t0);
+    OuterAcc<TF, TC> acc;
+    acc.zero();
+    for (int t0 = r0; t0 < r1; t0 += cap) {
+        const int nr = min(cap, r1 - t0);
         __syncthreads();
-        load_rows(sK, K + (size_t)t0 * a.d, nr * a.d);
-        load_rows(sV, V + (size_t)t0 * a.dv, nr * a.dv);
+        if (threadIdx.x < 2) mx[threadIdx.x] = 0u;
+        load_tile(sK, K + (size_t)t0 * a.d, nr, a.d, cap);
+        load_tile(sV, V + (size_t)t0 * a.dv, nr, a.dv, cap);
         __syncthreads();
-        phi_tile(lay, s, sK, nr, sPhi, nullptr, nullptr);
+        phi_rows(lay, s, sK, nr, cap, sPhi, nullptr, nullptr, mx);
+        tile_max(sV.p, cap * sV.ld, mx + 1);
         __syncthreads();
-        if (active) outer_accumulate(acc, zacc, true, sPhi, a.D, sV, a.dv, nullptr, nr, f0, c0);
+        const float zbound = (float)nr * __uint_as_float(mx[0]);
+        acc.add(sPhi, a.D, sV, a.dv, nullptr, nullptr, nr, pair_base(zbound * __uint_as_float(mx[1])), pair_base(zbound));
     }
     const size_t slot = (size_t)bh * a.nsplit + split;
-    store_tile(acc, zacc, active, tc, f0, c0, a.D, a.dv, a.S_part + slot * a.D * a.dv, a.z_part + slot * a.D);
-    if (last_arrival(a.counters + bh, a.nsplit)) {
+    acc.store(a.D, a.dv, a.S_part, a.z_part, slot, pairs != 0);
+    if (finish && last_arrival(a.counters + bh, a.nsplit)) {
         if (a.seg_S) {  // causal: exclusive prefix at every segment start, total in slot nsplit
             exclusive_scan(a.S_part + (size_t)bh * a.nsplit * a.D * a.dv, a.nsplit, a.D * a.dv,
                            a.seg_S + head_state(a, bh) * (a.nsplit + 1) * a.D * a.dv, false);
             exclusive_scan(a.z_part + (size_t)bh * a.nsplit * a.D, a.nsplit, a.D,
                            a.seg_z + head_state(a, bh) * (a.nsplit + 1) * a.D, false);
         } else {
-            ordered_sum(a.S_part + (size_t)bh * a.nsplit * a.D * a.dv, a.nsplit, a.D * a.dv,
+            const int np = pairs ? 2 * a.nsplit : a.nsplit;
+            ordered_sum(a.S_part + (size_t)bh * np * a.D * a.dv, np, a.D * a.dv,
                         a.S_fin + head_state(a, bh) * a.D * a.dv);
-            ordered_sum(a.z_part + (size_t)bh * a.nsplit * a.D, a.nsplit, a.D, a.z_fin + head_state(a, bh) * a.D);
+            ordered_sum(a.z_part + (size_t)bh * np * a.D, np, a.D, a.z_fin + head_state(a, bh) * a.D);
         }
         if (threadIdx.x == 0) a.counters[bh] = 0;
     }
@@ -130,83 +138,91 @@ __global__ void __launch_bounds__(kThreads) k_keystats(AttnArgs a) {
 // query side: O_i = phi(q_i)^T S / (phi(q_i)^T z + eps)   (Eq. kernel-attn)
 
 template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_query(AttnArgs a) {
+__global__ void __launch_bounds__(kThr, 1) k_query(AttnArgs a, int cap, int rows_per_block) {
     extern __shared__ __align__(16) float smem[];
     const int bh = blockIdx.y;
-    const int q0 = blockIdx.x * kTileQ;
+    const int b0 = blockIdx.x * rows_per_block, b1 = min(a.n, b0 + rows_per_block);
     const int len = head_length(a.lengths, bh / a.H, a.n);
     IO *O = static_cast<IO *>(a.O) + head_rows(a, bh) * a.dv;
-    const int nrows = min(kTileQ, a.n - q0);
-    if (q0 >= len) {  // padded rows only
-        for (int e = threadIdx.x; e < nrows * a.dv; e += blockDim.x) io_store(O + (size_t)q0 * a.dv + e, 0.0f);
-        return;
-    }
+    zero_rows(O, max(b0, len), b1, a.dv);  // padded rows
+    if (b0 >= len) return;
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    SmemPhi s = carve_phi(cv, lay);
-    float *sS = cv.take(a.D * a.dv);
-    float *sz = cv.take(a.D);
-    float *sQ = cv.take(kTileQ * a.d);
-    float *sPhi = cv.take(kTileQ * a.D);
-    float *sden = cv.take(kTileQ);
+    const int D = a.D, dv = a.dv, Dp = (D + 3) & ~3;
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    const Rows sS = take_rows(cv, Dp, dv);
+    float *sz = cv.take(D);
+    const Rows sQ = take_rows(cv, cap, a.d), sPhi = take_rows(cv, cap, D);
+    float *sden = cv.take(cap);
     if (!carve_fits(cv, smem)) return;
-    load_phi(s, lay, a.table);
-    for (int e = threadIdx.x; e < a.D * a.dv; e += blockDim.x) sS[e] = a.S_fin[head_state(a, bh) * a.D * a.dv + e];
-    for (int e = threadIdx.x; e < a.D; e += blockDim.x) sz[e] = a.z_fin[head_state(a, bh) * a.D + e];
-    const int nr = min(nrows, len - q0);
-    load_rows(sQ, static_cast<const IO *>(a.Q) + (head_rows(a, bh) + q0) * a.d, nr * a.d);
-    __syncthreads();
-    phi_tile(lay, s, sQ, nr, sPhi, nullptr, nullptr);
-    __syncthreads();
-    for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-        float den = a.eps;
-        for (int f = 0; f < a.D; ++f) den = fmaf(sPhi[r * a.D + f], sz[f], den);
-        sden[r] = den;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nrows * a.dv; e += blockDim.x) {
-        const int r = e / a.dv, c = e - r * a.dv;
-        float o = 0.0f;
-        if (r < nr && sden[r] != 0.0f) {
-            float num = 0.0f;
-            for (int f = 0; f < a.D; ++f) num = fmaf(sPhi[r * a.D + f], sS[f * a.dv + c], num);
-            o = num / sden[r];
-        }
-        io_store(O + (size_t)q0 * a.dv + e, o);
+    load_phi_tile(s, lay, a.table);
+    load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv);
+    const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * a.d;
+    const Rows none{};
+    const bool vec = vec_store(O, dv);
+    const int e1 = min(b1, len);
+    for (int t0 = b0; t0 < e1; t0 += cap) {
+        const int nr = min(cap, e1 - t0);
+        __syncthreads();
+        load_tile(sQ, Q + (size_t)t0 * a.d, nr, a.d, cap);
+        __syncthreads();
+        phi_rows(lay, s, sQ, nr, cap, sPhi, nullptr, nullptr, nullptr);
+        __syncthreads();
+        row_dots(sPhi, nr, D, [&](int, int f) { return sz[f]; }, none, [](int) { return 0; },
+                 [&](int r, float h, float l) {
+                     pair_mac_any(h, l, a.eps, 1.0f);
+                     sden[r] = pair_value(h, l);
+                 });
+        __syncthreads();
+        prod_nn_plain(sPhi, nr, sS, Dp, dv, none, none, 0, [&](int r0, int c0, const float (&h)[2][4]) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                if (r0 + i >= nr) continue;
+                const float den = sden[r0 + i];
+                float o[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) o[m] = den != 0.0f ? h[i][m] / den : 0.0f;
+                store4(O + (size_t)(t0 + r0 + i) * dv + c0, o, dv - c0, vec);
+            }
+        });
     }
 }
 
 // query side of the backward pass (non-causal):
 //   dnum_i = do_i / den_i,  dden_i = -(do_i . o_i) / den_i
 //   dphi(q_i) = S dnum_i + z dden_i,  dS += phi(q_i) dnum_i^T,  dz += phi(q_i) dden_i
-template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_bwd_query(AttnArgs a) {
+// den, the sum dnum_i . num_i and dden are pairs (RowPairs), dphi is a pair rounded once.
+template <typename IO, int TF, int TC>
+__global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int nbuf, int finish) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    const int D = a.D, dv = a.dv, d = a.d, M = a.M;
-    SmemPhi s = carve_phi(cv, lay);
-    float *sS = cv.take(D * dv);
-    float *sz = cv.take(D);
-    float *sQ = cv.take(kTileB * d);
-    float *sdO = cv.take(kTileB * dv);
-    float *sPhi = cv.take(kTileB * D);
-    float *sdPhi = cv.take(kTileB * D);
-    float *sdnum = cv.take(kTileB * dv);
-    float *sden = cv.take(kTileB);
-    float *sdden = cv.take(kTileB);
-    float *sU = cv.take(kTileB * M);
-    int *sJ = reinterpret_cast<int *>(cv.take(kTileB * M));
-    float *sdU = cv.take(kTileB * M);
+    const int D = a.D, dv = a.dv, d = a.d, M = a.M, Dp = (D + 3) & ~3, dvp = (dv + 3) & ~3;
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    float *tiles = cv.p;
+    const Rows sS = take_rows(cv, Dp, dv);
+    float *sz = cv.take(Dp);
+    const Rows sQ = take_rows(cv, cap, d), sdO = take_rows(cv, cap, dv), sPhi = take_rows(cv, cap, D);
+    Rows sP{cv.take(cap * max(row_stride(dv), row_stride(D))), row_stride(dv)};  // parts of dnum . num, then dphi(q_i)
+    const Rows sdPhi{sP.p, row_stride(D)};
+    const RowPairs rp = take_row_pairs(cv, cap);
+    float *sU = cv.take(cap * M);
+    int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
+    float *sdU = cv.take(cap * du_stride(M));
+    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(8));  // largest |S|, |z|, |phi|, |dO|, |dnum|, |dden|
+    cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
-    load_phi(s, lay, a.table);
+    zero_words(tiles, (int)(cv.p - tiles));
+    load_phi_tile(s, lay, a.table);
     const int bh = blockIdx.y, split = blockIdx.x;
     const size_t slot = (size_t)bh * a.nsplit_b + split;
-    double *gp = reinterpret_cast<double *>(a.gpart) + slot * a.gsize;
-    double *shist = gp + M * d + M;  // the block's fp64 histogram, accumulated in place by L2 atomics
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) sS[e] = a.S_fin[head_state(a, bh) * D * dv + e];
-    for (int e = threadIdx.x; e < D; e += blockDim.x) sz[e] = a.z_fin[head_state(a, bh) * D + e];
-    for (int e = threadIdx.x; e < mlp_words(lay) + var_words(lay); e += blockDim.x) shist[e] = 0.0;
+    double *gp = reinterpret_cast<double *>(a.gpart) + (slot % nbuf) * a.gsize;
+    double *hist = gp + M * d + M;
+    __syncthreads();
+    load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv);
+    __syncthreads();
+    tile_max(sS.p, Dp * sS.ld, mx);
+    tile_max(sz, Dp, mx + 1);
 
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = split * a.rows_per_split_b;
@@ -215,71 +231,79 @@ __global__ void __launch_bounds__(kThreads) k_bwd_query(AttnArgs a) {
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *dO = static_cast<const IO *>(a.dO) + head_rows(a, bh) * dv;
     IO *dQ = static_cast<IO *>(a.dQ) + head_rows(a, bh) * d;
-    // padded rows of this range receive zero gradients
-    for (int e = threadIdx.x + max(r0, len) * d; e < rend * d; e += blockDim.x) io_store(dQ + e, 0.0f);
+    zero_rows(dQ, max(r0, len), rend, d);  // padded rows of this range receive zero gradients
 
-    const int nc = (dv + 7) / 8, nf = (D + 7) / 8;
-    const bool active = threadIdx.x < nf * nc;
-    const int tf = active ? threadIdx.x / nc : 0, tc = active ? threadIdx.x % nc : 0;
-    const int f0 = tf * 8, c0 = tc * 8;
-    double acc[8][8] = {}, zacc[8] = {};
-    GradAcc g = {};
-    for (int t0 = r0; t0 < r1; t0 += kTileB) {
-        const int nr = min(kTileB, r1 - t0);
+    const Rows none{};
+    OuterAcc<TF, TC> acc;
+    acc.zero();
+    GradTile g;
+    grad_zero(g);
+    for (int t0 = r0; t0 < r1; t0 += cap) {
+        const int nr = min(cap, r1 - t0);
         __syncthreads();
-        load_rows(sQ, Q + (size_t)t0 * d, nr * d);
-        load_rows(sdO, dO + (size_t)t0 * dv, nr * dv);
+        if (threadIdx.x < 4) mx[2 + threadIdx.x] = 0u;
+        load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
+        load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_tile(lay, s, sQ, nr, sPhi, sU, sJ);
+        phi_rows(lay, s, sQ, nr, cap, sPhi, sU, sJ, mx + 2);
+        tile_max(sdO.p, cap * sdO.ld, mx + 3);
         __syncthreads();
-        // den and o_i are formed in fp64 and rounded once: the gradients below cancel to a small part of
-        // their terms (the loss barely changes under a common scale of phi(q_i)), so each row's rounding
-        // must stay at half an ulp
-        for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-            double den = a.eps;
-            for (int f = 0; f < D; ++f) den = fma((double)sPhi[r * D + f], (double)sz[f], den);
-            sden[r] = (float)den;
-        }
+        row_dots(sPhi, nr, D, [&](int, int f) { return sz[f]; }, none, [](int) { return 0; },
+                 [&](int r, float h, float l) { rp.set_den(r, h, l, a.eps); });
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {  // o_i into sdnum for now
-            const int r = e / dv, c = e - r * dv;
-            float o = 0.0f;
-            if (sden[r] != 0.0f) {
-                double num = 0.0;
-                for (int f = 0; f < D; ++f) num = fma((double)sPhi[r * D + f], (double)sS[f * dv + c], num);
-                o = (float)(num / (double)sden[r]);
+        {
+            float m = 0.0f;
+            for (int e = threadIdx.x; e < nr * dvp; e += blockDim.x) {  // dnum in place
+                const int r = e / dvp, c = e - r * dvp;
+                const float v = rp.over_den(r, sdO[r][c]);
+                sdO[r][c] = v;
+                m = fmaxf(m, fabsf(v));
             }
-            sdnum[e] = o;
+            block_max(m, mx + 4);
         }
         __syncthreads();
-        for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-            double dot = 0.0;  // dden and dphi are formed in fp64 and rounded once: they cancel
-            for (int c = 0; c < dv; ++c) dot = fma((double)sdO[r * dv + c], (double)sdnum[r * dv + c], dot);
-            sdden[r] = (sden[r] != 0.0f) ? (float)(-dot / (double)sden[r]) : 0.0f;
-        }
+        const float mS = __uint_as_float(mx[0]), mz = __uint_as_float(mx[1]), mp = __uint_as_float(mx[2]);
+        const float mdO = __uint_as_float(mx[3]);
+        const float bnum = pair_base((float)D * mS * mp);
+        prod_nn(sPhi, nr, sS, Dp, dv, none, none, [&](int) { return bnum; },
+                [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
+                    unit_dots(sdO, sP, nr, q0, c0, h, l, bnum);
+                });
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-            const int r = e / dv;
-            sdnum[e] = (sden[r] != 0.0f) ? (float)((double)sdO[e] / (double)sden[r]) : 0.0f;
-        }
+        sum_unit_dots(sP, nr, dvp / 4, [&](int r, float h, float l) {
+            rp.set_dden(r, h, l);
+            atomicMax(mx + 5, __float_as_uint(fabsf(rp.gh[r])));
+        });
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * D; e += blockDim.x) {
-            const int r = e / D, f = e - r * D;
-            double acc2 = (double)sz[f] * (double)sdden[r];
-            for (int c = 0; c < dv; ++c) acc2 = fma((double)sS[f * dv + c], (double)sdnum[r * dv + c], acc2);
-            sdPhi[e] = (float)acc2;
-        }
+        const float bound = (float)nr * mp;
+        acc.add(sPhi, D, sdO, dv, rp.gh, rp.gl, nr, pair_base(bound * __uint_as_float(mx[4])),
+                pair_base(bound * __uint_as_float(mx[5])));
+        const float bdot = 2.0f * (float)dv * mS * mdO;
+        auto base = [&](int r) {
+            return r < nr && rp.dh[r] != 0.0f ? pair_base(fmaf(bdot, fabsf(rp.inv[r]), mz * fabsf(rp.gh[r]))) : 0.0f;
+        };
+        prod_nt<kNone>(sdO, nr, sS, D, dvp, none, none, 0,
+                       [&](int r, int f, float &h, float &l) {
+                           h = base(r);
+                           l = 0.0f;
+                           if (r < nr) {
+                               l = sz[f] * rp.gl[r];
+                               pair_mac(h, l, sz[f], rp.gh[r]);
+                           }
+                       },
+                       [&](int r, int f, float h, float l) {
+                           if (r < nr) sdPhi[r][f] = pair_value(h - base(r), l);
+                       });
         __syncthreads();
-        if (active) outer_accumulate(acc, zacc, true, sPhi, D, sdnum, dv, sdden, nr, f0, c0);
-        phi_backward_tile(lay, s, sQ, nr, sPhi, sdPhi, sU, sJ, sdU, shist, shist + mlp_words(lay), g);
-        store_dx(lay, s, sdU, nr, dQ + (size_t)t0 * d);
+        phi_backward_rows(lay, s, sQ, nr, cap, sPhi, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
+        store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
-    __syncthreads();
-    store_tile(acc, zacc, active, tc, f0, c0, D, dv, a.dS_part + slot * D * dv, a.dz_part + slot * D);
-    store_grad_partial(lay, g, gp);
-    if (last_arrival(a.counters + a.B * a.H + bh, a.nsplit_b)) {
-        ordered_sum(a.dS_part + (size_t)bh * a.nsplit_b * D * dv, a.nsplit_b, D * dv, a.dS_fin + (size_t)bh * D * dv);
-        ordered_sum(a.dz_part + (size_t)bh * a.nsplit_b * D, a.nsplit_b, D, a.dz_fin + (size_t)bh * D);
+    acc.store(D, dv, a.dS_part, a.dz_part, slot, true);
+    add_grad_tile(lay, g, gp);
+    if (finish && last_arrival(a.counters + a.B * a.H + bh, a.nsplit_b)) {
+        const int np = 2 * a.nsplit_b;
+        ordered_sum(a.dS_part + (size_t)bh * np * D * dv, np, D * dv, a.dS_fin + (size_t)bh * D * dv);
+        ordered_sum(a.dz_part + (size_t)bh * np * D, np, D, a.dz_fin + (size_t)bh * D);
         if (threadIdx.x == 0) a.counters[a.B * a.H + bh] = 0;
     }
 }
@@ -287,30 +311,32 @@ __global__ void __launch_bounds__(kThreads) k_bwd_query(AttnArgs a) {
 // key side of the backward pass (non-causal):
 //   dv_j = dS^T phi(k_j),  dphi(k_j) = dS v_j + dz
 template <typename IO>
-__global__ void __launch_bounds__(kThreads) k_bwd_key(AttnArgs a) {
+__global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nbuf) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
-    const int D = a.D, dv = a.dv, d = a.d, M = a.M;
-    SmemPhi s = carve_phi(cv, lay);
-    float *sdS = cv.take(D * dv);
-    float *sdz = cv.take(D);
-    float *sK = cv.take(kTileB * d);
-    float *sV = cv.take(kTileB * dv);
-    float *sPhi = cv.take(kTileB * D);
-    float *sdPhi = cv.take(kTileB * D);
-    float *sU = cv.take(kTileB * M);
-    int *sJ = reinterpret_cast<int *>(cv.take(kTileB * M));
-    float *sdU = cv.take(kTileB * M);
+    const int D = a.D, dv = a.dv, d = a.d, M = a.M, Dp = (D + 3) & ~3, dvp = (dv + 3) & ~3;
+    SmemPhi s = carve_phi_tile(cv, lay, cap);
+    float *tiles = cv.p;
+    const Rows sdS = take_rows(cv, Dp, dv);
+    float *sdz = cv.take(Dp);
+    const Rows sK = take_rows(cv, cap, d), sV = take_rows(cv, cap, dv), sPhi = take_rows(cv, cap, D);
+    const Rows sdPhi = take_rows(cv, cap, D);
+    float *sU = cv.take(cap * M);
+    int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
+    float *sdU = cv.take(cap * du_stride(M));
+    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(4));  // largest |dS|, |dz|, |V|
     if (!carve_fits(cv, smem)) return;
-    load_phi(s, lay, a.table);
+    zero_words(tiles, (int)(cv.p - tiles));
+    load_phi_tile(s, lay, a.table);
     const int bh = blockIdx.y, split = blockIdx.x;
-    const size_t slot = (size_t)a.B * a.H * a.nsplit_b + (size_t)bh * a.nsplit_b + split;
-    double *gp = reinterpret_cast<double *>(a.gpart) + slot * a.gsize;
-    double *shist = gp + M * d + M;  // the block's fp64 histogram, accumulated in place by L2 atomics
-    for (int e = threadIdx.x; e < D * dv; e += blockDim.x) sdS[e] = a.dS_fin[(size_t)bh * D * dv + e];
-    for (int e = threadIdx.x; e < D; e += blockDim.x) sdz[e] = a.dz_fin[(size_t)bh * D + e];
-    for (int e = threadIdx.x; e < mlp_words(lay) + var_words(lay); e += blockDim.x) shist[e] = 0.0;
+    double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nsplit_b + split) % nbuf) * a.gsize;
+    double *hist = gp + M * d + M;
+    __syncthreads();
+    load_state(sdS, sdz, a.dS_fin + (size_t)bh * D * dv, a.dz_fin + (size_t)bh * D, D, dv);
+    __syncthreads();
+    tile_max(sdS.p, Dp * sdS.ld, mx);
+    tile_max(sdz, Dp, mx + 1);
 
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = split * a.rows_per_split_b;
@@ -320,36 +346,77 @@ __global__ void __launch_bounds__(kThreads) k_bwd_key(AttnArgs a) {
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
     IO *dK = static_cast<IO *>(a.dK) + head_rows(a, bh) * d;
     IO *dV = static_cast<IO *>(a.dV) + head_rows(a, bh) * dv;
-    for (int e = threadIdx.x + max(r0, len) * d; e < rend * d; e += blockDim.x) io_store(dK + e, 0.0f);
-    for (int e = threadIdx.x + max(r0, len) * dv; e < rend * dv; e += blockDim.x) io_store(dV + e, 0.0f);
+    zero_rows(dK, max(r0, len), rend, d);
+    zero_rows(dV, max(r0, len), rend, dv);
 
-    GradAcc g = {};
-    for (int t0 = r0; t0 < r1; t0 += kTileB) {
-        const int nr = min(kTileB, r1 - t0);
+    const Rows none{};
+    const bool vec = vec_store(dV, dv);
+    GradTile g;
+    grad_zero(g);
+    for (int t0 = r0; t0 < r1; t0 += cap) {
+        const int nr = min(cap, r1 - t0);
         __syncthreads();
-        load_rows(sK, K + (size_t)t0 * d, nr * d);
-        load_rows(sV, V + (size_t)t0 * dv, nr * dv);
+        if (threadIdx.x == 0) mx[2] = 0u;
+        load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_tile(lay, s, sK, nr, sPhi, sU, sJ);
+        phi_rows(lay, s, sK, nr, cap, sPhi, sU, sJ, nullptr);
+        tile_max(sV.p, cap * sV.ld, mx + 2);
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * dv; e += blockDim.x) {
-            const int r = e / dv, c = e - r * dv;
-            float acc2 = 0.0f;
-            for (int f = 0; f < D; ++f) acc2 = fmaf(sPhi[r * D + f], sdS[f * dv + c], acc2);
-            io_store(dV + (size_t)t0 * dv + e, acc2);
-        }
-        for (int e = threadIdx.x; e < nr * D; e += blockDim.x) {
-            const int r = e / D, f = e - r * D;
-            double acc2 = sdz[f];
-            for (int c = 0; c < dv; ++c) acc2 = fma((double)sdS[f * dv + c], (double)sV[r * dv + c], acc2);
-            sdPhi[e] = (float)acc2;
-        }
+        prod_nn_plain(sPhi, nr, sdS, Dp, dv, none, none, 0, [&](int q0, int c0, const float (&h)[2][4]) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);
+        });
+        const float base = pair_base(fmaf((float)dv * __uint_as_float(mx[0]), __uint_as_float(mx[2]),
+                                          __uint_as_float(mx[1])));
+        prod_nt<kNone>(sV, nr, sdS, D, dvp, none, none, 0,
+                       [&](int, int f, float &h, float &l) {
+                           h = base;
+                           l = 0.0f;
+                           pair_mac(h, l, sdz[f], 1.0f);
+                       },
+                       [&](int r, int f, float h, float l) {
+                           if (r < nr) sdPhi[r][f] = pair_value(h - base, l);
+                       });
         __syncthreads();
-        phi_backward_tile(lay, s, sK, nr, sPhi, sdPhi, sU, sJ, sdU, shist, shist + mlp_words(lay), g);
-        store_dx(lay, s, sdU, nr, dK + (size_t)t0 * d);
+        phi_backward_rows(lay, s, sK, nr, cap, sPhi, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
+        store_dx_rows(lay, s, sdU, nr, dK + (size_t)t0 * d);
     }
-    __syncthreads();
-    store_grad_partial(lay, g, gp);
+    add_grad_tile(lay, g, gp);
+}
+
+// ---------------------------------------------------------------------------
+// The partials of every head summed (or scanned) in order, one element per thread with eight loads in flight.
+
+__global__ void __launch_bounds__(256) k_part_reduce(PartReduce mode, int np, int nS, int nz, const float *S_part,
+                                                     const float *z_part, float *S, float *z, size_t S_step,
+                                                     size_t z_step, int hs_mul) {
+    int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool isz = e >= nS;
+    if (isz) e -= nS;
+    const int count = isz ? nz : nS;
+    if (e >= count) return;
+    const float *p = (isz ? z_part : S_part) + (size_t)blockIdx.y * np * count + e;
+    float *out = (isz ? z + (size_t)blockIdx.y * hs_mul * z_step : S + (size_t)blockIdx.y * hs_mul * S_step) + e;
+    double t = 0.0;
+    for (int p0 = 0; p0 < np; p0 += 8) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int q = p0 + k;
+            v[k] = q < np ? __ldcg(p + (size_t)(mode == kScanDown ? np - 1 - q : q) * count) : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int q = p0 + k;
+            if (q >= np) break;
+            if (mode != kSum) out[(size_t)(mode == kScanDown ? np - 1 - q : q) * count] = (float)t;
+            t += (double)v[k];
+        }
+    }
+    if (mode == kSum) *out = (float)t;
+    else if (mode == kScanUp) out[(size_t)np * count] = (float)t;
 }
 
 // ---------------------------------------------------------------------------
@@ -572,37 +639,88 @@ __global__ void __launch_bounds__(128) k_mlp_fc1_sum(TableLayout lay, const doub
 // ---------------------------------------------------------------------------
 // host side
 
-size_t smem_keystats(const AttnArgs &a) {
-    HostCarve cv; carve_phi_host(cv, a.lay);
-    cv.take(kTileK * a.d); cv.take(kTileK * a.dv); cv.take(kTileK * a.D);
+size_t smem_keystats(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
+    cv.take(4); cv.take(kSlack);
     return cv.bytes();
 }
-size_t smem_query(const AttnArgs &a) {
-    HostCarve cv; carve_phi_host(cv, a.lay);
-    cv.take(a.D * a.dv); cv.take(a.D); cv.take(kTileQ * a.d); cv.take(kTileQ * a.D); cv.take(kTileQ);
+size_t smem_query(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, r4(a.D), a.dv); cv.take(a.D); take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.D);
+    cv.take(cap);
     return cv.bytes();
 }
-size_t smem_bwd_query(const AttnArgs &a) {
-    HostCarve cv; carve_phi_host(cv, a.lay);
-    cv.take(a.D * a.dv); cv.take(a.D); cv.take(kTileB * a.d); cv.take(kTileB * a.dv); cv.take(kTileB * a.D);
-    cv.take(kTileB * a.D); cv.take(kTileB * a.dv); cv.take(kTileB); cv.take(kTileB); cv.take(kTileB * a.M);
-    cv.take(kTileB * a.M); cv.take(kTileB * a.M);
+size_t smem_bwd_query(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
+    take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
+    cv.take(cap * std::max(row_stride(a.dv), row_stride(a.D)));
+    take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
+    cv.take(8); cv.take(kSlack);
     return cv.bytes();
 }
-size_t smem_bwd_key(const AttnArgs &a) {
-    HostCarve cv; carve_phi_host(cv, a.lay);
-    cv.take(a.D * a.dv); cv.take(a.D); cv.take(kTileB * a.d); cv.take(kTileB * a.dv); cv.take(kTileB * a.D);
-    cv.take(kTileB * a.D); cv.take(kTileB * a.M); cv.take(kTileB * a.M); cv.take(kTileB * a.M);
+size_t smem_bwd_key(const AttnArgs &a, int cap) {
+    HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
+    take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
+    take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
+    take_rows_host(cv, cap, a.D);
+    cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M)); cv.take(4);
     return cv.bytes();
 }
 
+// Rows per block of a kernel that walks `n` rows of each of BH heads in tiles of cap rows, in at most max_splits
+// ranges per head.  Of the splits that fill one to eight waves of one block per SM, the one with the smallest
+// time in tiles: waves x (tiles per block + the half tile that a block's table and state loads take).
+struct Range { int splits, rows; };
+Range split_rows(int BH, int n, int cap, int max_splits) {
+    const int64_t tiles = (n + cap - 1) / cap;
+    Range best{1, (int)(tiles * cap)};
+    double best_cost = 1e300;
+    for (int w = 1; w <= 8; ++w) {
+        int64_t ns = std::max<int64_t>(1, (int64_t)w * kSMs / BH);
+        ns = std::min<int64_t>(std::min<int64_t>(ns, tiles), max_splits);
+        const int64_t tps = (tiles + ns - 1) / ns;
+        ns = (tiles + tps - 1) / tps;
+        const double cost = (double)((BH * ns + kSMs - 1) / kSMs) * ((double)tps + 0.5);
+        if (cost < best_cost * 0.999) {
+            best_cost = cost;
+            best = Range{(int)ns, (int)(tps * cap)};
+        }
+    }
+    return best;
+}
+
 template <typename IO>
-cudaError_t stats_impl(const AttnArgs &a, cudaStream_t s) {
-    const size_t sm = smem_keystats(a);
-    cudaError_t e = set_smem(k_keystats<IO>, sm);
+cudaError_t stats_impl(const AttnArgs &a0, cudaStream_t s) {
+    AttnArgs a = a0;
+    const int cap = pick_cap(a.B * a.H, a.n, [&](int c) { return smem_keystats(a, c); });
+    int pairs = 0;
+    if (!a.seg_S) {  // (the streaming form's ranges are its state segments)
+        const Range r = split_rows(a.B * a.H, a.n, cap, a.nsplit);
+        pairs = 2 * r.splits <= a.nsplit;  // the partials' buffer has room for high and low parts
+        a.nsplit = r.splits;
+        a.rows_per_split = r.rows;
+    }
+    const size_t sm = smem_keystats(a, cap);
+    cudaError_t e = cudaSuccess;
+    outer_dispatch(a.D, a.dv, [&](auto tf, auto tc) {
+        auto k = k_keystats<IO, decltype(tf)::value, decltype(tc)::value>;
+        if ((e = set_smem(k, sm)) != cudaSuccess) return;
+        LUNA_LAUNCH("keystats", k, dim3(a.nsplit, a.B * a.H), kThr, sm, s, a, cap, pairs, a.nsplit <= kFinishParts);
+        e = cudaGetLastError();
+    });
     if (e != cudaSuccess) return e;
-    LUNA_LAUNCH("keystats", k_keystats<IO>, dim3(a.nsplit, a.B * a.H), kThreads, sm, s, a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (a.nsplit > kFinishParts) {
+        const size_t SD = (size_t)a.D * a.dv;
+        if (a.seg_S)
+            e = launch_part_reduce(kScanUp, a, a.nsplit, a.S_part, a.z_part, a.seg_S, a.seg_z, (a.nsplit + 1) * SD,
+                                   (size_t)(a.nsplit + 1) * a.D, s);
+        else
+            e = launch_part_reduce(kSum, a, pairs ? 2 * a.nsplit : a.nsplit, a.S_part, a.z_part, a.S_fin, a.z_fin, SD,
+                                   a.D, s);
+        if (e != cudaSuccess) return e;
+    }
     return launch_chrms_scale_state(a, s);
 }
 
@@ -610,40 +728,68 @@ template <typename IO>
 cudaError_t fwd_impl(const AttnArgs &a, cudaStream_t s) {
     cudaError_t e = stats_impl<IO>(a, s);
     if (e != cudaSuccess) return e;
-    const size_t sm = smem_query(a);
+    const int cap = pick_cap(a.B * a.H, a.n, [&](int c) { return smem_query(a, c); });
+    const Range r = split_rows(a.B * a.H, a.n, cap, 1 << 24);
+    const size_t sm = smem_query(a, cap);
     if ((e = set_smem(k_query<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("query", k_query<IO>, dim3((a.n + kTileQ - 1) / kTileQ, a.B * a.H), kThreads, sm, s, a);
+    LUNA_LAUNCH("query", k_query<IO>, dim3(r.splits, a.B * a.H), kThr, sm, s, a, cap, r.rows);
     return cudaGetLastError();
 }
 
 template <typename IO>
 cudaError_t bwd_impl(const AttnArgs &a0, bool have_stats, cudaStream_t s) {
     AttnArgs a = a0;
-    a.gpart64 = 1;  // the generic kernels write fp64 parameter-gradient partials
+    a.gpart64 = 1;  // the generic kernels write fp64 parameter-gradient sums
     cudaError_t e;
     if (!have_stats && (e = stats_impl<IO>(a, s)) != cudaSuccess) return e;
-    size_t sm = smem_bwd_query(a);
-    if ((e = set_smem(k_bwd_query<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("bwd_query", k_bwd_query<IO>, dim3(a.nsplit_b, a.B * a.H), kThreads, sm, s, a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int BH = a.B * a.H;
+    const int cap = pick_cap(BH, a.n, [&](int c) { return std::max(smem_bwd_query(a, c), smem_bwd_key(a, c)); });
+    const Range r = split_rows(BH, a.n, cap, a.nsplit_b);
+    const int64_t slots = 2 * (int64_t)BH * a.nsplit_b;
+    a.nsplit_b = r.splits;
+    a.rows_per_split_b = r.rows;
+    const int nbuf = grad_buffers(BH * (int64_t)r.splits, slots);
+    if ((e = cudaMemsetAsync(a.gpart, 0, (size_t)nbuf * a.gsize * sizeof(double), s)) != cudaSuccess) return e;
+    size_t sm = smem_bwd_query(a, cap);
+    outer_dispatch(a.D, a.dv, [&](auto tf, auto tc) {
+        auto k = k_bwd_query<IO, decltype(tf)::value, decltype(tc)::value>;
+        if ((e = set_smem(k, sm)) != cudaSuccess) return;
+        LUNA_LAUNCH("bwd_query", k, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, nbuf, a.nsplit_b <= kFinishParts);
+        e = cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
+    if (a.nsplit_b > kFinishParts) {
+        AttnArgs b = a;
+        b.hs_mul = 1;  // dS, dz are indexed by the sub-problem's own heads
+        if ((e = launch_part_reduce(kSum, b, 2 * a.nsplit_b, a.dS_part, a.dz_part, a.dS_fin, a.dz_fin,
+                                    (size_t)a.D * a.dv, a.D, s)) != cudaSuccess)
+            return e;
+    }
     if ((e = launch_chrms_dstate(a, s)) != cudaSuccess) return e;
-    sm = smem_bwd_key(a);
+    sm = smem_bwd_key(a, cap);
     if ((e = set_smem(k_bwd_key<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("bwd_key", k_bwd_key<IO>, dim3(a.nsplit_b, a.B * a.H), kThreads, sm, s, a);
+    LUNA_LAUNCH("bwd_key", k_bwd_key<IO>, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, nbuf);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     int nparts = 0;
-    if ((e = launch_chrms_backward(a, 2 * a.B * a.H * a.nsplit_b, &nparts, s)) != cudaSuccess) return e;
+    if ((e = launch_chrms_backward(a, nbuf, &nparts, s)) != cudaSuccess) return e;
     return launch_grad_reduce(a, nparts, s);
 }
 
 }  // namespace
 
+cudaError_t launch_part_reduce(PartReduce mode, const AttnArgs &a, int np, const float *S_part, const float *z_part,
+                               float *S, float *z, size_t S_step, size_t z_step, cudaStream_t s) {
+    const int nS = a.D * a.dv;
+    LUNA_LAUNCH("part_reduce", k_part_reduce, dim3((nS + a.D + 255) / 256, a.B * a.H), 256, 0, s, mode, np, nS, a.D, S_part,
+                z_part, S, z, S_step, z_step, a.hs_mul);
+    return cudaGetLastError();
+}
+
 size_t simt_max_smem(const AttnArgs &a) {
-    size_t m = smem_keystats(a);
-    m = m > smem_query(a) ? m : smem_query(a);
-    m = m > smem_bwd_query(a) ? m : smem_bwd_query(a);
-    m = m > smem_bwd_key(a) ? m : smem_bwd_key(a);
-    return m;
+    size_t m = smem_keystats(a, kMinC);
+    m = std::max(m, smem_query(a, kMinC));
+    m = std::max(m, smem_bwd_query(a, kMinC));
+    return std::max(m, smem_bwd_key(a, kMinC));
 }
 
 cudaError_t launch_grad_reduce(const AttnArgs &a, int nparts, cudaStream_t s) {
@@ -671,8 +817,8 @@ cudaError_t launch_grad_reduce(const AttnArgs &a, int nparts, cudaStream_t s) {
 cudaError_t launch_featmap(const TableLayout &lay, const char *table, const void *X, luna_dtype xt, int64_t rows,
                            float *Phi, cudaStream_t s) {
     if (lay_variant(lay)) {
-        HostCarve cv; carve_phi_host(cv, lay);
-        cv.take(kPhiRows * lay.d); cv.take(kPhiRows * lay.D);
+        HostCarve cv; carve_phi_tile_host(cv, lay, kPhiRows);
+        take_rows_host(cv, kPhiRows, lay.d); take_rows_host(cv, kPhiRows, lay.D);
         const size_t sm = cv.bytes();
         const int64_t tiles = (rows + kPhiRows - 1) / kPhiRows;
         const int blocks = (int)(tiles < 4096 ? (tiles > 0 ? tiles : 1) : 4096);
@@ -687,7 +833,7 @@ cudaError_t launch_featmap(const TableLayout &lay, const char *table, const void
         }
         return cudaGetLastError();
     }
-    HostCarve cv; carve_phi_host(cv, lay);
+    HostCarve cv; carve_phi_tile_host(cv, lay, 0);
     const size_t sm = cv.bytes();
     int64_t work = rows * lay.M;
     int blocks = (int)((work + kThreads - 1) / kThreads);

@@ -31,7 +31,8 @@ struct AttnArgs {
     int chunk, seg_len, nseg;          // state segments of seg_len rows (multiple of chunk)
     float *seg_S, *seg_z;              // [BH][nseg+1][D][dv], [BH][nseg+1][D]: prefix at each segment start, total last
     float *seg_dS, *seg_dz;            // [BH][nseg][D][dv], [BH][nseg][D]: suffix after segment end
-    float *rowstat;                    // [BH][n][2]: (den_i, dden_i) of the backward pass
+    float *rowstat;                    // backward pass, per row: [BH][n][4] den_i and dden_i as pairs
+                                       // (tensor cores: [BH][n][2])
     // streaming-form backward on tensor cores
     float *dphi;                       // [BH][n][D] fp32: dLoss/dphi of Q, then of K
     void *phik, *pq2;                  // [BH][n][2D] bf16 phi(k), phi(q)/den, each as (hi | lo)
@@ -90,6 +91,14 @@ cudaError_t launch_featmap(const TableLayout &lay, const char *table, const void
 cudaError_t launch_simt_fwd(const AttnArgs &a, luna_dtype io, cudaStream_t s);
 cudaError_t launch_simt_stats(const AttnArgs &a, luna_dtype io, cudaStream_t s);
 cudaError_t launch_simt_bwd(const AttnArgs &a, luna_dtype io, bool have_stats, cudaStream_t s);
+// Sums (kSum), forward exclusive prefixes with the total last (kScanUp) or exclusive suffixes (kScanDown) of each
+// head's np partials [np][D][dv], [np][D] into S, z (steps S_step, z_step between the heads' blocks).  A kernel that
+// writes at most kFinishParts partials per head lets the head's last block do this instead: with more, that one
+// block's loads are a serial tail (16 elements per thread and 304 partials: 0.3 ms at one head of 40k rows).
+enum PartReduce { kSum, kScanUp, kScanDown };
+constexpr int kFinishParts = 8;
+cudaError_t launch_part_reduce(PartReduce mode, const AttnArgs &a, int np, const float *S_part, const float *z_part,
+                               float *S, float *z, size_t S_step, size_t z_step, cudaStream_t s);
 cudaError_t launch_grad_reduce(const AttnArgs &a, int nparts, cudaStream_t s);
 cudaError_t launch_causal_fwd(const AttnArgs &a, luna_dtype io, bool write_state, cudaStream_t s);
 cudaError_t launch_causal_bwd(const AttnArgs &a, luna_dtype io, bool have_state, cudaStream_t s);
