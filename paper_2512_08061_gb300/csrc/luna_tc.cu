@@ -1,14 +1,16 @@
 // Tensor-core (tcgen05 / TMEM / TMA) kernels for bf16 I/O on sm_103a.
 //
 // Persistent kernels: one block per SM walks a contiguous range of work items
-// (head, chunk of 128-row tiles).  Warp roles in a block of 576 threads:
+// (head, chunk of 128-row tiles).  Warp roles in a block of 704 threads:
 //   warps 0..15  workers, four per row: warps w, w+4, w+8, w+12 own TMEM lanes
 //                32*(w%4)..+31 and each evaluates the feature map for a
 //                quarter of the M projections of those rows;
 //   warp 16      TMA: lane 0 streams the X (query / key) tiles, lane 1 the V
 //                tiles, each into its own ring of shared-memory stages;
 //   warp 17      MMA: lane 0 issues every tcgen05.mma and commits it to the
-//                mbarriers that release stages and wake the workers.
+//                mbarriers that release stages and wake the workers;
+//   warps 18..21 move a head's statistics out of tensor memory (key pass) or
+//                into the operand of the next head (query pass).
 //
 // Forward key pass per tile (Sec. 4, S_KV and S_K1):
 //   MMA  U = K [W_hi; W_lo]^T                      (projections -> TMEM)
@@ -18,7 +20,7 @@
 //   MMA  S += [phi_hi | phi_lo]^T V                 (MN-major operands)
 // Forward query pass (Eq. kernel-attn):
 //   MMA U, workers phi(Q) (bf16) and the fp32 normaliser phi.z,
-//   MMA  num = phi [S_hi; S_lo]^T,  O = num / (phi.z + eps)
+//   MMA  num = phi [S_hi | S_lo],  O = num / (phi.z + eps)
 // S and W enter their products split into bf16 hi + lo parts.
 #include <atomic>
 
@@ -32,8 +34,10 @@ using namespace tcdev;
 
 constexpr int kWorkerWarps = 16;
 constexpr int kWorkers = kWorkerWarps * 32;
-constexpr int kTmaWarp = 16, kMmaWarp = 17;
-constexpr int kThreadsTC = kWorkers + 64;
+constexpr int kTmaWarp = 16, kMmaWarp = 17, kAuxWarp = 18;
+constexpr int kAux = 128;  // four warps that move the statistics: out of tensor memory (keys), into the operand (queries)
+constexpr int kThreadsTC = kWorkers + 64 + kAux;
+constexpr int kNU = 3;     // projection buffers in tensor memory
 
 template <int DX_, int DV_, int MP_>
 struct Cfg {
@@ -59,58 +63,62 @@ struct Cfg {
     static constexpr int NX_K = SMALL ? 3 : 2;
     static constexpr int NV_K = SMALL ? 3 : 1;
     static constexpr int NP_K = SMALL ? 2 : 1;
-    static constexpr uint32_t ZPART = 4u * D * 4;
-    static constexpr uint32_t SSTAGE = MERGE ? 64u * DV * 4 : 0u;
+    static constexpr uint32_t ZPART = 2u * 4 * D * 4;
+    static constexpr uint32_t SSTAGE = MERGE ? 64u * (DV + 1) * 4 : 0u;  // odd stride: a row per lane
     static constexpr uint32_t FIX_K = WOP + TABLE + ZPART + SSTAGE + MISC + 1024;
     static constexpr uint32_t SMEM_K = NX_K * XT + NV_K * VT + NP_K * 2 * PT + FIX_K;
-    static constexpr int TMEM_K_USED = 2 * NU + 2 * DV;
+    static constexpr int TMEM_K_USED = kNU * NU + 2 * DV;
     static constexpr int TMEM_K = TMEM_K_USED <= 64 ? 64 : TMEM_K_USED <= 128 ? 128 : TMEM_K_USED <= 256 ? 256 : 512;
     // query pass
-    static constexpr uint32_t SOP = 2u * DV * D * 2;  // [S_hi; S_lo]^T operand
+    static constexpr uint32_t SOP = 2u * DV * D * 2;  // [S_hi | S_lo] operand: D rows, blocks of 64 columns
+    static constexpr int NSOP = SMALL ? 2 : 1;        // operand buffers: the next head's is written during this one's tiles
     static constexpr int NP_Q = SMALL ? 2 : 1;
     static constexpr int NX_Q = SMALL ? 4 : 2;
-    static constexpr uint32_t FIX_Q = WOP + SOP + TABLE + D * 4 + 2 * 4 * 128 * 4 + MISC + 1024;
+    static constexpr uint32_t FIX_Q = WOP + NSOP * SOP + TABLE + NSOP * D * 4 + 2 * 4 * 128 * 4 + MISC + 1024;
     static constexpr uint32_t SMEM_Q = NX_Q * XT + NP_Q * PT + FIX_Q;
-    static constexpr int NN_Q = (2 * NU + 4 * DV <= 256) ? 2 : 1;
-    static constexpr int TMEM_Q_USED = 2 * NU + 2 * DV * NN_Q;
+    static constexpr int NN_Q = (kNU * NU + 4 * DV <= 256) ? 2 : 1;
+    static constexpr int TMEM_Q_USED = kNU * NU + 2 * DV * NN_Q;
     static constexpr int TMEM_Q = TMEM_Q_USED <= 64 ? 64 : TMEM_Q_USED <= 128 ? 128 : TMEM_Q_USED <= 256 ? 256 : 512;
     static_assert(SMEM_K <= kSmemLimit && SMEM_Q <= kSmemLimit, "shared memory budget");
     static_assert(TMEM_K_USED <= 512 && TMEM_Q_USED <= 512, "tensor memory budget");
     static_assert(PP == 2 || PP == 4, "projections per worker");
 };
 
-// Worker: phi for projections [Q*PP, Q*PP+PP) of row r from the projection
-// columns in TMEM.  The PP interval searches run interleaved over the
-// bucketed search block (j = the number of kinks strictly below u).
+// Worker, first half: starts reading this thread's PP projections of a tile (hi parts at columns Q*PP.., lo parts
+// MP columns further; tmem_u_row: the row's projection columns).
+template <class C>
+struct Proj {
+    uint32_t xh[C::PP], xl[C::PP];
+    __device__ __forceinline__ void load(int Q, uint32_t tmem_u_row) {
+        if constexpr (C::PP == 2) {
+            tmem_ld2(tmem_u_row + Q * C::PP, xh);
+            tmem_ld2(tmem_u_row + C::MP + Q * C::PP, xl);
+        } else {
+            tmem_ld4(tmem_u_row + Q * C::PP, xh);
+            tmem_ld4(tmem_u_row + C::MP + Q * C::PP, xl);
+        }
+    }
+};
+
+// The projections u = hi + lo + bias and their intervals, from the columns `load` has started to read.
+template <class C>
+__device__ __forceinline__ void proj_search(const Proj<C> &x, const float (&bias)[C::PP], const float *sTe,
+                                            float (&u)[C::PP], int (&node)[C::PP]) {
+#pragma unroll
+    for (int q = 0; q < C::PP; ++q) u[q] = __uint_as_float(x.xh[q]) + __uint_as_float(x.xl[q]) + bias[q];
+    search_bucketed<C::PP>(sTe, u, node);
+}
+
+// Worker, second half: the channel values of projections [Q*PP, Q*PP+PP) of row r from u and its intervals.
 // Writes the bf16 chunks of the phi tile (and, if plo is not null, the bf16
 // residual phi - bf16(phi) into a second tile), zeros for rows that are not
 // valid.  Optionally adds phi into zacc (fp32 feature sums) and accumulates the
 // fp32 normaliser phi . z.
 template <class C>
-__device__ __forceinline__ void phi_row_quarter(int Q, uint32_t tmem_u_row, const float *sTe, const float *sAB,
-                                                const float *sbias, float fl, bool valid, int r, uint8_t *phi,
-                                                uint8_t *plo,
-                                                float *zacc, const float *sz, float &den) {
+__device__ __forceinline__ void phi_row_quarter(int Q, const float (&u)[C::PP], const int (&node)[C::PP],
+                                                const float *sAB, float fl, bool valid, int r, uint8_t *phi,
+                                                uint8_t *plo, float *zacc, const float *sz, float &den) {
     constexpr int PP = C::PP;
-    float u[PP];
-    {
-        // this thread's PP projections: hi parts at columns Q*PP.., lo parts MP columns further
-        uint32_t xh[PP], xl[PP];
-        if constexpr (PP == 2) {
-            tmem_ld2(tmem_u_row + Q * PP, xh);
-            tmem_ld2(tmem_u_row + C::MP + Q * PP, xl);
-        } else {
-            tmem_ld4(tmem_u_row + Q * PP, xh);
-            tmem_ld4(tmem_u_row + C::MP + Q * PP, xl);
-        }
-        tmem_wait_ld();
-#pragma unroll
-        for (int q = 0; q < PP; ++q) u[q] = __uint_as_float(xh[q]) + __uint_as_float(xl[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < PP; ++q) u[q] += sbias[Q * PP + q];
-    int node[PP];
-    search_bucketed<PP>(sTe, u, node);
 #pragma unroll
     for (int q = 0; q < PP; ++q) {
         const int i = Q * PP + q;
@@ -149,7 +157,26 @@ __device__ __forceinline__ void phi_row_quarter(int Q, uint32_t tmem_u_row, cons
     }
 }
 
-// Projection MMA of tile g into TMEM stage g & 1.
+// Sums each of N values (a power of two, at most 32) over the warp's lanes: the sum of value `lane * N / 32` is
+// returned (in 32 / N adjacent lanes).  Every step halves the values a lane holds; the pairs added are those of an
+// xor tree per value.
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
+    int o = 16;
+#pragma unroll
+    for (int half = N / 2; half >= 1; half /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < half; ++k) {
+            const float send = up ? v[k] : v[k + half], keep = up ? v[k + half] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    for (; o >= 1; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+
+// Projection MMA of a tile into a TMEM buffer.
 template <class C>
 __device__ __forceinline__ void issue_proj(uint32_t tmem_u, uint64_t dx, uint64_t dw) {
     constexpr uint32_t idesc = idesc_bf16(128, C::NU, false, false);
@@ -167,11 +194,20 @@ __device__ __forceinline__ void issue_proj(uint32_t tmem_u, uint64_t dx, uint64_
 // phi(K) enters the contraction as bf16 hi + lo tiles so that the key
 // statistics carry ~16 significant bits of phi (the backward pass subtracts
 // nearly equal terms built from S and z); z is summed by the workers in fp32.
-// Each run's statistics go to its partial slot; the last run of a head to
-// finish sums the partials in order (warps 0..3 only, so that the pipeline
-// keeps running).  Per-item mode (the state segments of the streaming form,
-// a.seg_S set): every item is its own run, its statistics go to slot
-// (head, item), and nothing is summed here.
+// The auxiliary warps read a run's statistics out of tensor memory while the
+// workers are already at the next run's tiles (accumulators and z partials are
+// double-buffered).  The statistics of a head that one block holds whole are
+// final; otherwise they go to the run's partial slot and the last run of the
+// head to finish sums the partials in order.  Per-item mode (the state segments
+// of the streaming form, a.seg_S set): every item is its own run, its
+// statistics go to slot (head, item), and nothing is summed here.
+//
+// Bound by the latency of the workers' chain (tensor-memory read, search,
+// table gather, operand store): a thread searches tile g + 1 while it evaluates
+// tile g, so that the two halves of the chain overlap.  Measured (us, before ->
+// after the auxiliary warps and the search ahead): 768 heads of 197 rows, d = 64,
+// 87 -> 44; 384 heads of 512, 61 -> 41; the LRA shape 63 -> 59; state segments
+// of 2048 heads of 1024 rows, d = 128, 470 -> 386.
 
 template <class C>
 __global__ void __launch_bounds__(kThreadsTC, 1)
@@ -187,18 +223,19 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     float *sTe = reinterpret_cast<float *>(Wop + C::WOP);
     float *sAB = sTe + kEytzinger;
     float *sbias = sAB + kNint * 16;
-    float *zpart = sbias + 32;         // [4][D]
-    float *sstage = zpart + 4 * C::D;  // [64][DV] (stacked operand only)
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sstage + C::SSTAGE / 4);
+    float *zpart = sbias + 32;         // [2][4][D]
+    float *sstage = zpart + 8 * C::D;  // [64][DV + 1] (stacked operand only)
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sstage + (C::SSTAGE / 4 + 1) / 2 * 2);
     uint64_t *fullx = bars;            // [NX] X tile landed
     uint64_t *xfree = fullx + NX;      // [NX] projection MMA consumed it
     uint64_t *fullv = xfree + NX;      // [NV] V tile landed
     uint64_t *vfree = fullv + NV;      // [NV] contraction consumed it
-    uint64_t *uready = vfree + NV;     // [2] projection in TMEM
-    uint64_t *phiready = uready + 2;   // [NP] workers wrote phi (count 512)
+    uint64_t *uready = vfree + NV;     // [kNU] projection in TMEM
+    uint64_t *phiready = uready + kNU; // [NP] workers wrote phi (one arrival per worker warp)
     uint64_t *pfree = phiready + NP;   // [NP] contraction consumed phi
-    uint64_t *accdone = pfree + NP;    // [2] item statistics complete
-    uint64_t *accfree = accdone + 2;   // [2] item statistics read (count 128)
+    uint64_t *accdone = pfree + NP;    // [2] run statistics complete in TMEM
+    uint64_t *zready = accdone + 2;    // [2] run's z partials written (one arrival per worker warp)
+    uint64_t *accfree = zready + 2;    // [2] run statistics and z partials read (one arrival per auxiliary warp)
     uint32_t *tslot = reinterpret_cast<uint32_t *>(accfree + 2);
     int *slast = reinterpret_cast<int *>(tslot + 1);
 
@@ -208,9 +245,11 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     if (tid == 0) {
         for (int i = 0; i < NX; ++i) { mbar_init(fullx + i, 1); mbar_init(xfree + i, 1); }
         for (int i = 0; i < NV; ++i) { mbar_init(fullv + i, 1); mbar_init(vfree + i, 1); }
-        for (int i = 0; i < 2; ++i) mbar_init(uready + i, 1);
-        for (int i = 0; i < NP; ++i) { mbar_init(phiready + i, kWorkers); mbar_init(pfree + i, 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(accdone + i, 1); mbar_init(accfree + i, 128); }
+        for (int i = 0; i < kNU; ++i) mbar_init(uready + i, 1);
+        for (int i = 0; i < NP; ++i) { mbar_init(phiready + i, kWorkers / 32); mbar_init(pfree + i, 1); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(accdone + i, 1); mbar_init(zready + i, kWorkers / 32); mbar_init(accfree + i, kAux / 32);
+        }
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, C::TMEM_K); tmem_relinquish(); }
@@ -222,7 +261,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tslot;
-    const uint32_t tmem_acc = tbase + 2 * C::NU;  // [2] x DV cols
+    const uint32_t tmem_acc = tbase + kNU * C::NU;  // [2] x DV cols
 
     if (warp == kTmaWarp) {
         if (lane < 2) {
@@ -266,12 +305,11 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                 const int x = g % NX;
                 wait_or_fail(fullx + x, (g / NX) & 1, failed, status);
                 tc_fence_after();
-                issue_proj<C>(tbase + (g & 1) * C::NU, dadd(dx0, x * C::XT), dw0);
-                mma_commit(uready + (g & 1));
+                issue_proj<C>(tbase + (g % kNU) * C::NU, dadd(dx0, x * C::XT), dw0);
+                mma_commit(uready + g % kNU);
                 mma_commit(xfree + x);
             };
-            if (T > 0) proj(0);
-            if (T > 1) proj(1);
+            for (int g = 0; g < kNU && g < T; ++g) proj(g);
             // runs: maximal stretches of this block's items that share a head; S accumulates over a run
             int g = 0, ne = 0;
             for (int i0 = it.begin; i0 < it.end && !failed;) {
@@ -301,21 +339,112 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                         mma_commit(pfree + p);
                         mma_commit(vfree + v);
                         if (t == run_tiles - 1) mma_commit(accdone + b);
-                        if (g + 2 < T) proj(g + 2);
+                        if (g + kNU < T) proj(g + kNU);
                     }
                     ++ne;
                 }
                 i0 = i1;
             }
         }
+    } else if (warp >= kAuxWarp) {
+        // TMEM lanes of this warp's quarter: accumulator rows, feature f, and (stacked operand) the lo part of
+        // feature f at row 64 + f
+        const int et = tid - kAuxWarp * 32, row = ((warp & 3) << 5) | lane;
+        const uint32_t lrow = (uint32_t)((warp & 3) << 5) << 16;
+        const int f = C::MERGE ? (row & 63) : row;
+        bool failed = false;
+        int ne = 0;
+        for (int i0 = it.begin; i0 < it.end;) {
+            const int bh = i0 / it.nchunk;
+            const int i1 = per_item ? i0 + 1 : min(it.end, (bh + 1) * it.nchunk);
+            int run_tiles = 0;
+            for (int item = i0; item < i1; ++item) run_tiles += item_range(a, it, item).ntiles;
+            const RunSlot rs = run_slot(a, it, bh);
+            const bool whole = !per_item && rs.nruns == 1;
+            const size_t slot = per_item ? (size_t)i0 : (size_t)bh * it.nchunk + rs.rank;
+            float *Sp = whole ? a.S_fin + head_state(a, bh) * C::D * C::DV : a.S_part + slot * C::D * C::DV;
+            float *zp = whole ? a.z_fin + head_state(a, bh) * C::D : a.z_part + slot * C::D;
+            const bool have = run_tiles > 0;
+            const int b = ne & 1;
+            if (have) {
+                wait_or_fail(accdone + b, (ne >> 1) & 1, failed, status);
+                wait_or_fail(zready + b, (ne >> 1) & 1, failed, status);
+                tc_fence_after();
+            }
+            const uint32_t tmem_s = lrow + tmem_acc + b * C::DV;
+            if (C::MERGE && row >= 64) {
+#pragma unroll
+                for (int c0 = 0; c0 < C::DV; c0 += 16) {
+                    uint32_t x[16];
+                    if (have) { tmem_ld16(tmem_s + c0, x); tmem_wait_ld(); }
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        sstage[f * (C::DV + 1) + c0 + c] = have ? __uint_as_float(x[c]) : 0.0f;
+                }
+            }
+            if constexpr (C::MERGE) named_sync<kAux>(2);
+            if (!C::MERGE || row < 64) {
+#pragma unroll
+                for (int c0 = 0; c0 < C::DV; c0 += 16) {
+                    uint32_t x[16];
+                    if (have) { tmem_ld16(tmem_s + c0, x); tmem_wait_ld(); }
+                    float o[16];
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        o[c] = have ? __uint_as_float(x[c]) : 0.0f;
+                        if (C::MERGE) o[c] += sstage[f * (C::DV + 1) + c0 + c];
+                    }
+#pragma unroll
+                    for (int c = 0; c < 16; c += 8)  // whole sectors
+                        st_v8(Sp + f * C::DV + c0 + c, f4_bits(make_float4(o[c], o[c + 1], o[c + 2], o[c + 3])),
+                              f4_bits(make_float4(o[c + 4], o[c + 5], o[c + 6], o[c + 7])));
+                }
+                const float *zb = zpart + b * 4 * C::D;
+                zp[f] = have ? zb[f] + zb[C::D + f] + zb[2 * C::D + f] + zb[3 * C::D + f] : 0.0f;
+            }
+            tc_fence_before();
+            if (have) { mbar_arrive_warp(accfree + b); ++ne; }
+            if constexpr (C::MERGE) named_sync<kAux>(2);  // sstage is read
+            if (!per_item && !whole) {
+                // the last block of this head to finish sums the partials in block order
+                __threadfence();
+                named_sync<kAux>(2);
+                if (et == 0) *slast = atomicAdd(a.counters + bh, 1) == rs.nruns - 1 ? 1 : 0;
+                named_sync<kAux>(2);
+                if (*slast) {
+                    __threadfence();
+                    ordered_sum4(a.S_part + (size_t)bh * it.nchunk * C::D * C::DV, rs.nruns, C::D * C::DV,
+                                 a.S_fin + head_state(a, bh) * C::D * C::DV, et, kAux);
+                    ordered_sum4(a.z_part + (size_t)bh * it.nchunk * C::D, rs.nruns, C::D,
+                                 a.z_fin + head_state(a, bh) * C::D, et, kAux);
+                    if (et == 0) a.counters[bh] = 0;
+                }
+                named_sync<kAux>(2);
+            }
+            i0 = i1;
+        }
     } else {
         const int Q = warp >> 2, r = ((warp & 3) << 5) | lane;
-        const uint32_t lrow = (uint32_t)((warp & 3) << 5) << 16;
-        float zacc[C::PP * 8];
+        const uint32_t urow = tbase + ((uint32_t)((warp & 3) << 5) << 16);
+        const float fl = channel_floor(a.lay);
+        float zacc[C::PP * 8], bias[C::PP];
 #pragma unroll
         for (int k = 0; k < C::PP * 8; ++k) zacc[k] = 0.0f;
+#pragma unroll
+        for (int q = 0; q < C::PP; ++q) bias[q] = sbias[Q * C::PP + q];
         float dummy = 0.0f;
         bool failed = false;
+        const int T = block_tiles(a, it);
+        Proj<C> x;
+        float u[C::PP];
+        int node[C::PP];
+        if (T > 0) {
+            wait_or_fail(uready, 0, failed, status);
+            tc_fence_after();
+            x.load(Q, urow);
+            tmem_wait_ld();
+            proj_search<C>(x, bias, sTe, u, node);
+        }
         int g = 0, ne = 0;
         for (int i0 = it.begin; i0 < it.end;) {
             const int bh = i0 / it.nchunk;
@@ -327,13 +456,16 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                 for (int t = 0; t < ir.ntiles; ++t, ++g) {
                     const int p = g % NP, v = g % NV;
                     const int nvalid = min(128, ir.r1 - (ir.r0 + t * 128));
-                    wait_or_fail(uready + (g & 1), (g >> 1) & 1, failed, status);
+                    const bool more = g + 1 < T;
+                    if (more) {  // the next tile's projections: three buffers, so they are usually there
+                        wait_or_fail(uready + (g + 1) % kNU, ((g + 1) / kNU) & 1, failed, status);
+                        tc_fence_after();
+                        x.load(Q, urow + ((g + 1) % kNU) * C::NU);
+                    }
                     if (g >= NP) wait_or_fail(pfree + p, ((g - NP) / NP) & 1, failed, status);
-                    tc_fence_after();
                     uint8_t *ph = Pb + p * 2 * C::PT, *pl = ph + C::PT;
                     const bool valid = r < nvalid;
-                    phi_row_quarter<C>(Q, tbase + lrow + (g & 1) * C::NU, sTe, sAB, sbias, channel_floor(a.lay), valid, r, ph, pl, zacc,
-                                   nullptr, dummy);
+                    phi_row_quarter<C>(Q, u, node, sAB, fl, valid, r, ph, pl, zacc, nullptr, dummy);
                     if (!valid && Q == 0) {  // padded rows: clear V so that no garbage enters S
                         wait_or_fail(fullv + v, (g / NV) & 1, failed, status);
                         uint8_t *vrow = Vb + v * C::VT;
@@ -344,95 +476,26 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                                 *reinterpret_cast<uint4 *>(vrow + vb * 16384 + sw128_chunk(r, c)) =
                                     make_uint4(0, 0, 0, 0);
                     }
+                    __syncwarp();
+                    tmem_wait_ld();
+                    if (more) proj_search<C>(x, bias, sTe, u, node);
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(phiready + p);
+                    mbar_arrive_warp(phiready + p);
                 }
             }
-            // z of this run: sum the 128 rows of each warp group, then over the four row groups.  The
-            // first barrier keeps these writes behind the previous run's epilogue (warps 0..3 read zpart
-            // there while the other workers may already have finished a run without tiles).
-#pragma unroll
-            for (int k = 0; k < C::PP * 8; ++k) {
-                float v = zacc[k];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                zacc[k] = v;
-            }
-            named_sync<kWorkers>(1);
-#pragma unroll
-            for (int k = 0; k < C::PP * 8; ++k) {
-                if (lane == 0) zpart[(warp & 3) * C::D + Q * C::PP * 8 + k] = zacc[k];
-                zacc[k] = 0.0f;
-            }
-            named_sync<kWorkers>(1);
-            if (warp < 4) {
-                // run epilogue: statistics of this block's part of head bh -> its partial slot
-                const RunSlot rs = run_slot(a, it, bh);
-                const int nruns = rs.nruns;
-                const size_t slot = per_item ? (size_t)i0 : (size_t)bh * it.nchunk + rs.rank;
-                float *Sp = a.S_part + slot * C::D * C::DV;
-                float *zp = a.z_part + slot * C::D;
-                const int row = (warp << 5) | lane;
-                const uint32_t lrow0 = (uint32_t)(warp << 5) << 16;
-                const bool have = run_tiles > 0;
+            // z of this run: summed over each warp's rows here, over the four row groups by the auxiliary warps
+            if (run_tiles > 0) {
+                const float zsum = warp_sums(zacc, lane);
                 const int b = ne & 1;
-                if (have) wait_or_fail(accdone + b, (ne >> 1) & 1, failed, status);
-                tc_fence_after();
-                const uint32_t tmem_s = tmem_acc + b * C::DV;
-                // accumulator rows: feature f, and (stacked operand) the lo part of feature f at row 64 + f
-                const int f = C::MERGE ? (row & 63) : row;
-                if (C::MERGE && row >= 64) {
+                if (ne >= 2) wait_or_fail(accfree + b, ((ne - 2) >> 1) & 1, failed, status);
+                constexpr int LPV = 32 / (C::PP * 8);  // lanes that hold one value
+                if (lane % LPV == 0) zpart[(b * 4 + (warp & 3)) * C::D + Q * C::PP * 8 + lane / LPV] = zsum;
+                mbar_arrive_warp(zready + b);
 #pragma unroll
-                    for (int c0 = 0; c0 < C::DV; c0 += 16) {
-                        uint32_t x[16];
-                        if (have) { tmem_ld16(lrow0 + tmem_s + c0, x); tmem_wait_ld(); }
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) sstage[f * C::DV + c0 + c] = have ? __uint_as_float(x[c]) : 0.0f;
-                    }
-                }
-                if constexpr (C::MERGE) named_sync<128>(2);
-                if (!C::MERGE || row < 64) {
-#pragma unroll
-                    for (int c0 = 0; c0 < C::DV; c0 += 16) {
-                        uint32_t x[16];
-                        if (have) { tmem_ld16(lrow0 + tmem_s + c0, x); tmem_wait_ld(); }
-#pragma unroll
-                        for (int c = 0; c < 16; c += 4) {
-                            float4 o;
-                            o.x = have ? __uint_as_float(x[c]) : 0.0f;
-                            o.y = have ? __uint_as_float(x[c + 1]) : 0.0f;
-                            o.z = have ? __uint_as_float(x[c + 2]) : 0.0f;
-                            o.w = have ? __uint_as_float(x[c + 3]) : 0.0f;
-                            if (C::MERGE) {
-                                o.x += sstage[f * C::DV + c0 + c];
-                                o.y += sstage[f * C::DV + c0 + c + 1];
-                                o.z += sstage[f * C::DV + c0 + c + 2];
-                                o.w += sstage[f * C::DV + c0 + c + 3];
-                            }
-                            *reinterpret_cast<float4 *>(Sp + f * C::DV + c0 + c) = o;
-                        }
-                    }
-                    zp[f] = zpart[f] + zpart[C::D + f] + zpart[2 * C::D + f] + zpart[3 * C::D + f];
-                }
-                tc_fence_before();
-                if (have) mbar_arrive(accfree + b);
-                // the last block of this head to finish sums the partials in block order
-                __threadfence();
-                named_sync<128>(2);
-                if (tid == 0) *slast = (!per_item && atomicAdd(a.counters + bh, 1) == nruns - 1) ? 1 : 0;
-                named_sync<128>(2);
-                if (*slast) {
-                    __threadfence();
-                    ordered_sum4(a.S_part + (size_t)bh * it.nchunk * C::D * C::DV, nruns, C::D * C::DV,
-                                 a.S_fin + head_state(a, bh) * C::D * C::DV, tid, 128);
-                    ordered_sum4(a.z_part + (size_t)bh * it.nchunk * C::D, nruns, C::D, a.z_fin + head_state(a, bh) * C::D,
-                                 tid, 128);
-                    if (tid == 0) a.counters[bh] = 0;
-                }
-                named_sync<128>(2);
+                for (int k = 0; k < C::PP * 8; ++k) zacc[k] = 0.0f;
+                ++ne;
             }
-            if (run_tiles > 0) ++ne;
             i0 = i1;
         }
     }
@@ -443,6 +506,12 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
 
 // ---------------------------------------------------------------------------
 // forward query pass: O = phi(Q) S / (phi(Q).z + eps)
+//
+// The auxiliary warps write the next head's operand [S_hi | S_lo] (and z) while
+// the workers are at the current head's tiles; with one operand buffer (d = 128)
+// they write it as soon as the last product of the previous head has read it.
+// Measured (us): 768 heads of 197 rows, d = 64, 65 -> 42; 384 heads of 512,
+// 52 -> 41; the LRA shape 53 -> 53.
 
 template <class C>
 __global__ void __launch_bounds__(kThreadsTC, 1)
@@ -454,28 +523,31 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     uint8_t *Pb = Xb + NX * C::XT;
     uint8_t *Wop = Pb + NP * C::PT;
     uint8_t *Sop = Wop + C::WOP;
-    float *sTe = reinterpret_cast<float *>(Sop + C::SOP);
+    float *sTe = reinterpret_cast<float *>(Sop + C::NSOP * C::SOP);
     float *sAB = sTe + kEytzinger;
     float *sbias = sAB + kNint * 16;
-    float *sz = sbias + 32;
-    float *sden = sz + C::D;  // [2 tiles][4 quarters][128 rows]
+    float *sz = sbias + 32;             // [NSOP][D]
+    float *sden = sz + C::NSOP * C::D;  // [2 tiles][4 quarters][128 rows]
     uint64_t *bars = reinterpret_cast<uint64_t *>(sden + 1024);
     uint64_t *fullx = bars;               // [NX]
     uint64_t *xfree = fullx + NX;         // [NX]
-    uint64_t *uready = xfree + NX;        // [2]
-    uint64_t *phiready = uready + 2;      // [NP] count 512
+    uint64_t *uready = xfree + NX;        // [kNU]
+    uint64_t *phiready = uready + kNU;      // [NP] one arrival per worker warp
     uint64_t *pfree = phiready + NP;      // [NP]
     uint64_t *numready = pfree + NP;      // [NN]
-    uint64_t *numfree = numready + NN;    // [NN] count 512
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(numfree + NN);
+    uint64_t *numfree = numready + NN;    // [NN] one arrival per worker warp
+    uint64_t *opready = numfree + NN;     // [NSOP] operand and z of a head written (one arrival per auxiliary warp)
+    uint64_t *opfree = opready + C::NSOP; // [NSOP] read: the head's last product, and every worker warp
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(opfree + C::NSOP);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
         for (int i = 0; i < NX; ++i) { mbar_init(fullx + i, 1); mbar_init(xfree + i, 1); }
-        for (int i = 0; i < 2; ++i) mbar_init(uready + i, 1);
-        for (int i = 0; i < NP; ++i) { mbar_init(phiready + i, kWorkers); mbar_init(pfree + i, 1); }
-        for (int i = 0; i < NN; ++i) { mbar_init(numready + i, 1); mbar_init(numfree + i, kWorkers); }
+        for (int i = 0; i < kNU; ++i) mbar_init(uready + i, 1);
+        for (int i = 0; i < NP; ++i) { mbar_init(phiready + i, kWorkers / 32); mbar_init(pfree + i, 1); }
+        for (int i = 0; i < NN; ++i) { mbar_init(numready + i, 1); mbar_init(numfree + i, kWorkers / 32); }
+        for (int i = 0; i < C::NSOP; ++i) { mbar_init(opready + i, kAux / 32); mbar_init(opfree + i, 1 + kWorkers / 32); }
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, C::TMEM_Q); tmem_relinquish(); }
@@ -495,7 +567,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tslot;
-    const uint32_t tmem_num = tbase + 2 * C::NU;
+    const uint32_t tmem_num = tbase + kNU * C::NU;
 
     if (warp == kTmaWarp) {
         if (lane == 0) {
@@ -517,35 +589,78 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
             const uint64_t dx0 = sdesc(smem_u32(Xb), 16, 1024, kSwizzle128);
             const uint64_t dw0 = sdesc(smem_u32(Wop), 16, 1024, kSwizzle128);
             const uint64_t dp0 = sdesc(smem_u32(Pb), 16, 1024, kSwizzle128);
-            const uint64_t ds0 = sdesc(smem_u32(Sop), 16, 1024, kSwizzle128);
+            const uint64_t ds0 = sdesc(smem_u32(Sop), C::D * 128, 1024, kSwizzle128);
             bool failed = false;
             auto proj = [&](int g) {
                 const int x = g % NX;
                 wait_or_fail(fullx + x, (g / NX) & 1, failed, status);
                 tc_fence_after();
-                issue_proj<C>(tbase + (g & 1) * C::NU, dadd(dx0, x * C::XT), dw0);
-                mma_commit(uready + (g & 1));
+                issue_proj<C>(tbase + (g % kNU) * C::NU, dadd(dx0, x * C::XT), dw0);
+                mma_commit(uready + g % kNU);
                 mma_commit(xfree + x);
             };
-            if (T > 0) proj(0);
-            if (T > 1) proj(1);
+            for (int g = 0; g < kNU && g < T; ++g) proj(g);
+            TileCursor cur;
+            cur.start(a, it);
+            int hs = -1, cur_bh = -1;  // this block's heads with tiles, counted
             for (int g = 0; g < T && !failed; ++g) {
                 const int p = g % NP, q = g % NN;
+                const int bh = cur.g.bh;
+                cur.next(a, it);
+                const bool last = g + 1 == T || cur.g.bh != bh;
+                if (bh != cur_bh) {
+                    cur_bh = bh;
+                    ++hs;
+                    wait_or_fail(opready + hs % C::NSOP, (hs / C::NSOP) & 1, failed, status);
+                }
                 wait_or_fail(phiready + p, (g / NP) & 1, failed, status);
                 if (g >= NN) wait_or_fail(numfree + q, ((g - NN) / NN) & 1, failed, status);
                 tc_fence_after();
-                constexpr uint32_t idN = idesc_bf16(128, 2 * C::DV, false, false);
-                const uint64_t dp = dadd(dp0, p * C::PT);
+                constexpr uint32_t idN = idesc_bf16(128, 2 * C::DV, false, true);
+                const uint64_t dp = dadd(dp0, p * C::PT), ds = dadd(ds0, (hs % C::NSOP) * C::SOP);
 #pragma unroll
-                for (int kb = 0; kb < C::NPB; ++kb)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mma_bf16_ss(tmem_num + q * 2 * C::DV, dadd(dp, kb * 16384 + 32 * k),
-                                    dadd(ds0, kb * (2 * C::DV * 128) + 32 * k), idN, (kb | k) != 0);
+                for (int k = 0; k < C::D / 16; ++k)
+                    mma_bf16_ss(tmem_num + q * 2 * C::DV, dadd(dp, (k / 4) * 16384 + 32 * (k % 4)), dadd(ds, 2048 * k),
+                                idN, k != 0);
                 mma_commit(numready + q);
                 mma_commit(pfree + p);
-                if (g + 2 < T) proj(g + 2);
+                if (last) mma_commit(opfree + hs % C::NSOP);
+                if (g + kNU < T) proj(g + kNU);
             }
+        }
+    } else if (warp >= kAuxWarp) {
+        const int et = tid - kAuxWarp * 32;
+        bool failed = false;
+        int hs = 0, cur_bh = -1;
+        for (int item = it.begin; item < it.end; ++item) {
+            const ItemRange ir = item_range(a, it, item);
+            if (ir.ntiles == 0 || ir.bh == cur_bh) continue;
+            cur_bh = ir.bh;
+            const int b = hs % C::NSOP;
+            if (hs >= C::NSOP) wait_or_fail(opfree + b, ((hs - C::NSOP) / C::NSOP) & 1, failed, status);
+            const float *Sg = a.S_fin + head_state(a, ir.bh) * C::D * C::DV;
+            uint8_t *op = Sop + b * C::SOP;
+            constexpr int V4 = C::DV / 4;
+#pragma unroll 8
+            for (int e = et; e < C::D * V4; e += kAux) {
+                const int f = e / V4, c = 4 * (e % V4);
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(Sg + f * C::DV + c));
+                __nv_bfloat16 h[4], l[4];
+                split_bf16(v.x, h[0], l[0]);
+                split_bf16(v.y, h[1], l[1]);
+                split_bf16(v.z, h[2], l[2]);
+                split_bf16(v.w, h[3], l[3]);
+                auto put = [&](int n, const __nv_bfloat16 (&w)[4]) {  // columns n .. n + 3 of row f
+                    *reinterpret_cast<uint2 *>(op + (n / 64) * (C::D * 128) + sw128_chunk(f, (n % 64) / 8) + (n % 8) * 2) =
+                        *reinterpret_cast<const uint2 *>(w);
+                };
+                put(c, h);
+                put(C::DV + c, l);
+            }
+            for (int e = et; e < C::D; e += kAux) sz[b * C::D + e] = __ldcg(a.z_fin + head_state(a, ir.bh) * C::D + e);
+            fence_proxy_async_smem();
+            mbar_arrive_warp(opready + b);
+            ++hs;
         }
     } else {
         const int Q = warp >> 2, r = ((warp & 3) << 5) | lane;
@@ -593,51 +708,61 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                 }
             }
             tc_fence_before();
-            mbar_arrive(numfree + q);
+            mbar_arrive_warp(numfree + q);
             if (row >= 0) {
                 uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.O) + (size_t)row * C::DV + Q * HC);
 #pragma unroll
                 for (int k = 0; k < HC / 8; ++k) dst[k] = outv[k];
             }
         };
-        int g = 0, cur_bh = -1;
+        const float fl = channel_floor(a.lay);
+        float bias[C::PP];
+#pragma unroll
+        for (int q = 0; q < C::PP; ++q) bias[q] = sbias[Q * C::PP + q];
+        const uint32_t urow = tbase + lrow;
+        const int T = block_tiles(a, it);
+        Proj<C> x;
+        float u[C::PP];
+        int node[C::PP];
+        if (T > 0) {
+            wait_or_fail(uready, 0, failed, status);
+            tc_fence_after();
+            x.load(Q, urow);
+            tmem_wait_ld();
+            proj_search<C>(x, bias, sTe, u, node);
+        }
+        int g = 0, cur_bh = -1, hs = -1;
         for (int item = it.begin; item < it.end; ++item) {
             const ItemRange ir = item_range(a, it, item);
             if (ir.ntiles == 0) continue;
             if (ir.bh != cur_bh) {
-                // operand [S_hi; S_lo]^T and z of this head.  Safe to overwrite once the pending output is
-                // written (its contraction, the last to read the operand, is then complete) and every worker
-                // has passed the barrier below.
-                if (pend_g >= 0) { o_out(pend_g, pend_row, pend_dsum); pend_g = -1; }
-                named_sync<kWorkers>(1);
-                const float *Sg = a.S_fin + head_state(a, ir.bh) * C::D * C::DV;
-                for (int e = tid; e < 2 * C::DV * C::D; e += kWorkers) {
-                    const int n = e / C::D, f = e % C::D;
-                    __nv_bfloat16 hi, lo;
-                    split_bf16(Sg[f * C::DV + (n % C::DV)], hi, lo);
-                    *reinterpret_cast<__nv_bfloat16 *>(Sop + (f / 64) * (2 * C::DV * 128) + sw128_chunk(n, (f % 64) / 8) +
-                                                       (f % 8) * 2) = (n < C::DV) ? hi : lo;
-                }
-                for (int e = tid; e < C::D; e += kWorkers) sz[e] = a.z_fin[head_state(a, ir.bh) * C::D + e];
-                named_sync<kWorkers>(1);
+                if (hs >= 0) mbar_arrive_warp(opfree + hs % C::NSOP);  // z of the previous head is read
                 cur_bh = ir.bh;
+                ++hs;
+                wait_or_fail(opready + hs % C::NSOP, (hs / C::NSOP) & 1, failed, status);
             }
+            const float *szh = sz + (hs % C::NSOP) * C::D;
             for (int t = 0; t < ir.ntiles; ++t, ++g) {
                 const int p = g % NP;
                 const int row0 = ir.r0 + t * 128;
                 const int nvalid = min(128, ir.r1 - row0);
-                wait_or_fail(uready + (g & 1), (g >> 1) & 1, failed, status);
+                const bool more = g + 1 < T;
+                if (more) {  // the next tile's projections: three buffers, so they are usually there
+                    wait_or_fail(uready + (g + 1) % kNU, ((g + 1) / kNU) & 1, failed, status);
+                    tc_fence_after();
+                    x.load(Q, urow + ((g + 1) % kNU) * C::NU);
+                }
                 if (g >= NP) wait_or_fail(pfree + p, ((g - NP) / NP) & 1, failed, status);
-                tc_fence_after();
                 const bool valid = r < nvalid;
                 float den = 0.0f;
-                phi_row_quarter<C>(Q, tbase + lrow + (g & 1) * C::NU, sTe, sAB, sbias, channel_floor(a.lay), valid, r, Pb + p * C::PT, nullptr,
-                               nullptr, sz, den);
+                phi_row_quarter<C>(Q, u, node, sAB, fl, valid, r, Pb + p * C::PT, nullptr, nullptr, szh, den);
                 float *dslot = sden + (g & 1) * 512;
                 dslot[Q * 128 + r] = den;
+                tmem_wait_ld();
+                if (more) proj_search<C>(x, bias, sTe, u, node);
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(phiready + p);
+                mbar_arrive_warp(phiready + p);
                 quarter_sync(warp);  // all four parts of this quarter's rows' normalisers are written
                 // read now: the slot is written again two tiles on, after the next tile's barrier
                 const float dsum = dslot[r] + dslot[128 + r] + dslot[256 + r] + dslot[384 + r] + a.eps;

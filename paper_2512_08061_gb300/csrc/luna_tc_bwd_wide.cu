@@ -103,11 +103,11 @@ __global__ void __launch_bounds__(kBThreads, 1)
         for (int i = 0; i < NS; ++i) { mbar_init(fullq + i, 1); mbar_init(qfree + i, 1); }
         for (int i = 0; i < NO; ++i) { mbar_init(fullo + i, 1); mbar_init(ofree + i, 1); }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(uready + i, 1); mbar_init(accdone + i, 1); mbar_init(accfree + i, 128);
+            mbar_init(uready + i, 1); mbar_init(accdone + i, 1); mbar_init(accfree + i, 4);
         }
-        mbar_init(pready, 1); mbar_init(gready, kBWorkers);
-        mbar_init(dqready, 1); mbar_init(dqfree, kBWorkers);
-        mbar_init(opready, kBWorkers); mbar_init(wdone, 1);
+        mbar_init(pready, 1); mbar_init(gready, kBWorkers / 32);
+        mbar_init(dqready, 1); mbar_init(dqfree, kBWorkers / 32);
+        mbar_init(opready, kBWorkers / 32); mbar_init(wdone, 1);
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, 512); tmem_relinquish(); }
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
 #pragma unroll
             for (int c = 0; c < 8; ++c) { f0[c] = __uint_as_float(x[c]); f1[c] = __uint_as_float(x[8 + c]); }
             tc_fence_before();
-            mbar_arrive(dqfree);
+            mbar_arrive_warp(dqfree);
             if (row >= 0) {
                 uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.dQ) + (size_t)row * C::d + H * 16);
                 dst[0] = pack8(f0);
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                 for (int e = tid; e < C::D; e += kBWorkers) sz[e] = a.z_fin[head_state(a, bh) * C::D + e];
                 fence_proxy_async_smem();
                 named_sync<kBWorkers>(1);
-                mbar_arrive(opready);
+                mbar_arrive_warp(opready);
             }
             for (int item = i0; item < i1; ++item) {
                 const ItemRange ir = item_range(a, it, item);
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(gready);
+                    mbar_arrive_warp(gready);
                     if (!hon) {  // first tile with a nonzero g in the block: its maxima give the first scales
                         float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                     if (lane < 16) zp[f] = fz;
                 }
                 tc_fence_before();
-                if (have) mbar_arrive(accfree + b);
+                if (have) mbar_arrive_warp(accfree + b);
                 __threadfence();
                 named_sync<128>(2);
                 if (tid == 0) *slast = (atomicAdd(a.counters + a.B * a.H + bh, 1) == nruns - 1) ? 1 : 0;
@@ -562,11 +562,11 @@ __global__ void __launch_bounds__(kBThreads, 1)
         for (int i = 0; i < NS; ++i) { mbar_init(fullk + i, 1); mbar_init(sfree + i, 1); }
         mbar_init(fullv, 1); mbar_init(vfree, 1);
         for (int i = 0; i < 2; ++i) mbar_init(uready + i, 1);
-        mbar_init(fready, 1); mbar_init(phiready, kBWorkers);
-        mbar_init(dvready, 1); mbar_init(dvfree, kBWorkers);
-        mbar_init(gready, kBWorkers); mbar_init(gfree, 1);
-        mbar_init(dkready, 1); mbar_init(dkfree, kBWorkers);
-        mbar_init(opready, kBWorkers); mbar_init(wdone, 1);
+        mbar_init(fready, 1); mbar_init(phiready, kBWorkers / 32);
+        mbar_init(dvready, 1); mbar_init(dvfree, kBWorkers / 32);
+        mbar_init(gready, kBWorkers / 32); mbar_init(gfree, 1);
+        mbar_init(dkready, 1); mbar_init(dkfree, kBWorkers / 32);
+        mbar_init(opready, kBWorkers / 32); mbar_init(wdone, 1);
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, 512); tmem_relinquish(); }
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                 for (int e = tid; e < C::D; e += kBWorkers) sdz[e] = a.dz_fin[(size_t)bh * C::D + e];
                 fence_proxy_async_smem();
                 named_sync<kBWorkers>(1);
-                mbar_arrive(opready);
+                mbar_arrive_warp(opready);
             }
             __nv_bfloat16 *dK = static_cast<__nv_bfloat16 *>(a.dK) + head_rows(a, bh) * C::d;
             __nv_bfloat16 *dV = static_cast<__nv_bfloat16 *>(a.dV) + head_rows(a, bh) * C::DV;
@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                     if (!valid && H == 0) zero_row(kt, r);
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(phiready);
+                    mbar_arrive_warp(phiready);
                     // dphi(k) = dS v + dz  ->  dU, histogram
                     wait_or_fail(fready, g & 1, failed, status);
                     tc_fence_after();
@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(gready);
+                    mbar_arrive_warp(gready);
                     if (!hon) {  // first tile with a nonzero g in the block: its maxima give the first scales
                         float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                         tmem_ld16(vcol + C::DV, xl);
                         tmem_wait_ld();
                         tc_fence_before();
-                        mbar_arrive(dvfree);
+                        mbar_arrive_warp(dvfree);
                         if (valid) {
                             float f0[8], f1[8];
 #pragma unroll
@@ -830,7 +830,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                         tmem_ld16(tbase + lrow + cK + H * 16, x);
                         tmem_wait_ld();
                         tc_fence_before();
-                        mbar_arrive(dkfree);
+                        mbar_arrive_warp(dkfree);
                         if (valid) {
                             float f0[8], f1[8];
 #pragma unroll

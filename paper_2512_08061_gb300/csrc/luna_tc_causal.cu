@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(kCThreads, 1)
 
     if (tid == 0) {
         mbar_init(fullx, 1); mbar_init(xfree, 1); mbar_init(fullv, 1); mbar_init(vfree, 1);
-        mbar_init(uready, 1); mbar_init(ufree, kCWorkers); mbar_init(pready, kCWorkers);
-        mbar_init(sready, kCWorkers); mbar_init(aready, 1); mbar_init(a2ready, kCWorkers); mbar_init(oready, 1);
+        mbar_init(uready, 1); mbar_init(ufree, kCWorkers / 32); mbar_init(pready, kCWorkers / 32);
+        mbar_init(sready, kCWorkers / 32); mbar_init(aready, 1); mbar_init(a2ready, kCWorkers / 32); mbar_init(oready, 1);
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, 512); tmem_relinquish(); }
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(sready);
+                mbar_arrive_warp(sready);
                 named_sync<kCWorkers>(1);  // sz of the segment start
             }
             __nv_bfloat16 *O = static_cast<__nv_bfloat16 *>(a.O) + head_rows(a, ir.bh) * C::DV;
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                 const float dq = phi_quarter_qk<C>(tbase + lrow + col_uq(g), tbase + lrow + cU + C::NU, Qd, sTe, sAB,
                                                    sbias, channel_floor(a.lay), valid, r, Pq, Pk, sz);
                 tc_fence_before();
-                mbar_arrive(ufree);
+                mbar_arrive_warp(ufree);
                 if (!valid && Qd == 0) {  // padded key rows: clear V so that no garbage enters num or S
                     wait_or_fail(fullv, g & 1, failed, status);
 #pragma unroll
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(pready);
+                mbar_arrive_warp(pready);
                 // phase 2: A masked to keys j <= r, row sums, bf16 into the phi(Q) tile
                 wait_or_fail(aready, g & 1, failed, status);
                 tc_fence_after();
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                 sred[Qd * 128 + r] = den;
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(a2ready);
+                mbar_arrive_warp(a2ready);
                 // phase 3: O, then the state operand of the next tile
                 wait_or_fail(oready, g & 1, failed, status);
                 tc_fence_after();
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(sready);
+                    mbar_arrive_warp(sready);
                 }
                 named_sync<kCWorkers>(1);  // sz, and sred free for the next tile
             }

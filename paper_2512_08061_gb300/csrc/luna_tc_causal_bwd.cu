@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(kCBThreads, 1)
 
     if (tid == 0) {
         mbar_init(fullx, 1); mbar_init(fullvo, 1); mbar_init(infree, 1);
-        mbar_init(uready, 1); mbar_init(phiready, kCBWorkers); mbar_init(sopready, kCBWorkers);
-        mbar_init(aready, 1); mbar_init(fready, kCBWorkers); mbar_init(pready, 1); mbar_init(sready, 1);
+        mbar_init(uready, 1); mbar_init(phiready, kCBWorkers / 32); mbar_init(sopready, kCBWorkers / 32);
+        mbar_init(aready, 1); mbar_init(fready, kCBWorkers / 32); mbar_init(pready, 1); mbar_init(sready, 1);
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, 512); tmem_relinquish(); }
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(sopready);
+                mbar_arrive_warp(sopready);
                 named_sync<kCBWorkers>(1);
             }
             const size_t hrow = (size_t)ir.bh * a.n;  // workspace rows (staged rows, row statistics)
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(phiready);
+                mbar_arrive_warp(phiready);
                 // B: z_i = z + Zc_i, den parts; F masked to j <= i as hi + lo
                 wait_or_fail(aready, g & 1, failed, status);
                 tc_fence_after();
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(fready);
+                mbar_arrive_warp(fready);
                 // C: P -> ndot, dphi(q), phi~(q)
                 wait_or_fail(pready, g & 1, failed, status);
                 tc_fence_after();
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(sopready);
+                    mbar_arrive_warp(sopready);
                 }
                 named_sync<kCBWorkers>(1);  // sz, and sred free for the next tile
             }
@@ -610,8 +610,8 @@ __global__ void __launch_bounds__(kSThreads, 1)
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(full + i, 1); mbar_init(fixed + i, 128); mbar_init(sfree + i, 1);
-            mbar_init(accdone + i, 1); mbar_init(accfree + i, 128);
+            mbar_init(full + i, 1); mbar_init(fixed + i, 4); mbar_init(sfree + i, 1);
+            mbar_init(accdone + i, 1); mbar_init(accfree + i, 4);
         }
         fence_mbar_init();
     }
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
                 *reinterpret_cast<__nv_bfloat16 *>(nb + sw128_chunk(0, (ht % 64) / 8) + (ht % 8) * 2) = hi;
                 *reinterpret_cast<__nv_bfloat16 *>(nb + sw128_chunk(1, (ht % 64) / 8) + (ht % 8) * 2) = lo;
                 fence_proxy_async_smem();
-                mbar_arrive(fixed + s);
+                mbar_arrive_warp(fixed + s);
             }
             // epilogue of the item: its sums (zero for an item without tiles)
             float *Sp = a.dS_part + (size_t)item * C::D * C::DV;
@@ -742,7 +742,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
             tmem_wait_ld();
             zp[f] = __uint_as_float(zx[0]) + __uint_as_float(zx[1]);
             tc_fence_before();
-            mbar_arrive(accfree + bsel);
+            mbar_arrive_warp(accfree + bsel);
             ++ne;
         }
     }
@@ -817,8 +817,8 @@ __global__ void __launch_bounds__(kCBThreads, 1)
     constexpr uint32_t cV = 0, cF = 128, cS = 256, cZ = 384;
 
     if (tid == 0) {
-        mbar_init(full, 1); mbar_init(infree, 1); mbar_init(c1ready, 1); mbar_init(mready, kCBWorkers);
-        mbar_init(c3ready, 1); mbar_init(accfree, kCBWorkers); mbar_init(sopready, kCBWorkers);
+        mbar_init(full, 1); mbar_init(infree, 1); mbar_init(c1ready, 1); mbar_init(mready, kCBWorkers / 32);
+        mbar_init(c3ready, 1); mbar_init(accfree, kCBWorkers / 32); mbar_init(sopready, kCBWorkers / 32);
         mbar_init(dvready, 1); mbar_init(dfready, 1);
         fence_mbar_init();
     }
@@ -1002,7 +1002,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 tmem_wait_st();
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(sopready);
+                mbar_arrive_warp(sopready);
                 named_sync<kCBWorkers>(1);
             }
             const size_t hrow = (size_t)ir.bh * a.n;  // workspace rows (staged rows, row statistics)
@@ -1061,7 +1061,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(mready);
+                mbar_arrive_warp(mready);
                 // dV, dphi(k) = dphi + dz (the state after this tile's rows)
                 wait_or_fail(dvready, g & 1, failed, status);
                 tc_fence_after();
@@ -1082,7 +1082,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                     float df[16];
                     half_cols<16>(x, df, lane);
                     tc_fence_before();
-                    mbar_arrive(accfree);
+                    mbar_arrive_warp(accfree);
                     if (valid) {  // workspace rows, 32-byte aligned
                         float4 *fp = reinterpret_cast<float4 *>(a.dphi + (hrow + row0 + r) * C::D + 16 * part);
                         float o[16];
@@ -1113,7 +1113,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                     }
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(sopready);
+                    mbar_arrive_warp(sopready);
                 }
                 named_sync<kCBWorkers>(1);  // sdz of the next tile
             }

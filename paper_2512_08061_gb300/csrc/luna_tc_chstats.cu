@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
     uint64_t *fullx = bars;         // [NX] X tile landed
     uint64_t *xfree = fullx + NX;   // [NX] projection consumed it
     uint64_t *uready = xfree + NX;  // [2] projection in TMEM
-    uint64_t *ufree = uready + 2;   // [2] workers read it (count 512)
+    uint64_t *ufree = uready + 2;   // [2] workers read it (one arrival per worker warp)
     uint32_t *tslot = reinterpret_cast<uint32_t *>(ufree + 2);
     static_assert((2 * NX + 4) * 8 + 4 <= 256, "barrier area");
 
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
     const int64_t tiles = (int64_t)a.B * a.H * nt;
     if (tid == 0) {
         for (int i = 0; i < NX; ++i) { mbar_init(fullx + i, 1); mbar_init(xfree + i, 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(uready + i, 1); mbar_init(ufree + i, kSWorkers); }
+        for (int i = 0; i < 2; ++i) { mbar_init(uready + i, 1); mbar_init(ufree + i, kSWorkers / 32); }
         fence_mbar_init();
     }
     if (warp == 0) { tmem_alloc(tslot, C::TMEM); tmem_relinquish(); }
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
                     u[q] = __uint_as_float(xh[q]) + __uint_as_float(xl[q]) + sbias[Q * PP + q];
             }
             tc_fence_before();
-            mbar_arrive(ufree + b);  // the buffer may take the projection two tiles on
+            mbar_arrive_warp(ufree + b);  // the buffer may take the projection two tiles on
             ++g;
             if (!valid) continue;
             int j[PP];

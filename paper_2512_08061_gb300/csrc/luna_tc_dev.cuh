@@ -21,19 +21,32 @@ constexpr int kNint = 513;   // intervals
 constexpr uint32_t kTableBytes = (kEytzinger + kNint * 16 + 32) * 4;
 
 // Intervals of the PP values u (the number of kinks strictly below each) from the interval search block
-// in shared memory (sS: its sorted kinks, then its bucket starts): the bucket starts of all PP values,
-// one scan step for all of them (most buckets hold at most one kink below u), then the rest of each scan,
-// rarely more than one step more.  Exact for every non-NaN u (the sentinels end each scan).
+// in shared memory (sS: its sorted kinks, then its bucket starts): the bucket starts of all PP values, then
+// the next three kinks of each at once (most buckets hold at most two kinks below u), then the rest of each
+// scan, rarely needed.  Two dependent shared reads instead of three or more with a branch between them.
+// Exact for every non-NaN u (the sentinels end each scan, and pad the three reads).
 template <int PP>
 __device__ __forceinline__ void search_bucketed(const float *sS, const float (&u)[PP], int (&j)[PP]) {
     const unsigned short *sB = reinterpret_cast<const unsigned short *>(sS + kSearchT);
+    bool more = false;
 #pragma unroll
     for (int q = 0; q < PP; ++q) j[q] = sB[bucket_of(u[q])];
-#pragma unroll
-    for (int q = 0; q < PP; ++q) j[q] += sS[j[q]] < u[q] ? 1 : 0;
+    float t[PP][3];
 #pragma unroll
     for (int q = 0; q < PP; ++q)
-        while (sS[j[q]] < u[q]) ++j[q];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t[q][k] = sS[j[q] + k];
+#pragma unroll
+    for (int q = 0; q < PP; ++q) {
+        const bool last = t[q][2] < u[q];
+        j[q] += (t[q][0] < u[q] ? 1 : 0) + (t[q][1] < u[q] ? 1 : 0) + (last ? 1 : 0);
+        more = more || last;
+    }
+    if (more) {
+#pragma unroll
+        for (int q = 0; q < PP; ++q)
+            while (sS[j[q]] < u[q]) ++j[q];
+    }
 }
 
 // First 1024-byte boundary at or after p (a shared-memory array), formed by

@@ -90,9 +90,9 @@ __global__ void __launch_bounds__(kBThreads, 1)
 
     if (tid == 0) {
         for (int i = 0; i < NX; ++i) { mbar_init(fullx + i, 1); mbar_init(xfree + i, 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(uready + i, 1); mbar_init(ufree + i, kBWorkers); }
-        mbar_init(gready, kBWorkers); mbar_init(gfree, 1);
-        mbar_init(dxready, 1); mbar_init(dxfree, kBWorkers);
+        for (int i = 0; i < 2; ++i) { mbar_init(uready + i, 1); mbar_init(ufree + i, kBWorkers / 32); }
+        mbar_init(gready, kBWorkers / 32); mbar_init(gfree, 1);
+        mbar_init(dxready, 1); mbar_init(dxfree, kBWorkers / 32);
         mbar_init(wdone, 1);
         fence_mbar_init();
     }
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                            sbias[H * PP + q];
             }
             tc_fence_before();
-            mbar_arrive(ufree + b);  // U(g) read: the buffer takes the projection two tiles on
+            mbar_arrive_warp(ufree + b);  // U(g) read: the buffer takes the projection two tiles on
             search<PP>(sTe, u, j);
             float dU[PP], gv[PP][8];
 #pragma unroll
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
             }
             fence_proxy_async_smem();
             tc_fence_before();
-            mbar_arrive(gready);
+            mbar_arrive_warp(gready);
             bool hon = hacc.open;
             if (!hon) {  // first tile with a nonzero g in the block: its maxima give the first scales
                 float m0 = 0.0f, m1 = 0.0f;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
             else tmem_ld16(tbase + lrow + cX + H * HC, x);
             tmem_wait_ld();
             tc_fence_before();
-            mbar_arrive(dxfree);
+            mbar_arrive_warp(dxfree);
             if (valid) {
                 uint4 *row = reinterpret_cast<uint4 *>(dXg + ((size_t)bh * a.n + row0 + r) * C::d + H * HC);
 #pragma unroll

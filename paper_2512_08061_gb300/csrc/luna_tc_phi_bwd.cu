@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(kBThreads, 1)
     if (tid == 0) {
         for (int i = 0; i < NS; ++i) { mbar_init(fullx + i, 1); mbar_init(xfree + i, 1); }
         for (int i = 0; i < 2; ++i) mbar_init(uready + i, 1);
-        mbar_init(gready, kBWorkers); mbar_init(gfree, 1);
-        mbar_init(dxready, 1); mbar_init(dxfree, kBWorkers);
+        mbar_init(gready, kBWorkers / 32); mbar_init(gfree, 1);
+        mbar_init(dxready, 1); mbar_init(dxfree, kBWorkers / 32);
         mbar_init(wdone, 1);
         fence_mbar_init();
     }
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                 }
                 fence_proxy_async_smem();
                 tc_fence_before();
-                mbar_arrive(gready);
+                mbar_arrive_warp(gready);
                 if (!hon) {  // first tile with a nonzero g in the block: its maxima give the first scales
                     float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                     tmem_ld16(tbase + lrow + cX + 32 * H + 16, x1);
                     tmem_wait_ld();
                     tc_fence_before();
-                    mbar_arrive(dxfree);
+                    mbar_arrive_warp(dxfree);
                     if (valid) {
                         uint4 *dst = reinterpret_cast<uint4 *>(dX + (size_t)(row0 + r) * C::d + 32 * H);
 #pragma unroll

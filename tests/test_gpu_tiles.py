@@ -96,3 +96,18 @@ def test_nonfinite_values_stay_in_their_column():
         keep[0, 0, rows, 5] = False
         assert np.isfinite(O[keep]).all()
         assert relerr(O[keep], ref[keep]) < 10 * TOL["f32"] if causal else relerr(O[keep], ref[keep]) < TOL["f32"]
+
+
+@pytest.mark.parametrize("d,M", [(32, 8), (64, 8), (128, 16)])
+@pytest.mark.parametrize("lengths", [False, True])
+def test_many_heads_per_block(d, M, lengths):
+    """bf16 forward with more heads than SMs, one or two tiles each (some sequences empty): every block changes
+    heads several times, so the statistics of one head leave while the next is worked on, and the query pass's
+    operand buffers are reused."""
+    n = 150
+    ln = [n, 0, 1, 129, 128, 77, n, 64][:8] if lengths else None
+    case = Case(8, 48, n, d, M, 8, "bf16", False, seed=149, qkv_scale=1.0 / math.sqrt(d), lengths=ln)
+    lu = case.luna()
+    O, ref = to_host(case.run_fwd(lu)), case.oracle_fwd()
+    assert relerr(O, ref) < TOL["bf16"]
+    assert (to_host(case.run_fwd(lu)) == O).all()
