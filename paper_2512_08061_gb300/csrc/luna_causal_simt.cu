@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
     const Rows sQ = take_rows(cv, cap, d), sK = take_rows(cv, cap, d), sV = take_rows(cv, cap, dv);
     const Rows sPq = take_rows(cv, cap, D), sPk = take_rows(cv, cap, D), sA = take_rows(cv, cap, cap);
     float *sden = cv.take(cap), *sinv = cv.take(cap);
-    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(4));  // largest |phi(k)|, |V|
+    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(8));  // [2 tiles] largest |phi(k)|, |V|
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
     const int len = head_length(a.lengths, bh / a.H, a.n);
@@ -74,22 +74,23 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
     load_phi_tile(s, lay, a.table);
     const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
     __syncthreads();
-    load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv);
+    load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv, nullptr);
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
     const bool vec = vec_store(O, dv);
-    for (int t0 = r0; t0 < r1; t0 += cap) {
+    int par = 0;
+    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 4) {
         const int nr = min(cap, r1 - t0);
+        unsigned *mx = mxs + par;
         __syncthreads();
-        if (threadIdx.x < 2) mx[threadIdx.x] = 0u;
+        if (threadIdx.x < 4) mxs[(par ^ 4) + threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
+        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + 1);
         __syncthreads();
         phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, nullptr);
         phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx);
-        tile_max(sV.p, cap * sV.ld, mx + 1);
         __syncthreads();
         scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int) { return 0.0f; }, [](int, float &, float &) {});
         __syncthreads();
@@ -111,7 +112,8 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
         if (t0 + cap >= r1) break;
         __syncthreads();
         const float zbound = (float)nr * __uint_as_float(mx[0]);
-        advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base(zbound * __uint_as_float(mx[1])), pair_base(zbound));
+        advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base(zbound * __uint_as_float(mx[1])), pair_base(zbound),
+                     nullptr);
     }
 }
 
@@ -138,7 +140,8 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
     float *sU = cv.take(cap * M);
     int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
     float *sdU = cv.take(cap * du_stride(M));
-    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(8));  // |S|, |V|, |dO|, |phi(q)|, |phi(k)|, |z|, |dnum|, |dden|
+    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(16));  // [2 tiles] largest |S|, |z|, |V|, |dO|, |phi(q)|,
+                                                               // |phi(k)|, |dnum|, |dden|
     cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
@@ -160,31 +163,29 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
         load_phi_tile(s, lay, a.table);
         const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
         __syncthreads();
-        load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv);
+        load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv, mxs);
     }
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
     const IO *dO = static_cast<const IO *>(a.dO) + head_rows(a, bh) * dv;
     const Rows none{};
-    for (int t0 = r0; t0 < r1; t0 += cap) {
+    int par = 0;
+    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 8) {
         const int nr = min(cap, r1 - t0);
+        unsigned *mx = mxs + par, *mx_next = mxs + (par ^ 8);
         __syncthreads();
-        if (threadIdx.x < 8) mx[threadIdx.x] = 0u;
+        if (threadIdx.x < 8) mx_next[threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
-        load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
+        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + 2);
+        block_max(load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap), mx + 3);
         __syncthreads();
-        phi_rows(lay, s, sQ, nr, cap, sPq, sU, sJ, mx + 3);
-        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx + 4);
-        tile_max(S.p, Dp * S.ld, mx);
-        tile_max(z, Dp, mx + 5);
-        tile_max(sV.p, cap * sV.ld, mx + 1);
-        tile_max(sdO.p, cap * sdO.ld, mx + 2);
+        phi_rows(lay, s, sQ, nr, cap, sPq, sU, sJ, mx + 4);
+        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx + 5);
         __syncthreads();
-        const float mS = __uint_as_float(mx[0]), mV = __uint_as_float(mx[1]), mdO = __uint_as_float(mx[2]);
-        const float mq = __uint_as_float(mx[3]), mk = __uint_as_float(mx[4]), mz = __uint_as_float(mx[5]);
+        const float mS = __uint_as_float(mx[0]), mz = __uint_as_float(mx[1]), mV = __uint_as_float(mx[2]);
+        const float mdO = __uint_as_float(mx[3]), mq = __uint_as_float(mx[4]), mk = __uint_as_float(mx[5]);
         // pairs too: o and den are formed from A, and a common rounding error of theirs does not cancel in dphi
         const float bA = pair_base((float)D * mq * mk);
         scores_lower<true>(sPq, sPk, nr, Dp, sA, [&](int) { return bA; }, [](int, float &, float &) {});
@@ -192,16 +193,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
         row_dots(sPq, nr, D, [&](int, int f) { return z[f]; }, sA, [](int r) { return r + 1; },
                  [&](int r, float h, float l) { rp.set_den(r, h, l, a.eps); });
         __syncthreads();
-        {
-            float m = 0.0f;
-            for (int e = threadIdx.x; e < nr * dvp; e += blockDim.x) {  // dnum in place
-                const int r = e / dvp, c = e - r * dvp;
-                const float v = rp.over_den(r, sdO[r][c]);
-                sdO[r][c] = v;
-                m = fmaxf(m, fabsf(v));
-            }
-            block_max(m, mx + 6);
-        }
+        block_max(rp.divide_rows(sdO, nr, dv), mx + 6);  // dnum in place
         __syncthreads();
         const float bnum = pair_base((float)D * mq * fmaf((float)nr * mk, mV, mS));
         prod_nn(sPq, nr, S, Dp, dv, sA, sV, [&](int) { return bnum; },
@@ -212,32 +204,25 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
         sum_unit_dots(sR, nr, dvp / 4, [&](int r, float h, float l) {
             rp.set_dden(r, h, l);
             atomicMax(mx + 7, __float_as_uint(fabsf(rp.gh[r])));
+            // starts of the row's sums: |dP[r][.]| and the terms of dphi(q_r) stay below these bounds
+            const bool live = rp.dh[r] != 0.0f;
+            const float iv = fabsf(rp.inv[r]), gd = fabsf(rp.gh[r]);
+            const float bound_p = fmaf(2.0f * (float)dv * mV * mdO, iv, gd);
+            rp.bp[r] = live ? pair_base(bound_p) : 0.0f;
+            rp.bq[r] = live ? pair_base(fmaf(2.0f * (float)dv * mS * mdO, iv, mz * gd) + (float)nr * mk * bound_p) : 0.0f;
             *reinterpret_cast<float4 *>(a.rowstat + ((size_t)bh * a.n + t0 + r) * 4) =
                 make_float4(rp.dh[r], rp.dl[r], rp.gh[r], rp.gl[r]);
         });
         __syncthreads();
-        // starts of row r's sums: |dP[r][.]| and the terms of dphi(q_r) stay below these bounds
-        auto bound_p = [&](int r) {
-            return r < nr && rp.dh[r] != 0.0f ? fmaf(2.0f * (float)dv * mV * mdO, fabsf(rp.inv[r]), fabsf(rp.gh[r])) : 0.0f;
-        };
-        auto base_p = [&](int r) { return pair_base(bound_p(r)); };
-        auto base_q = [&](int r) {
-            return r < nr && rp.dh[r] != 0.0f
-                       ? pair_base(fmaf(2.0f * (float)dv * mS * mdO, fabsf(rp.inv[r]), mz * fabsf(rp.gh[r])) +
-                                   (float)nr * mk * bound_p(r))
-                       : 0.0f;
-        };
-        scores_lower<true>(sdO, sV, nr, dvp, sA, base_p, [&](int r, float &h, float &l) {
+        scores_lower<true>(sdO, sV, nr, dvp, sA, [&](int r) { return rp.bp[r]; }, [&](int r, float &h, float &l) {
             pair_mac(h, l, rp.gh[r], 1.0f);
             l = __fadd_rn(l, rp.gl[r]);
         });
         acc.add(sPq, D, sdO, dv, rp.gh, rp.gl, nr, pair_base((float)nr * mq * __uint_as_float(mx[6])),
                 pair_base((float)nr * mq * __uint_as_float(mx[7])));
         __syncthreads();
-        prod_nt<kLower>(sdO, nr, S, D, dvp, sA, sPk, nr,
+        prod_nt<kLower>(sdO, nr, S, D, dvp, sA, sPk, nr, [&](int r) { return rp.bq[r]; },
                         [&](int r, int f, float &h, float &l) {
-                            h = base_q(r);
-                            l = 0.0f;
                             if (r < nr) {
                                 l = z[f] * rp.gl[r];
                                 pair_mac(h, l, z[f], rp.gh[r]);
@@ -245,13 +230,13 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
                         },
                         [&](int r, int f, float h, float l) {
                             if (r >= nr) return;
-                            h -= base_q(r);
                             sdPhi[r][f] = pair_value(h, l);
                             if (a.ch_T) atomicAdd(sT + f % a.L, (double)sPq[r][f] * ((double)h + (double)l));
                         });
         __syncthreads();
         if (t0 + cap < r1)
-            advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base((float)nr * mk * mV), pair_base((float)nr * mk));
+            advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base((float)nr * mk * mV), pair_base((float)nr * mk),
+                         mx_next);
         phi_backward_rows(lay, s, sQ, nr, cap, sPq, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
@@ -290,7 +275,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     float *sU = cv.take(cap * M);
     int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
     float *sdU = cv.take(cap * du_stride(M));
-    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(8));  // largest |V|, |dden|, |dnum|, |phi(q)|, |G|, |g|
+    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(16));  // [2 tiles] largest |G|, |g|, |V|, |dden|, |dnum|, |phi(q)|
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
     double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nseg + seg) % nbuf) * a.gsize;
@@ -306,7 +291,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     load_phi_tile(s, lay, a.table);
     const size_t so = (size_t)bh * a.nseg + seg;
     __syncthreads();
-    load_state(G, gz, a.seg_dS + so * D * dv, a.seg_dz + so * D, D, dv);
+    load_state(G, gz, a.seg_dS + so * D * dv, a.seg_dz + so * D, D, dv, mxs);
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
@@ -314,61 +299,54 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     const bool vec = vec_store(dV, dv);
     GradTile g;
     grad_zero(g);
-    for (int t0 = r0 + ((r1 - 1 - r0) / cap) * cap; t0 >= r0; t0 -= cap) {
+    int par = 0;
+    for (int t0 = r0 + ((r1 - 1 - r0) / cap) * cap; t0 >= r0; t0 -= cap, par ^= 8) {
         const int nr = min(cap, r1 - t0);
+        unsigned *mx = mxs + par, *mx_next = mxs + (par ^ 8);
         __syncthreads();
-        if (threadIdx.x < 8) mx[threadIdx.x] = 0u;
+        if (threadIdx.x < 8) mx_next[threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
+        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + 2);
         load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
+        float mdd = 0.0f;
         for (int r = threadIdx.x; r < cap; r += blockDim.x) {
             const float4 v = r < nr ? ld4(a.rowstat + ((size_t)bh * a.n + t0 + r) * 4) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             rp.dh[r] = v.x; rp.dl[r] = v.y; rp.inv[r] = 1.0f / v.x;
             rp.gh[r] = v.z; rp.gl[r] = v.w;
+            mdd = fabsf(v.z);
         }
+        block_max(mdd, mx + 3);
         __syncthreads();
-        for (int e = threadIdx.x; e < nr * dvp; e += blockDim.x) {  // dnum in place
-            const int r = e / dvp, c = e - r * dvp;
-            sdO[r][c] = rp.over_den(r, sdO[r][c]);
-        }
-        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, mx + 3);
+        block_max(rp.divide_rows(sdO, nr, dv), mx + 4);  // dnum in place
+        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, mx + 5);
         phi_rows(lay, s, sK, nr, cap, sPk, sU, sJ, nullptr);
-        tile_max(G.p, Dp * G.ld, mx + 4);
-        tile_max(gz, Dp, mx + 5);
-        tile_max(sV.p, cap * sV.ld, mx);
-        tile_max(rp.gh, cap, mx + 1);
         __syncthreads();
-        tile_max(sdO.p, cap * sdO.ld, mx + 2);
         scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int) { return 0.0f; }, [](int, float &, float &) {});
-        __syncthreads();
-        const float mV = __uint_as_float(mx[0]), mdd = __uint_as_float(mx[1]), mdn = __uint_as_float(mx[2]);
-        const float mq = __uint_as_float(mx[3]), mG = __uint_as_float(mx[4]), mg = __uint_as_float(mx[5]);
+        const float mG = __uint_as_float(mx[0]), mg = __uint_as_float(mx[1]), mV = __uint_as_float(mx[2]);
+        mdd = __uint_as_float(mx[3]);
+        const float mdn = __uint_as_float(mx[4]), mq = __uint_as_float(mx[5]);
         const float bound_p = fmaf((float)dv * mdn, mV, mdd), bp = pair_base(bound_p);
         const float bk = pair_base(fmaf((float)dv * mG, mV, mg) + (float)nr * mq * bound_p);
         scores_lower<true>(sdO, sV, nr, dvp, sP, [&](int) { return bp; }, [&](int r, float &h, float &l) {
             pair_mac(h, l, rp.gh[r], 1.0f);
             l = __fadd_rn(l, rp.gl[r]);
         });
+        __syncthreads();
         prod_nn_plain(sPk, nr, G, Dp, dv, sA, sdO, nr, [&](int q0, int c0, const float (&h)[2][4]) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
                 if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);
         });
-        __syncthreads();
-        prod_nt<kUpper>(sV, nr, G, D, dvp, sP, sPq, nr,
-                        [&](int, int f, float &h, float &l) {
-                            h = bk;
-                            l = 0.0f;
-                            pair_mac(h, l, gz[f], 1.0f);
-                        },
+        prod_nt<kUpper>(sV, nr, G, D, dvp, sP, sPq, nr, [&](int) { return bk; },
+                        [&](int, int f, float &h, float &l) { pair_mac(h, l, gz[f], 1.0f); },
                         [&](int r, int f, float h, float l) {
-                            if (r < nr) sdPhi[r][f] = pair_value(h - bk, l);
+                            if (r < nr) sdPhi[r][f] = pair_value(h, l);
                         });
         __syncthreads();
         if (t0 > r0)
             advance_rows(G, gz, sPq, D, sdO, dv, rp.gh, rp.gl, nr, pair_base((float)nr * mq * mdn),
-                         pair_base((float)nr * mq * mdd));
+                         pair_base((float)nr * mq * mdd), mx_next);
         phi_backward_rows(lay, s, sK, nr, cap, sPk, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dK + (size_t)t0 * d);
     }
@@ -382,7 +360,7 @@ size_t smem_out(const AttnArgs &a, int cap) {
     take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
     take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv);
     take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, cap);
-    cv.take(cap); cv.take(cap); cv.take(4);
+    cv.take(cap); cv.take(cap); cv.take(8);
     return cv.bytes();
 }
 size_t smem_bwd_query(const AttnArgs &a, int cap) {
@@ -392,7 +370,7 @@ size_t smem_bwd_query(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, cap);
     cv.take(cap * std::max(row_stride(a.d), std::max(row_stride(a.dv), row_stride(a.D))));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
-    cv.take(8); cv.take(kSlack);
+    cv.take(16); cv.take(kSlack);
     return cv.bytes();
 }
 size_t smem_bwd_key(const AttnArgs &a, int cap) {
@@ -403,7 +381,7 @@ size_t smem_bwd_key(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, cap); take_rows_host(cv, cap, cap);
     cv.take(cap * std::max(row_stride(a.d), row_stride(a.D)));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
-    cv.take(8);
+    cv.take(16);
     return cv.bytes();
 }
 

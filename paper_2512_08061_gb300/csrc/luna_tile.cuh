@@ -111,6 +111,16 @@ __device__ __forceinline__ float pair_base(float bound) {
     return __int_as_float((e + 2) << 23 | 0x400000);
 }
 
+// e / n for 0 <= e < 2^20, a shift where n is a power of two (M, and most widths / 4).
+struct Div {
+    int n, sh;
+    __device__ __forceinline__ explicit Div(int n_) {
+        n = n_;
+        sh = (n_ & (n_ - 1)) == 0 ? 31 - __clz(n_) : -1;
+    }
+    __device__ __forceinline__ int operator()(int e) const { return sh >= 0 ? e >> sh : e / n; }
+};
+
 // ---------------------------------------------------------------------------
 // Row tiles.
 
@@ -133,36 +143,51 @@ __device__ __forceinline__ bool vec_rows(const void *p, int w) {
     return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (w * sizeof(IO)) % 16 == 0;
 }
 
-__device__ __forceinline__ void put16(float *dst, const float *, const uint4 &v) {
-    st4(dst, make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w)));
+__device__ __forceinline__ float max4(const float4 &v, float m) {
+    if (v.x != v.x || v.y != v.y || v.z != v.z || v.w != v.w) return INFINITY;
+    return fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fmaxf(fabsf(v.y), fabsf(v.z))), fabsf(v.w));
 }
-__device__ __forceinline__ void put16(float *dst, const __nv_bfloat16 *, const uint4 &v) {
-    st4(dst, make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
-                         __uint_as_float(v.y & 0xffff0000u)));
-    st4(dst + 4, make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
-                             __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u)));
+__device__ __forceinline__ float put16(float *dst, const float *, const uint4 &v, float m) {
+    const float4 a = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+    st4(dst, a);
+    return max4(a, m);
+}
+__device__ __forceinline__ float put16(float *dst, const __nv_bfloat16 *, const uint4 &v, float m) {
+    const float4 a = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                                 __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+    const float4 b = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
+                                 __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
+    st4(dst, a);
+    st4(dst + 4, b);
+    return max4(b, max4(a, m));
 }
 
-// nr contiguous rows of w elements into the tile (cap rows); the pad columns and the rows from nr on are 0.
+// nr contiguous rows of w elements into the tile (cap rows); the pad columns and the rows from nr on are 0.  Returns
+// the largest |value| this thread has read (infinity with a NaN), for block_max.
 template <typename IO>
-__device__ void load_tile(const Rows &t, const IO *src, int nr, int w, int cap) {
+__device__ float load_tile(const Rows &t, const IO *src, int nr, int w, int cap) {
     constexpr int VE = 16 / sizeof(IO);
+    float m = 0.0f;
     if (vec_rows<IO>(src, w)) {
-        const int wv = w / VE;
-        for (int e = threadIdx.x; e < nr * wv; e += blockDim.x) {
-            const int r = e / wv, c = (e - r * wv) * VE;
-            put16(t[r] + c, src, *reinterpret_cast<const uint4 *>(src + (size_t)r * w + c));
+        const Div wv(w / VE);
+#pragma unroll 2
+        for (int e = threadIdx.x; e < nr * wv.n; e += blockDim.x) {
+            const int r = wv(e), c = (e - r * wv.n) * VE;
+            m = put16(t[r] + c, src, *reinterpret_cast<const uint4 *>(src + (size_t)e * VE), m);
         }
     } else {
         for (int e = threadIdx.x; e < nr * w; e += blockDim.x) {
             const int r = e / w, c = e - r * w;
-            t[r][c] = io_load(src + e);
+            const float v = io_load(src + e);
+            t[r][c] = v;
+            m = v == v ? fmaxf(m, fabsf(v)) : INFINITY;
         }
         const int wp = (w + 3) & ~3;
         if (wp != w)
             for (int e = threadIdx.x; e < nr * (wp - w); e += blockDim.x) t[e / (wp - w)][w + e % (wp - w)] = 0.0f;
     }
     for (int e = threadIdx.x; e < (cap - nr) * t.ld; e += blockDim.x) t[nr][e] = 0.0f;
+    return m;
 }
 
 // The largest of the threads' values m >= 0 into *slot, as the bits of a float (zeroed before, in an earlier phase).
@@ -170,17 +195,6 @@ __device__ __forceinline__ void block_max(float m, unsigned *slot) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(slot, __float_as_uint(m));
-}
-
-// Largest |value| of a tile (infinity with a NaN in it).
-__device__ void tile_max(const float *p, int count, unsigned *slot) {
-    float m = 0.0f;
-    for (int e = 4 * threadIdx.x; e < count; e += 4 * blockDim.x) {
-        const float4 v = ld4(p + e);
-        m = fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fmaxf(fabsf(v.y), fabsf(v.z))), fabsf(v.w));
-        if (v.x != v.x || v.y != v.y || v.z != v.z || v.w != v.w) m = INFINITY;
-    }
-    block_max(m, slot);
 }
 
 // ---------------------------------------------------------------------------
@@ -265,9 +279,10 @@ __device__ void phi_rows(const TableLayout &lay, const SmemPhi &s, const Rows &X
     }
     const float sc = phi_scale(lay);
     const unsigned short *sB = reinterpret_cast<const unsigned short *>(s.T + kSearchT);
+    const Div byM(M);
     float mx = 0.0f;
     for (int e = threadIdx.x; e < cap * M; e += blockDim.x) {
-        const int r = e / M, i = e - r * M;
+        const int r = byM(e), i = e - r * M;
         float *out = Phi[r] + i * L;
         if (i == M - 1)
             for (int f = D; f < ((D + 3) & ~3); ++f) Phi[r][f] = 0.0f;
@@ -277,6 +292,7 @@ __device__ void phi_rows(const TableLayout &lay, const SmemPhi &s, const Rows &X
         }
         const float *x = X[r], *w = s.W + i * ldw;
         float u = s.b[i];
+#pragma unroll 4
         for (int c = 0; c < dp; c += 4) {
             const float4 a = ld4(w + c), b = ld4(x + c);
             u = fmaf(a.x, b.x, u);
@@ -288,11 +304,23 @@ __device__ void phi_rows(const TableLayout &lay, const SmemPhi &s, const Rows &X
         if (!lay.act) {
             j = interval_bucketed(s.T, sB, u);
             const float *ab = s.AB + j * ab_stride(lay);
-            for (int l = 0; l < L; ++l) {
-                const float2 p = ab_pair(ab, l);
-                const float v = fmaxf(fmaf(p.x, u, p.y), fl);
-                out[l] = v;
-                mx = fmaxf(mx, fabsf(v));
+            if (L == 8) {
+                float y[8];
+#pragma unroll
+                for (int l = 0; l < 8; ++l) {
+                    const float2 p = ab_pair(ab, l);
+                    y[l] = fmaxf(fmaf(p.x, u, p.y), fl);
+                    mx = fmaxf(mx, fabsf(y[l]));
+                }
+                st4(out, make_float4(y[0], y[1], y[2], y[3]));
+                st4(out + 4, make_float4(y[4], y[5], y[6], y[7]));
+            } else {
+                for (int l = 0; l < L; ++l) {
+                    const float2 p = ab_pair(ab, l);
+                    const float v = fmaxf(fmaf(p.x, u, p.y), fl);
+                    out[l] = v;
+                    mx = fmaxf(mx, fabsf(v));
+                }
             }
         } else {
             for (int l = 0; l < L; ++l) {
@@ -349,8 +377,9 @@ template <typename Base, typename Done>
 __device__ __forceinline__ void prod_nn(const Rows &A, int rows, const Rows &B, int K, int cols, const Rows &T,
                                         const Rows &B2, Base base, Done done) {
     const int ng = (cols + 3) / 4, nu = ((rows + 1) / 2) * ng;
+    const Div by(ng);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
-        const int g = u / ng, r0 = 2 * g, c0 = 4 * (u - g * ng);
+        const int g = by(u), r0 = 2 * g, c0 = 4 * (u - g * ng);
         float h[2][4], l[2][4];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -382,8 +411,9 @@ template <typename Done>
 __device__ __forceinline__ void prod_nn_plain(const Rows &A, int rows, const Rows &B, int K, int cols, const Rows &T,
                                               const Rows &B2, int k2, Done done) {
     const int ng = (cols + 3) / 4, nu = ((rows + 1) / 2) * ng;
+    const Div by(ng);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
-        const int g = u / ng, r0 = 2 * g, c0 = 4 * (u - g * ng);
+        const int g = by(u), r0 = 2 * g, c0 = 4 * (u - g * ng);
         float h[2][4] = {};
         for (int k = 0; k < K; k += 4) unit_nn(h, ld4(A[r0] + k), ld4(A[r0 + 1] + k), B[k] + c0, B.ld);
         if (T.p)
@@ -403,22 +433,28 @@ __device__ __forceinline__ void prod_nn_plain(const Rows &A, int rows, const Row
 // out(r, f) = init(r, f) + sum_{k < K} A[r][k] B[f][k] + (second sum) for f < F: a unit is rows r0, r0 + 1 and the
 // four f of f0, f0 + F4, f0 + 2 F4, f0 + 3 F4 (F4 = ceil(F / 4)), so that consecutive lanes read consecutive rows
 // of B.  The second sum runs over the rows k of B2: of A2[r][k] B2[k][f] for k <= r (Lower), or of
-// A2[k][r] B2[k][f] for r <= k < k2 (Upper), with A2 lower triangular.  init(r, f, h, l) sets a pair's start;
-// done(r, f, h, l) is called for f < F.
+// A2[k][r] B2[k][f] for r <= k < k2 (Upper), with A2 lower triangular.  Row r's sums start at base(r);
+// init(r, f, h, l) adds to them, and done(r, f, h, l) gets them without the start, for f < F.
 enum Second { kNone, kLower, kUpper };
-template <Second MODE, typename Init, typename Done>
+template <Second MODE, typename Base, typename Init, typename Done>
 __device__ __forceinline__ void prod_nt(const Rows &A, int rows, const Rows &B, int F, int K, const Rows &A2,
-                                        const Rows &B2, int k2, Init init, Done done) {
+                                        const Rows &B2, int k2, Base base, Init init, Done done) {
     const int F4 = (F + 3) / 4, nu = ((rows + 1) / 2) * F4;
+    const Div by(F4);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
-        const int g = u / F4, r0 = 2 * g, f0 = u - g * F4;
+        const int g = by(u), r0 = 2 * g, f0 = u - g * F4;
         float h[2][4], l[2][4];
+        const float start[2] = {base(r0), base(r0 + 1)};
         int f[4];
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             f[m] = min(f0 + m * F4, F - 1);
 #pragma unroll
-            for (int i = 0; i < 2; ++i) init(r0 + i, f[m], h[i][m], l[i][m]);
+            for (int i = 0; i < 2; ++i) {
+                h[i][m] = start[i];
+                l[i][m] = 0.0f;
+                init(r0 + i, f[m], h[i][m], l[i][m]);
+            }
         }
         const float *a0 = A[r0], *a1 = A[r0 + 1];
         for (int k = 0; k < K; k += 4) {
@@ -459,7 +495,7 @@ __device__ __forceinline__ void prod_nt(const Rows &A, int rows, const Rows &B, 
         for (int m = 0; m < 4; ++m)
 #pragma unroll
             for (int i = 0; i < 2; ++i)
-                if (f0 + m * F4 < F) done(r0 + i, f[m], h[i][m], l[i][m]);
+                if (f0 + m * F4 < F) done(r0 + i, f[m], __fsub_rn(h[i][m], start[i]), l[i][m]);
     }
 }
 
@@ -470,14 +506,15 @@ template <bool PAIR, typename Base, typename Add>
 __device__ __forceinline__ void scores_lower(const Rows &A, const Rows &B, int rows, int K, const Rows &S, Base base,
                                              Add add) {
     const int F4 = (rows + 3) / 4, nu = ((rows + 1) / 2) * F4;
+    const Div by(F4);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
-        const int g = u / F4, r0 = 2 * g, f0 = u - g * F4;
-        float h[2][4], l[2][4];
+        const int g = by(u), r0 = 2 * g, f0 = u - g * F4;
+        float h[2][4], l[2][4], start[2];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const float s = PAIR ? base(r0 + i) : 0.0f;
+            start[i] = PAIR ? base(r0 + i) : 0.0f;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) { h[i][m] = s; l[i][m] = 0.0f; }
+            for (int m = 0; m < 4; ++m) { h[i][m] = start[i]; l[i][m] = 0.0f; }
         }
         const int nm = f0 <= r0 + 1 ? min(4, (r0 + 1 - f0) / F4 + 1) : 0;  // columns at or below the diagonal
         if (nm) {
@@ -512,7 +549,7 @@ __device__ __forceinline__ void scores_lower(const Rows &A, const Rows &B, int r
                 if (j <= r && r < rows) {
                     if (PAIR) {
                         add(r, h[i][m], l[i][m]);
-                        v = pair_value(h[i][m] - base(r), l[i][m]);
+                        v = pair_value(h[i][m] - start[i], l[i][m]);
                     } else {
                         v = h[i][m];
                     }
@@ -571,19 +608,24 @@ struct OuterAcc {
         const int nc = (dv + TC - 1) / TC;
         const int tf = threadIdx.x / nc, tc = threadIdx.x - tf * nc;
         if (tf * TF < D) {
-            float h[TF][TC], l[TF][TC];
 #pragma unroll
-            for (int i = 0; i < TF; ++i)
+            for (int q = 0; q < TC; q += 4) {  // four columns at a time: the tile's pairs beside all the running ones
+                float h[TF][4], l[TF][4];
 #pragma unroll
-                for (int m = 0; m < TC; ++m) { h[i][m] = base; l[i][m] = 0.0f; }
-            outer_rows<TF, TC>(h, l, A.p + tf * TF, A.ld, B.p + tc * TC, B.ld, nr);
+                for (int i = 0; i < TF; ++i)
 #pragma unroll
-            for (int i = 0; i < TF; ++i)
+                    for (int m = 0; m < 4; ++m) { h[i][m] = base; l[i][m] = 0.0f; }
+                outer_rows<TF, 4>(h, l, A.p + tf * TF, A.ld, B.p + tc * TC + q, B.ld, nr);
 #pragma unroll
-                for (int m = 0; m < TC; ++m) pair_add(H[i][m], L[i][m], __fsub_rn(h[i][m], base), l[i][m]);
+                for (int i = 0; i < TF; ++i)
+#pragma unroll
+                    for (int m = 0; m < 4; ++m)
+                        pair_add(H[i][q + m], L[i][q + m], __fsub_rn(h[i][m], base), l[i][m]);
+            }
         }
         if ((int)threadIdx.x < D) {
             float h = zbase, l = 0.0f;
+#pragma unroll 4
             for (int r = 0; r < nr; ++r) {
                 const float x = A[r][threadIdx.x];
                 pair_mac(h, l, x, w ? w[r] : 1.0f);
@@ -617,8 +659,10 @@ struct OuterAcc {
 
 // S[f][c] += sum_{r < nr} A[r][f] B[r][c] and z[f] += sum_r A[r][f] (w, wl)[r] (null: 1) in shared memory, each rounded
 // once; the tile's sums start at base and zbase as in OuterAcc.  The running state loses half an ulp per tile.
+// slots (or null): the largest |S| and |z| after it, as for block_max.
 __device__ void advance_rows(const Rows &S, float *z, const Rows &A, int D, const Rows &B, int dv, const float *w,
-                             const float *wl, int nr, float base, float zbase) {
+                             const float *wl, int nr, float base, float zbase, unsigned *slots) {
+    float mS = 0.0f, mz = 0.0f;
     const int ng = (dv + 3) / 4, nu = ((D + 1) / 2) * ng;
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
         const int g = u / ng, f0 = 2 * g, c0 = 4 * (u - g * ng);
@@ -638,18 +682,26 @@ __device__ void advance_rows(const Rows &S, float *z, const Rows &A, int D, cons
                 pair_add(H, L, __fsub_rn(h[i][m], base), l[i][m]);
                 o[m] = pair_value(H, L);
             }
-            st4(S[f0 + i] + c0, make_float4(o[0], o[1], o[2], o[3]));
+            const float4 nv = make_float4(o[0], o[1], o[2], o[3]);
+            st4(S[f0 + i] + c0, nv);
+            mS = max4(nv, mS);
         }
     }
     if ((int)threadIdx.x < D) {
         float h = zbase, l = 0.0f, H = z[threadIdx.x], L = 0.0f;
+#pragma unroll 4
         for (int r = 0; r < nr; ++r) {
             const float x = A[r][threadIdx.x];
             pair_mac(h, l, x, w ? w[r] : 1.0f);
             if (w) l = __fmaf_rn(x, wl[r], l);
         }
         pair_add(H, L, __fsub_rn(h, zbase), l);
-        z[threadIdx.x] = pair_value(H, L);
+        mz = pair_value(H, L);
+        z[threadIdx.x] = mz;
+    }
+    if (slots) {
+        block_max(mS, slots);
+        block_max(fabsf(mz), slots + 1);
     }
 }
 
@@ -693,6 +745,7 @@ __device__ __forceinline__ void pair_quot(float h, float l, float dh, float dl, 
 struct RowPairs {
     float *dh, *dl, *inv;  // den (and 1 / dh)
     float *gh, *gl;        // dden
+    float *bp, *bq;        // starts of the row's sums of dP and dphi
     __device__ __forceinline__ void set_den(int r, float h, float l, float eps) const {
         pair_mac_any(h, l, eps, 1.0f);
         const float v = pair_value(h, l);
@@ -710,20 +763,36 @@ struct RowPairs {
         gh[r] = v;
         gl[r] = fabsf(v) < INFINITY ? __fadd_rn(__fsub_rn(qh, v), ql) : 0.0f;
     }
-    // x / den, rounded once
-    __device__ __forceinline__ float over_den(int r, float x) const {
-        if (dh[r] == 0.0f) return 0.0f;
-        float qh, ql;
-        pair_quot(x, 0.0f, dh[r], dl[r], inv[r], qh, ql);
-        return pair_value(qh, ql);
+    // rows [0, nr) of dO divided by den, each element rounded once, in place; returns this thread's largest |value|
+    __device__ __forceinline__ float divide_rows(const Rows &dO, int nr, int cols) const {
+        const Div by((cols + 3) / 4);
+        float m = 0.0f;
+#pragma unroll 2
+        for (int e = threadIdx.x; e < nr * by.n; e += blockDim.x) {
+            const int r = by(e);
+            float *p = dO[r] + 4 * (e - r * by.n);
+            const float den = dh[r], lo = dl[r], iv = inv[r];
+            float4 v = ld4(p);
+            float *x = &v.x;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float qh, ql;
+                pair_quot(x[k], 0.0f, den, lo, iv, qh, ql);
+                x[k] = den != 0.0f ? pair_value(qh, ql) : 0.0f;
+            }
+            st4(p, v);
+            m = max4(v, m);
+        }
+        return m;
     }
 };
 __device__ RowPairs take_row_pairs(Carve &cv, int cap) {
     RowPairs p;
     p.dh = cv.take(cap); p.dl = cv.take(cap); p.inv = cv.take(cap); p.gh = cv.take(cap); p.gl = cv.take(cap);
+    p.bp = cv.take(cap); p.bq = cv.take(cap);
     return p;
 }
-void take_row_pairs_host(HostCarve &cv, int cap) { for (int k = 0; k < 5; ++k) cv.take(cap); }
+void take_row_pairs_host(HostCarve &cv, int cap) { for (int k = 0; k < 7; ++k) cv.take(cap); }
 
 // A unit's share of sum_c dnum_c num_c of its two rows (num: the sums of prod_nn, which started at base) as pairs at
 // P[r][2 g], P[r][2 g + 1], g the unit's column group; rows < nr.
@@ -806,24 +875,38 @@ __device__ void zero_words(float *p, int n) {
     for (int e = threadIdx.x; e < n; e += blockDim.x) p[e] = 0.0f;
 }
 
-// The fp32 state [D][dv] into rows of shared memory (zeros in the pads), z beside it.
-__device__ void load_state(const Rows &S, float *z, const float *gS, const float *gz, int D, int dv) {
+// The fp32 state [D][dv] into rows of shared memory (zeros in the pads), z beside it.  slots (or null): the largest
+// |S| and |z|, as for block_max.
+__device__ void load_state(const Rows &S, float *z, const float *gS, const float *gz, int D, int dv, unsigned *slots) {
     const int Dp = (D + 3) & ~3;
+    float mS = 0.0f, mz = 0.0f;
     if (dv % 4 == 0 && (reinterpret_cast<uintptr_t>(gS) & 15) == 0) {
-        const int q = dv / 4;
-        for (int e = threadIdx.x; e < D * q; e += blockDim.x) {
-            const int f = e / q, c = 4 * (e - f * q);
-            st4(S[f] + c, ld4(gS + f * dv + c));
+        const Div q(dv / 4);
+#pragma unroll 4
+        for (int e = threadIdx.x; e < D * q.n; e += blockDim.x) {
+            const int f = q(e), c = 4 * (e - f * q.n);
+            const float4 v = ld4(gS + 4 * e);
+            st4(S[f] + c, v);
+            mS = max4(v, mS);
         }
     } else {
         const int wp = (dv + 3) & ~3;
         for (int e = threadIdx.x; e < D * wp; e += blockDim.x) {
             const int f = e / wp, c = e - f * wp;
-            S[f][c] = c < dv ? gS[f * dv + c] : 0.0f;
+            const float v = c < dv ? gS[f * dv + c] : 0.0f;
+            S[f][c] = v;
+            mS = v == v ? fmaxf(mS, fabsf(v)) : INFINITY;
         }
     }
     for (int e = threadIdx.x; e < (Dp - D) * S.ld; e += blockDim.x) S[D][e] = 0.0f;
-    for (int f = threadIdx.x; f < D; f += blockDim.x) z[f] = gz[f];
+    for (int f = threadIdx.x; f < D; f += blockDim.x) {
+        z[f] = gz[f];
+        mz = fmaxf(mz, fabsf(gz[f]));
+    }
+    if (slots) {
+        block_max(mS, slots);
+        block_max(mz, slots + 1);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -880,13 +963,30 @@ __device__ void phi_backward_rows(const TableLayout &lay, const SmemPhi &s, cons
         __syncthreads();
     }
     // per sample (row, projection): g_l = dLoss/dphi0_l on an active output; dU = sum_l g_l dphi0_l/du
+    const Div byM(M);
     for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
-        const int r = e / M, i = e - r * M;
+        const int r = byM(e), i = e - r * M;
         const float u = sU[e];
         float uh = 0.0f, ul = 0.0f;
         float *gp = dPhi[r] + i * L;
         const float *ph = Phi[r] + i * L;
-        if (!lay.act) {
+        if (L == 8 && !lay.act && !ev) {
+            const int j = sJ[e];
+            const float *ab = s.AB + j * ab_stride(lay);
+            double *hj = hist + (size_t)j * 16;
+            const double u64 = widen(u);
+            const float4 g0 = ld4(gp), g1 = ld4(gp + 4), p0 = ld4(ph), p1 = ld4(ph + 4);
+#pragma unroll
+            for (int l = 0; l < 8; ++l) {
+                const float gl = at(l < 4 ? g0 : g1, l & 3);
+                if (at(l < 4 ? p0 : p1, l & 3) > fl && gl != 0.0f) {  // outer ReLU on (always, for signed outputs)
+                    pair_mac_any(uh, ul, gl, ab_pair(ab, l).x);
+                    const double gw = widen(gl);
+                    atomicAdd(hj + 2 * l, gw);
+                    atomicAdd(hj + 2 * l + 1, gw * u64);  // exact product
+                }
+            }
+        } else if (!lay.act) {
             const int j = sJ[e];
             const float *ab = s.AB + j * ab_stride(lay);
             double *hj = hist + (size_t)j * L * 2;
@@ -1033,9 +1133,11 @@ template <typename IO>
 __device__ void store_dx_rows(const TableLayout &lay, const SmemPhi &s, const float *sdU, int nr, IO *dX) {
     const int M = lay.M, d = lay.d, L = lay.L, ldw = row_stride(d), du_ld = du_stride(M), nc = (d + 3) / 4;
     const bool vec = (reinterpret_cast<uintptr_t>(dX) & 15) == 0 && d % 4 == 0;
+    const Div by(nc);
     for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
-        const int r = e / nc, c0 = 4 * (e - r * nc);
+        const int r = by(e), c0 = 4 * (e - r * nc);
         float acc[4] = {};
+#pragma unroll 4
         for (int i = 0; i < M; ++i) {
             const float4 w = ld4(s.W + i * ldw + c0);
             const float du = sdU[r * du_ld + i];
