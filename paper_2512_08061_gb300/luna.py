@@ -106,18 +106,20 @@ EXPORTED = ("luna_status_string", "luna_version", "luna_phi_table_size", "luna_p
 
 
 def _ptr(t):
-    """Device address of a tensor, or a raw address given as an int."""
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return ctypes.c_void_p(t)
-    return ctypes.c_void_p(t.data_ptr())
+    """Device address of a tensor, or a raw address given as an int (both convert to void * by argtypes)."""
+    return t if t is None or isinstance(t, int) else t.data_ptr()
+
+
+# The current stream's handle without building a torch Stream object for it (1.5 us a call, against 0.2).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _check(st: int, where: str) -> None:
@@ -220,10 +222,8 @@ def luna_state_final(ad, pd, state) -> tuple[int, int, int, int]:
 
 def luna_attn_decode(ad, pd, table, q, k, v, o, S, S_stride, z, z_stride, stream=None) -> None:
     """S, z: tensors (their data pointers are used) or raw device addresses."""
-    sp = _ptr(S) if isinstance(S, torch.Tensor) else ctypes.c_void_p(S)
-    zp = _ptr(z) if isinstance(z, torch.Tensor) else ctypes.c_void_p(z)
     _check(_lib.luna_attn_decode(ctypes.byref(ad), ctypes.byref(pd), _ptr(table), _ptr(q), _ptr(k), _ptr(v), _ptr(o),
-                                 sp, S_stride, zp, z_stride, _stream(stream)), "luna_attn_decode")
+                                 _ptr(S), S_stride, _ptr(z), z_stride, _stream(stream)), "luna_attn_decode")
 
 
 def luna_device_status(workspace: torch.Tensor, stream=None) -> int:
@@ -281,6 +281,11 @@ class Luna:
         self.ws = alloc_bytes(max(luna_workspace_size(self.ad, self.pd, False),
                                   luna_workspace_size(self.ad, self.pd, True)), self.device)
         self.state = alloc_bytes(luna_state_size(self.ad, self.pd), self.device)
+        self._final = None
+        if causal and self.state.data_ptr() and B and H and n:  # where the final S, z lie in any state buffer
+            S, Ss, z, zs = luna_state_final(self.ad, self.pd, self.state)
+            at = self.state.data_ptr()
+            self._final = (S - at, Ss, z - at, zs)
 
     def prepare(self, params: dict, stream=None):
         """params: W, b, w1, b1, w2, b2 device tensors (with a leading head axis for per-head parameters),
@@ -323,6 +328,11 @@ class Luna:
         (saved with save_state=True), which it advances in place.  q, k: (B, H, d); v: (B, H, dv)."""
         if o is None:
             o = torch.empty(q.shape[:-1] + (self.ad.dv,), dtype=q.dtype, device=q.device)
-        S, Ss, z, zs = luna_state_final(self.ad, self.pd, self.state)
+        if self._final is None:
+            S, Ss, z, zs = luna_state_final(self.ad, self.pd, self.state)
+        else:
+            at = self.state.data_ptr()
+            S, Ss, z, zs = self._final
+            S, z = at + S, at + z
         luna_attn_decode(self.ad, self.pd, self.table, q, k, v, o, S, Ss, z, zs, stream)
         return o
