@@ -200,7 +200,8 @@ __device__ __forceinline__ void issue_proj(uint32_t tmem_u, uint64_t dx, uint64_
 // final; otherwise they go to the run's partial slot and the last run of the
 // head to finish sums the partials in order.  Per-item mode (the state segments
 // of the streaming form, a.seg_S set): every item is its own run, its
-// statistics go to slot (head, item), and nothing is summed here.
+// statistics go to slot (head, item), and nothing is summed here; with one
+// segment per head they go straight to the state (no scan follows).
 //
 // Bound by the latency of the workers' chain (tensor-memory read, search,
 // table gather, operand store): a thread searches tile g + 1 while it evaluates
@@ -361,9 +362,19 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
             for (int item = i0; item < i1; ++item) run_tiles += item_range(a, it, item).ntiles;
             const RunSlot rs = run_slot(a, it, bh);
             const bool whole = !per_item && rs.nruns == 1;
+            const bool one_seg = per_item && a.nseg == 1;  // the segment's sums are the head's total
             const size_t slot = per_item ? (size_t)i0 : (size_t)bh * it.nchunk + rs.rank;
-            float *Sp = whole ? a.S_fin + head_state(a, bh) * C::D * C::DV : a.S_part + slot * C::D * C::DV;
-            float *zp = whole ? a.z_fin + head_state(a, bh) * C::D : a.z_part + slot * C::D;
+            float *Sp = a.S_part + slot * C::D * C::DV, *zp = a.z_part + slot * C::D;
+            if (whole) {
+                Sp = a.S_fin + head_state(a, bh) * C::D * C::DV;
+                zp = a.z_fin + head_state(a, bh) * C::D;
+            } else if (one_seg) {
+                Sp = a.seg_S + (2 * head_state(a, bh) + 1) * C::D * C::DV;
+                zp = a.seg_z + (2 * head_state(a, bh) + 1) * C::D;
+                for (int e = et; e < C::D * C::DV / 4; e += kAux)  // the prefix at its start
+                    reinterpret_cast<float4 *>(Sp - C::D * C::DV)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int e = et; e < C::D; e += kAux) (zp - C::D)[e] = 0.0f;
+            }
             const bool have = run_tiles > 0;
             const int b = ne & 1;
             if (have) {

@@ -323,6 +323,7 @@ __global__ void __launch_bounds__(kCThreads, 1)
                 named_sync<kCWorkers>(1);  // sz of the segment start
             }
             __nv_bfloat16 *O = static_cast<__nv_bfloat16 *>(a.O) + head_rows(a, ir.bh) * C::DV;
+            const bool wide = (reinterpret_cast<uintptr_t>(O) & 31) == 0;
             for (int t = 0; t < ir.ntiles; ++t, ++g) {
                 const int row0 = ir.r0 + t * 128;
                 const int nvalid = min(128, ir.r1 - row0);
@@ -371,32 +372,11 @@ __global__ void __launch_bounds__(kCThreads, 1)
                 fence_proxy_async_smem();
                 tc_fence_before();
                 mbar_arrive_warp(a2ready);
-                // phase 3: O, then the state operand of the next tile
+                // phase 3: the state operand of the next tile (its first products wait for it), then O
                 wait_or_fail(oready, g & 1, failed, status);
                 tc_fence_after();
                 named_sync<kCWorkers>(1);  // normaliser parts
                 const float dsum = ((sred[r] + sred[128 + r]) + (sred[256 + r] + sred[384 + r])) + a.eps;
-                {
-                    uint32_t x0[16], x1[16];
-                    tmem_ld16(tbase + lrow + cN + 32 * Qd, x0);
-                    tmem_ld16(tbase + lrow + cN + 32 * Qd + 16, x1);
-                    tmem_wait_ld();
-                    if (valid) {
-                        const float inv = dsum != 0.0f ? 1.0f / dsum : 0.0f;  // one division per row
-                        float o[32];
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            o[c] = __uint_as_float(x0[c]) * inv;
-                            o[16 + c] = __uint_as_float(x1[c]) * inv;
-                        }
-                        uint4 *dst = reinterpret_cast<uint4 *>(O + (size_t)(row0 + r) * C::DV + 32 * Qd);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            dst[k] = make_uint4(pack_bf16x2(o[8 * k], o[8 * k + 1]), pack_bf16x2(o[8 * k + 2], o[8 * k + 3]),
-                                                pack_bf16x2(o[8 * k + 4], o[8 * k + 5]),
-                                                pack_bf16x2(o[8 * k + 6], o[8 * k + 7]));
-                    }
-                }
                 if (!last) {
                     // S after this tile -> bf16 operand; z -> sz
                     const int f = r, c0 = 32 * Qd;
@@ -417,6 +397,35 @@ __global__ void __launch_bounds__(kCThreads, 1)
                     fence_proxy_async_smem();
                     tc_fence_before();
                     mbar_arrive_warp(sready);
+                }
+                {
+                    uint32_t x0[16], x1[16];
+                    tmem_ld16(tbase + lrow + cN + 32 * Qd, x0);
+                    tmem_ld16(tbase + lrow + cN + 32 * Qd + 16, x1);
+                    tmem_wait_ld();
+                    if (valid) {
+                        const float inv = dsum != 0.0f ? 1.0f / dsum : 0.0f;  // one division per row
+                        float o[32];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            o[c] = __uint_as_float(x0[c]) * inv;
+                            o[16 + c] = __uint_as_float(x1[c]) * inv;
+                        }
+                        uint4 *dst = reinterpret_cast<uint4 *>(O + (size_t)(row0 + r) * C::DV + 32 * Qd);
+                        uint4 w[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            w[k] = make_uint4(pack_bf16x2(o[8 * k], o[8 * k + 1]), pack_bf16x2(o[8 * k + 2], o[8 * k + 3]),
+                                              pack_bf16x2(o[8 * k + 4], o[8 * k + 5]),
+                                              pack_bf16x2(o[8 * k + 6], o[8 * k + 7]));
+                        if (wide) {  // whole sectors
+                            st_v8(dst, w[0], w[1]);
+                            st_v8(dst + 2, w[2], w[3]);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) dst[k] = w[k];
+                        }
+                    }
                 }
                 named_sync<kCWorkers>(1);  // sz, and sred free for the next tile
             }
@@ -475,6 +484,7 @@ cudaError_t launch_tc_causal_stats(const AttnArgs &a0, cudaStream_t s) {
     a.nsplit = a0.nseg;
     cudaError_t e = launch_tc_keys_items(a, s);
     if (e != cudaSuccess) return e;
+    if (a.nseg == 1) return cudaSuccess;  // the key pass wrote the state itself
     const size_t SD4 = (size_t)a.D * a.dv / 4;
     LUNA_LAUNCH_DEP("seg_scan", !a.ch_sigma, k_seg_scan, dim3((unsigned)((SD4 + 255) / 256), a.B * a.H), 256, 0, s, a);
     return cudaGetLastError();

@@ -106,31 +106,56 @@ __device__ __forceinline__ int ab_slot(int j, int k) { return (j << 2) | (k ^ ((
 // projection operand (NU rows x DX, K-major SW128): W split into bf16 terms
 // W_hi + W_mid (NU = 2M, about 16 significant bits) or W_hi + W_mid + W_lo and
 // M zero rows (NU = 4M, about 24 bits, as fp32).
+// Every global load is issued before the first shared store, so that a block waits for one
+// round trip to L2 and not for four.
 template <class C>
 __device__ void stage_phi_table(const AttnArgs &a, float *sTe, float *sAB, float *sbias, uint8_t *Wop) {
     const int tid = threadIdx.x, nthreads = blockDim.x;
     const TableLayout &lay = a.lay;
     const float4 *Te4 = reinterpret_cast<const float4 *>(a.table + lay.off_Te);
-    for (int e = tid; e < kEytzinger / 4; e += nthreads) reinterpret_cast<float4 *>(sTe)[e] = Te4[e];
     const float4 *AB4 = reinterpret_cast<const float4 *>(a.table + lay.off_AB);
-#pragma unroll 4
-    for (int e = tid; e < lay.nint * 4; e += nthreads) {
-        const int j = e >> 2, k = e & 3;
-        reinterpret_cast<float4 *>(sAB)[ab_slot(j, k)] = AB4[e];
-    }
     const float *b = reinterpret_cast<const float *>(a.table + lay.off_b);
-    for (int e = tid; e < C::MP; e += nthreads) sbias[e] = b[e];
     const float *W = reinterpret_cast<const float *>(a.table + lay.off_W);
-    for (int e = tid; e < C::NU * C::DX; e += nthreads) {
-        const int n = e / C::DX, c = e % C::DX;
-        const int i = n % C::MP, part = n / C::MP;  // rows: W_hi, W_mid[, W_lo, 0]
-        const float w = (c < a.d) ? W[i * a.d + c] : 0.0f;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-        const float r1 = w - __bfloat162float(hi);
-        const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-        *reinterpret_cast<__nv_bfloat16 *>(Wop + (c / 64) * (C::NU * 128) + sw128_chunk(n, (c % 64) / 8) + (c % 8) * 2) =
-            part == 0 ? hi : part == 1 ? mid : part == 2 ? lo : __float2bfloat16_rn(0.0f);
+    constexpr int kAb = 5;             // interval-table loads in flight: all of them with 512 threads or more
+    constexpr int W4 = C::DX / 4;      // four columns of one projection per thread
+    const int nab = lay.nint * 4;
+    float4 ab[kAb], te = make_float4(0.f, 0.f, 0.f, 0.f), w = te;
+    float bias = 0.0f;
+    const int wi = tid / W4, wc = 4 * (tid % W4);
+    if (tid < kEytzinger / 4) te = Te4[tid];
+    if (tid < C::MP) bias = b[tid];
+    if (wi < C::MP && wc < a.d) w = *reinterpret_cast<const float4 *>(W + wi * a.d + wc);
+#pragma unroll
+    for (int k = 0; k < kAb; ++k)
+        if (tid + k * nthreads < nab) ab[k] = AB4[tid + k * nthreads];
+    auto put_ab = [&](int e, const float4 &v) { reinterpret_cast<float4 *>(sAB)[ab_slot(e >> 2, e & 3)] = v; };
+    auto put_w = [&](int i, int c, const float4 &v) {  // rows: W_hi, W_mid[, W_lo, 0]
+        const float x[4] = {v.x, v.y, v.z, v.w};
+        __nv_bfloat16 part[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            part[0][k] = __float2bfloat16_rn(x[k]);
+            const float r1 = x[k] - __bfloat162float(part[0][k]);
+            part[1][k] = __float2bfloat16_rn(r1);
+            part[2][k] = __float2bfloat16_rn(r1 - __bfloat162float(part[1][k]));
+            part[3][k] = __float2bfloat16_rn(0.0f);
+        }
+#pragma unroll
+        for (int q = 0; q < C::NU / C::MP; ++q)
+            *reinterpret_cast<uint2 *>(Wop + (c / 64) * (C::NU * 128) + sw128_chunk(q * C::MP + i, (c % 64) / 8) +
+                                       (c % 8) * 2) = *reinterpret_cast<const uint2 *>(part[q]);
+    };
+    if (tid < kEytzinger / 4) reinterpret_cast<float4 *>(sTe)[tid] = te;
+    for (int e = tid + nthreads; e < kEytzinger / 4; e += nthreads) reinterpret_cast<float4 *>(sTe)[e] = Te4[e];
+    if (tid < C::MP) sbias[tid] = bias;
+#pragma unroll
+    for (int k = 0; k < kAb; ++k)
+        if (tid + k * nthreads < nab) put_ab(tid + k * nthreads, ab[k]);
+    for (int e = tid + kAb * nthreads; e < nab; e += nthreads) put_ab(e, AB4[e]);
+    if (wi < C::MP) put_w(wi, wc, w);
+    for (int e = tid + nthreads; e < C::MP * W4; e += nthreads) {
+        const int i = e / W4, c = 4 * (e % W4);
+        put_w(i, c, c < a.d ? *reinterpret_cast<const float4 *>(W + i * a.d + c) : make_float4(0.f, 0.f, 0.f, 0.f));
     }
 }
 
