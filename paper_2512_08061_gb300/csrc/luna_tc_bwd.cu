@@ -433,8 +433,9 @@ __global__ void __launch_bounds__(kBThreads, 1)
                 const RunSlot rs = run_slot(a, it, bh);
                 const int nruns = rs.nruns;
                 const size_t slot = (size_t)bh * it.nchunk + rs.rank;
-                float *Sp = a.dS_part + slot * C::D * C::DV;
-                float *zp = a.dz_part + slot * C::D;
+                // a head that one block holds whole needs no partials
+                float *Sp = nruns == 1 ? a.dS_fin + (size_t)bh * C::D * C::DV : a.dS_part + slot * C::D * C::DV;
+                float *zp = nruns == 1 ? a.dz_fin + (size_t)bh * C::D : a.dz_part + slot * C::D;
                 const uint32_t lr = (uint32_t)(warp << 5) << 16;
                 const bool have = run_tiles > 0;
                 const int b = ne & 1;
@@ -470,19 +471,21 @@ __global__ void __launch_bounds__(kBThreads, 1)
                 }
                 tc_fence_before();
                 if (have) mbar_arrive_warp(accfree + b);
-                __threadfence();
-                named_sync<128>(2);
-                if (tid == 0) *slast = (atomicAdd(a.counters + a.B * a.H + bh, 1) == nruns - 1) ? 1 : 0;
-                named_sync<128>(2);
-                if (*slast) {
+                if (nruns > 1) {
                     __threadfence();
-                    ordered_sum4(a.dS_part + (size_t)bh * it.nchunk * C::D * C::DV, nruns, C::D * C::DV,
-                                 a.dS_fin + (size_t)bh * C::D * C::DV, tid, 128);
-                    ordered_sum4(a.dz_part + (size_t)bh * it.nchunk * C::D, nruns, C::D, a.dz_fin + (size_t)bh * C::D,
-                                 tid, 128);
-                    if (tid == 0) a.counters[a.B * a.H + bh] = 0;
+                    named_sync<128>(2);
+                    if (tid == 0) *slast = (atomicAdd(a.counters + a.B * a.H + bh, 1) == nruns - 1) ? 1 : 0;
+                    named_sync<128>(2);
+                    if (*slast) {
+                        __threadfence();
+                        ordered_sum4(a.dS_part + (size_t)bh * it.nchunk * C::D * C::DV, nruns, C::D * C::DV,
+                                     a.dS_fin + (size_t)bh * C::D * C::DV, tid, 128);
+                        ordered_sum4(a.dz_part + (size_t)bh * it.nchunk * C::D, nruns, C::D, a.dz_fin + (size_t)bh * C::D,
+                                     tid, 128);
+                        if (tid == 0) a.counters[a.B * a.H + bh] = 0;
+                    }
+                    named_sync<128>(2);
                 }
-                named_sync<128>(2);
             }
             if (run_tiles > 0) ++ne;
             i0 = i1;

@@ -47,30 +47,43 @@ __device__ void stage_wx(const AttnArgs &a, uint8_t *dst, int ch0) {
 }
 
 // Operand rows per feature (hi rows 0..D-1, lo rows D..2D-1), K = value column:
-// the B operand of P = dO S^T and of dphi(k) = V dS^T.
+// the B operand of P = dO S^T and of dphi(k) = V dS^T.  Four columns per thread and step.
 template <class C>
 __device__ void stage_rows_per_feature(const float *Sg, uint8_t *op, int tid, int nthr) {
-    for (int e = tid; e < 2 * C::D * 64; e += nthr) {
-        const int n = e / 64, c = e % 64, f = n % C::D;
-        float v = 0.0f;
-        if (c < C::DV) {
-            __nv_bfloat16 hi, lo;
-            split_bf16(Sg[f * C::DV + c], hi, lo);
-            v = (n < C::D) ? __bfloat162float(hi) : __bfloat162float(lo);
-        }
-        *reinterpret_cast<__nv_bfloat16 *>(op + sw128_chunk(n, c / 8) + (c % 8) * 2) = __float2bfloat16_rn(v);
+    constexpr int V4 = C::DV / 4;
+    auto put = [&](int e, const float4 &x) {
+        const int f = e / V4, c = 4 * (e % V4);
+        const float v[4] = {x.x, x.y, x.z, x.w};
+        __nv_bfloat16 h[4], l[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) split_bf16(v[k], h[k], l[k]);
+        const uint32_t at = (c % 8) * 2;
+        *reinterpret_cast<uint2 *>(op + sw128_chunk(f, c / 8) + at) = *reinterpret_cast<const uint2 *>(h);
+        *reinterpret_cast<uint2 *>(op + sw128_chunk(C::D + f, c / 8) + at) = *reinterpret_cast<const uint2 *>(l);
+    };
+    for (int e = tid; e < C::D * V4; e += nthr) put(e, __ldcg(reinterpret_cast<const float4 *>(Sg) + e));
+    if constexpr (C::DV < 64) {  // the rest of the 64 columns
+        constexpr int Z = (64 - C::DV) / 8;
+        for (int e = tid; e < 2 * C::D * Z; e += nthr)
+            *reinterpret_cast<uint4 *>(op + sw128_chunk(e / Z, C::DV / 8 + e % Z)) = make_uint4(0, 0, 0, 0);
     }
 }
 
 // Operand rows per value column (hi rows 0..DV-1, lo rows DV..2DV-1), K = feature:
-// the B operand of dV = phi dS.
+// the B operand of dV = phi dS.  A thread packs four features of one column (lanes read consecutive columns).
 template <class C>
 __device__ void stage_rows_per_column(const float *Sg, uint8_t *op, int tid, int nthr) {
-    for (int e = tid; e < 2 * C::DV * C::D; e += nthr) {
-        const int n = e / C::D, f = e % C::D, c = n % C::DV;
-        __nv_bfloat16 hi, lo;
-        split_bf16(Sg[f * C::DV + c], hi, lo);
-        *reinterpret_cast<__nv_bfloat16 *>(op + sw128_chunk(n, f / 8) + (f % 8) * 2) = (n < C::DV) ? hi : lo;
+    for (int e = tid; e < C::DV * (C::D / 4); e += nthr) {
+        const int c = e % C::DV, f0 = 4 * (e / C::DV);
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldcg(Sg + (f0 + k) * C::DV + c);
+        __nv_bfloat16 h[4], l[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) split_bf16(v[k], h[k], l[k]);
+        const uint32_t at = (f0 % 8) * 2;
+        *reinterpret_cast<uint2 *>(op + sw128_chunk(c, f0 / 8) + at) = *reinterpret_cast<const uint2 *>(h);
+        *reinterpret_cast<uint2 *>(op + sw128_chunk(C::DV + c, f0 / 8) + at) = *reinterpret_cast<const uint2 *>(l);
     }
 }
 
