@@ -38,13 +38,13 @@ __device__ float down_threshold(float w, float c) {
     return t;
 }
 
-// One launch: every block computes the kink threshold of every hidden unit and
-// sorts the (threshold, unit index) pairs (a bitonic network over one element
-// per thread: warp shuffles for partners within a warp, shared memory across
-// warps; a stable total order), then computes its slice of alpha and beta,
-// eight threads per (interval, channel) entry; block 0 also writes the sorted
-// kink list and interval search block, each unit's rank and active side, and the
-// parameter copies.
+// One launch, bound by its chain of dependent steps (loads, thresholds, sort, output).  Every block but the
+// last computes the kink threshold of every hidden unit and sorts the (threshold, unit index) pairs (a
+// bitonic network over one element per thread: warp shuffles for partners within a warp, shared memory across
+// warps; a stable total order).  All but the last two then compute their slice of alpha and beta, eight
+// threads per (interval, channel) entry; the last but one writes the sorted kinks, the units' ranks and the
+// interval search block; the last copies the parameters, which needs no sort.  With those two parts in front
+// of the first slice, one block's chain was about twice as long as the others'.
 constexpr int kPrepThreads = kMaxUnits;                       // one thread per (padded) unit
 constexpr int kPrepSplit = 8;                                 // threads per (interval, channel) entry
 constexpr int kPrepEntries = kPrepThreads / kPrepSplit;       // entries per block
@@ -57,7 +57,9 @@ __device__ __forceinline__ bool pair_less(float ta, int ka, float tb, int kb) {
 // thread (warp shuffles for partners within a warp, shared memory across warps; a stable total order),
 // fully unrolled for the size.  Positions at or past 2^LOGN sort among themselves.
 template <int LOGN>
-__device__ __forceinline__ void bitonic_sort(float &key, int &idx, float *sk, int *si, int tid) {
+__device__ __forceinline__ void bitonic_sort(float &key, int &idx, float (*xk)[kMaxUnits], int (*xi)[kMaxUnits],
+                                             int tid) {
+    int b = 0;  // exchange buffer: two in turn, so that one barrier a step keeps reads and writes apart
 #pragma unroll
     for (int size = 2; size <= (1 << LOGN); size <<= 1) {
 #pragma unroll
@@ -65,10 +67,10 @@ __device__ __forceinline__ void bitonic_sort(float &key, int &idx, float *sk, in
             float pk;
             int pi;
             if (stride >= 32) {
-                sk[tid] = key; si[tid] = idx;
+                xk[b][tid] = key; xi[b][tid] = idx;
                 __syncthreads();
-                pk = sk[tid ^ stride]; pi = si[tid ^ stride];
-                __syncthreads();
+                pk = xk[b][tid ^ stride]; pi = xi[b][tid ^ stride];
+                b ^= 1;
             } else {
                 pk = __shfl_xor_sync(0xffffffffu, key, stride);
                 pi = __shfl_xor_sync(0xffffffffu, idx, stride);
@@ -87,37 +89,88 @@ __device__ __forceinline__ int unit_pos(const TableLayout &lay, int unit) {
     return lay.shared ? unit : (unit % lay.hid) * lay.L + unit / lay.hid;
 }
 
+// The side of its kink on which a unit is on: 1 above, -1 at or below (a constant unit: always off, always on,
+// with its kink at +inf).
+__device__ __forceinline__ int unit_type(float w, float c) {
+    return w > 0.0f ? 1 : w < 0.0f ? -1 : c > 0.0f ? -1 : 1;
+}
+
+// Parameter copies, the units' active sides and the header.
+__device__ __forceinline__ void copy_params(const luna_phi_params &prm, const TableLayout &lay, char *table, int tid,
+                                            int nt) {
+    auto at = [&](int64_t off) { return reinterpret_cast<float *>(table + off); };
+    const int P = lay.P, L = lay.L;
+    // one element of each array per thread first, every load before the first store
+    const int n2 = L * lay.hid, nW = lay.M * lay.d;
+    float w1 = 0.f, b1 = 0.f, w2 = 0.f, b = 0.f, b2 = 0.f, W[4] = {};
+    if (tid < P) { w1 = prm.w1[tid]; b1 = prm.b1[tid]; }
+    if (tid < n2) w2 = prm.w2[tid];
+    if (tid < lay.M) b = prm.b[tid];
+    if (tid < L) b2 = prm.b2[tid];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (tid + k * nt < nW) W[k] = prm.W[tid + k * nt];
+    if (tid < P) {  // P and n2 are at most kMaxUnits, the threads of the block
+        at(lay.off_w1)[tid] = w1;
+        at(lay.off_b1)[tid] = b1;
+        reinterpret_cast<int *>(table + lay.off_utype)[tid] = unit_type(w1, b1);
+    }
+    if (tid < n2) at(lay.off_w2)[tid] = w2;
+    if (tid < lay.M) at(lay.off_b)[tid] = b;
+    if (tid < L) at(lay.off_b2)[tid] = b2;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (tid + k * nt < nW) at(lay.off_W)[tid + k * nt] = W[k];
+    for (int e = tid + nt; e < n2; e += nt) at(lay.off_w2)[e] = prm.w2[e];
+    for (int e = tid + nt; e < lay.M; e += nt) at(lay.off_b)[e] = prm.b[e];
+    for (int e = tid + 4 * nt; e < nW; e += nt) at(lay.off_W)[e] = prm.W[e];
+    if (lay.env) {  // envelope gate
+        for (int e = tid; e < L * lay.d; e += nt) at(lay.off_We)[e] = prm.We[e];
+        for (int e = tid; e < L; e += nt) at(lay.off_be)[e] = prm.be[e];
+    }
+    if (lay.coef)  // Bank+Coef coefficients
+        for (int e = tid; e < L; e += nt) at(lay.off_coef)[e] = prm.coef[e];
+    if (tid == 0) {
+        TableHeader *h = reinterpret_cast<TableHeader *>(table);
+        h->magic = kTableMagic; h->version = kTableVersion;
+        h->M = lay.M; h->L = L; h->hid = lay.hid; h->d = lay.d; h->P = P; h->Ppad = lay.Ppad;
+    }
+}
+
 __global__ void __launch_bounds__(kPrepThreads) k_phi_prepare(luna_phi_params prm, TableLayout lay, char *table) {
-    __shared__ float sk[kMaxUnits];
-    __shared__ int si[kMaxUnits];
+    __shared__ float sk[kMaxUnits], xk[2][kMaxUnits];
+    __shared__ int si[kMaxUnits], xi[2][kMaxUnits];
     __shared__ float w1t[kMaxUnits], b1t[kMaxUnits];  // per-unit fc1 values
     __shared__ float w2t[kMaxUnits];                  // fc2 weight of (unit k, channel l) at k*L + l
     __shared__ int tyt[kMaxUnits], rkt[kMaxUnits];
     const int tid = threadIdx.x, nt = blockDim.x;
     const int P = lay.P, N = lay.Ppad, L = lay.L, hid = lay.hid;  // N: power of two >= P, <= kMaxUnits
+    const int nab = gridDim.x - 2;  // blocks of alpha and beta
+    if ((int)blockIdx.x == nab + 1) {
+        copy_params(prm, lay, table, tid, nt);
+        return;
+    }
     float key = INFINITY;  // this thread's element: unit tid, padding (+inf, index >= P) sorts last
     int idx = tid;
     if (tid < P) {
         const float w = prm.w1[tid], c = prm.b1[tid];
-        int ty;
-        if (w > 0.0f) { key = up_threshold(w, c); ty = 1; }
-        else if (w < 0.0f) { key = down_threshold(w, c); ty = -1; }
-        else { key = INFINITY; ty = (c > 0.0f) ? -1 : 1; }  // constant unit: always on / always off
+        if (w > 0.0f) key = up_threshold(w, c);
+        else if (w < 0.0f) key = down_threshold(w, c);
         const int tpos = unit_pos(lay, tid);
-        w1t[tpos] = w; b1t[tpos] = c; tyt[tpos] = ty;
+        w1t[tpos] = w; b1t[tpos] = c; tyt[tpos] = unit_type(w, c);
     }
     for (int e = tid; e < L * hid; e += nt) w2t[(e % hid) * L + e / hid] = prm.w2[e];  // w2[l][k]
     // bitonic sort of the first N elements (N a power of two, at most kMaxUnits = 512)
     switch (N) {
-        case 2: bitonic_sort<1>(key, idx, sk, si, tid); break;
-        case 4: bitonic_sort<2>(key, idx, sk, si, tid); break;
-        case 8: bitonic_sort<3>(key, idx, sk, si, tid); break;
-        case 16: bitonic_sort<4>(key, idx, sk, si, tid); break;
-        case 32: bitonic_sort<5>(key, idx, sk, si, tid); break;
-        case 64: bitonic_sort<6>(key, idx, sk, si, tid); break;
-        case 128: bitonic_sort<7>(key, idx, sk, si, tid); break;
-        case 256: bitonic_sort<8>(key, idx, sk, si, tid); break;
-        case 512: bitonic_sort<9>(key, idx, sk, si, tid); break;
+        case 2: bitonic_sort<1>(key, idx, xk, xi, tid); break;
+        case 4: bitonic_sort<2>(key, idx, xk, xi, tid); break;
+        case 8: bitonic_sort<3>(key, idx, xk, xi, tid); break;
+        case 16: bitonic_sort<4>(key, idx, xk, xi, tid); break;
+        case 32: bitonic_sort<5>(key, idx, xk, xi, tid); break;
+        case 64: bitonic_sort<6>(key, idx, xk, xi, tid); break;
+        case 128: bitonic_sort<7>(key, idx, xk, xi, tid); break;
+        case 256: bitonic_sort<8>(key, idx, xk, xi, tid); break;
+        case 512: bitonic_sort<9>(key, idx, xk, xi, tid); break;
         default: break;  // N = 1: nothing to sort
     }
     sk[tid] = key;
@@ -125,21 +178,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_phi_prepare(luna_phi_params pr
     if (idx < P) rkt[unit_pos(lay, idx)] = tid;
     __syncthreads();
 
-    if (blockIdx.x == 0) {
+    if ((int)blockIdx.x == nab) {
         float *T = reinterpret_cast<float *>(table + lay.off_T);
         int *rank = reinterpret_cast<int *>(table + lay.off_rank);
-        int *utype = reinterpret_cast<int *>(table + lay.off_utype);
         for (int r = tid; r < N; r += nt) {
             T[r] = sk[r];  // sorted kinks, +inf padding
             if (si[r] < P) rank[si[r]] = r;
         }
-        for (int k = tid; k < P; k += nt) {
-            const int tpos = unit_pos(lay, k);
-            utype[k] = tyt[tpos];
-            reinterpret_cast<float *>(table + lay.off_w1)[k] = w1t[tpos];
-            reinterpret_cast<float *>(table + lay.off_b1)[k] = b1t[tpos];
-        }
-        for (int e = tid; e < L * hid; e += nt) reinterpret_cast<float *>(table + lay.off_w2)[e] = prm.w2[e];
         // interval search block: the sorted kinks with +inf sentinels, then every bucket's start (the
         // number of kinks strictly below the bucket's smallest value, by binary search over the kinks)
         float *Ts = reinterpret_cast<float *>(table + lay.off_Te);
@@ -158,21 +203,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_phi_prepare(luna_phi_params pr
         }
         for (int e = kSearchT * 2 + kBuckets + tid; e < kEytzinger * 2; e += nt)
             reinterpret_cast<unsigned short *>(Ts)[e] = 0;  // the block's unused tail
-        float *W = reinterpret_cast<float *>(table + lay.off_W);
-        for (int e = tid; e < lay.M * lay.d; e += nt) W[e] = prm.W[e];
-        for (int e = tid; e < lay.M; e += nt) reinterpret_cast<float *>(table + lay.off_b)[e] = prm.b[e];
-        for (int e = tid; e < L; e += nt) reinterpret_cast<float *>(table + lay.off_b2)[e] = prm.b2[e];
-        if (lay.env) {  // envelope gate
-            for (int e = tid; e < L * lay.d; e += nt) reinterpret_cast<float *>(table + lay.off_We)[e] = prm.We[e];
-            for (int e = tid; e < L; e += nt) reinterpret_cast<float *>(table + lay.off_be)[e] = prm.be[e];
-        }
-        if (lay.coef)  // Bank+Coef coefficients
-            for (int e = tid; e < L; e += nt) reinterpret_cast<float *>(table + lay.off_coef)[e] = prm.coef[e];
-        if (tid == 0) {
-            TableHeader *h = reinterpret_cast<TableHeader *>(table);
-            h->magic = kTableMagic; h->version = kTableVersion;
-            h->M = lay.M; h->L = lay.L; h->hid = lay.hid; h->d = lay.d; h->P = P; h->Ppad = lay.Ppad;
-        }
+        return;
     }
     // alpha, beta of (interval j, channel l), scaled by 1/sqrt(M): thread p of the
     // entry's eight sums units k = p, p + 8, ... in order, then the eight partial
@@ -180,7 +211,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_phi_prepare(luna_phi_params pr
     float *AB = reinterpret_cast<float *>(table + lay.off_AB);
     const float scale = 1.0f / sqrtf((float)lay.M);
     const int p = tid % kPrepSplit;
-    for (int e0 = blockIdx.x * kPrepEntries; e0 < lay.nint * L; e0 += gridDim.x * kPrepEntries) {
+    for (int e0 = blockIdx.x * kPrepEntries; e0 < lay.nint * L; e0 += nab * kPrepEntries) {
         const int e = e0 + tid / kPrepSplit;
         const bool live = e < lay.nint * L;
         const int j = live ? e / L : 0, l = live ? e % L : 0;
@@ -209,7 +240,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_phi_prepare(luna_phi_params pr
 }  // namespace
 
 cudaError_t launch_phi_prepare(const luna_phi_params &prm, const TableLayout &lay, void *table, cudaStream_t s) {
-    const int blocks = (lay.nint * lay.L + kPrepEntries - 1) / kPrepEntries;
+    const int blocks = (lay.nint * lay.L + kPrepEntries - 1) / kPrepEntries + 2;  // two more: see k_phi_prepare
     LUNA_LAUNCH("phi_prepare", k_phi_prepare, blocks, kPrepThreads, 0, s, prm, lay, static_cast<char *>(table));
     return cudaGetLastError();
 }
