@@ -22,9 +22,9 @@
 //   2. k_tcc_dstats: per segment sum_i phi~(q_i) dO_i^T and sum_i phi~(q_i) ndot_i
 //   3. k_seg_rscan: exclusive suffix of those sums (dS, dz after each segment)
 //   4. k_tcc_key (reverse sweep, state dS, dz in tensor memory):
-//        MMA  C = phi(K) phi~(Q)^T,  E = V dO^T
+//        MMA  C = phi(K) phi~(Q)^T,  E = V dO^T,  dV = phi(K) [dS_hi; dS_lo]
 //        work C masked to i >= j (hi + lo); E + ndot_i masked (hi + lo)
-//        MMA  dV = phi(K) [dS_hi; dS_lo] + C dO,  dphi = V [dS_hi; dS_lo]^T + E phi~(Q)
+//        MMA  dV += C dO,  dphi = V [dS_hi; dS_lo]^T + E phi~(Q)
 //             dS += phi~(Q)^T dO,  dz += phi~(Q)^T [ndot_hi, ndot_lo]
 //        work dV, dphi(k) = dphi + dz
 //   5. chain rule for Q and for K, then the parameter-gradient reduction.
@@ -294,7 +294,6 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 const int tin = cur.t;  // tile index within the item (z restarts at 0)
                 wait_or_fail(phiready, g & 1, failed, status);
                 wait_or_fail(fullvo, g & 1, failed, status);
-                wait_or_fail(sopready, g & 1, failed, status);
                 tc_fence_after();
                 {
                     constexpr uint32_t idF = idesc_bf16(64, 64, false, false);
@@ -312,6 +311,8 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                         for (int k = 0; k < 4; ++k)
                             mma_bf16_ss(tbase + cZc, dadd(dL1, 32 * k), dadd(hl ? dPm : dKm, 2048 * k), idZc, (hl | k) != 0);
                     mma_commit(aready);  // the workers mask F while P = dO S^T runs
+                    wait_or_fail(sopready, g & 1, failed, status);  // staged while F and Zc run
+                    tc_fence_after();
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -360,8 +361,12 @@ __global__ void __launch_bounds__(kCBThreads, 1)
             const ItemRange ir = item_range(a, it, item);
             const int nt = tiles64(ir);
             if (nt == 0) continue;
-            // segment start: S (TMEM fp32 and the bf16 hi/lo operand) and z from the prefix state
+            // segment start: S (TMEM fp32 and the bf16 hi/lo operand) and z from the prefix state, once the
+            // products and the rows of the segment before are done
             {
+                if (g > 0) wait_or_fail(sready, (g - 1) & 1, failed, status);
+                tc_fence_after();
+                named_sync<kCBWorkers>(1);
                 const float *Sp = a.seg_S + (head_state(a, ir.bh) * (a.nseg + 1) + ir.chunk) * C::D * C::DV;
                 const int f = 32 * q + lane, c0 = 32 * cg;
                 float v[32];
@@ -460,6 +465,29 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 fence_proxy_async_smem();
                 tc_fence_before();
                 mbar_arrive_warp(phiready);
+                // S before this tile -> operand, z -> sz, while F and Zc run: only P needs them.  (At the end of
+                // the tile before, the tensor cores and the 2.5 k cycles of this waited for one another.)
+                if (t > 0) {
+                    wait_or_fail(sready, (g - 1) & 1, failed, status);
+                    tc_fence_after();
+                    const int f = 32 * q + lane, c0 = 32 * cg;
+                    uint32_t x[32];
+                    ld32(tbase + lq + cS + c0, x);
+                    float v[32];
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(x[c]);
+                    store_state32(Sh, Sl, f, c0, v);
+                    if (cg == 0) {
+                        uint32_t zx[2];
+                        tmem_ld2(tbase + lq + cz, zx);
+                        tmem_wait_ld();
+                        sz[f] = zpre[f] + __uint_as_float(zx[0]);
+                    }
+                    fence_proxy_async_smem();
+                    tc_fence_before();
+                    mbar_arrive_warp(sopready);
+                    named_sync<kCBWorkers>(1);  // sz, and sred free for this tile
+                }
                 // B: z_i = z + Zc_i, den parts; F masked to j <= i as hi + lo
                 wait_or_fail(aready, g & 1, failed, status);
                 tc_fence_after();
@@ -549,30 +577,10 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                                 make_float2(live ? den : 1.0f, live ? ndot : 0.0f);
                     }
                 }
-                // D: S after this tile -> operand of the next tile; z -> sz
-                wait_or_fail(sready, g & 1, failed, status);
-                tc_fence_after();
-                if (t + 1 < nt) {
-                    const int f = 32 * q + lane, c0 = 32 * cg;
-                    uint32_t x[32];
-                    ld32(tbase + lq + cS + c0, x);
-                    float v[32];
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(x[c]);
-                    store_state32(Sh, Sl, f, c0, v);
-                    if (cg == 0) {
-                        uint32_t zx[2];
-                        tmem_ld2(tbase + lq + cz, zx);
-                        tmem_wait_ld();
-                        sz[f] = zpre[f] + __uint_as_float(zx[0]);
-                    }
-                    fence_proxy_async_smem();
-                    tc_fence_before();
-                    mbar_arrive_warp(sopready);
-                }
-                named_sync<kCBWorkers>(1);  // sz, and sred free for the next tile
             }
         }
+        // the last tile's products end before tensor memory is released
+        if (g > 0) wait_or_fail(sready, (g - 1) & 1, failed, status);
         if constexpr (TSUM) {  // the block's row of T: warp sums, then fp64 adds (the launch cleared the row)
 #pragma unroll
             for (int l = 0; l < 8; ++l) {
@@ -813,8 +821,8 @@ __global__ void __launch_bounds__(kCBThreads, 1)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const Items it(a);
-    // TMEM: dV (C first) [128] | dphi (E first) [128] | dS [128] | dz [16]
-    constexpr uint32_t cV = 0, cF = 128, cS = 256, cZ = 384;
+    // TMEM: dV [128] | dphi (E first) [128] | dS [128] | dz [16] | C [64]
+    constexpr uint32_t cV = 0, cF = 128, cS = 256, cZ = 384, cC = 400;
 
     if (tid == 0) {
         mbar_init(full, 1); mbar_init(infree, 1); mbar_init(c1ready, 1); mbar_init(mready, kCBWorkers / 32);
@@ -901,19 +909,20 @@ __global__ void __launch_bounds__(kCBThreads, 1)
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             const uint32_t o = kb * T8 + 32 * k;
-                            mma_bf16_ss(tbase + cV, dadd(dPkK, o), dadd(dPqK, o), id64, (kb | k) != 0);
-                            mma_bf16_ss(tbase + cV, dadd(dPkK, o), dadd(dPqK, 2 * T8 + o), id64, 1u);
-                            mma_bf16_ss(tbase + cV, dadd(dPkK, 2 * T8 + o), dadd(dPqK, o), id64, 1u);
+                            mma_bf16_ss(tbase + cC, dadd(dPkK, o), dadd(dPqK, o), id64, (kb | k) != 0);
+                            mma_bf16_ss(tbase + cC, dadd(dPkK, o), dadd(dPqK, 2 * T8 + o), id64, 1u);
+                            mma_bf16_ss(tbase + cC, dadd(dPkK, 2 * T8 + o), dadd(dPqK, o), id64, 1u);
                             mma_bf16_ss(tbase + cF, dadd(dVk, o), dadd(dOk, o), id64, (kb | k) != 0);
                         }
                     mma_commit(c1ready);
                 }
-                wait_or_fail(mready, g & 1, failed, status);
+                // dV = phi(K) dS ([hi, hi, lo] x [hi, lo, hi]) + C dO (C hi + lo).  C has columns of its own, so
+                // that the 24 products of the state part run while the workers mask C and E: the workers'
+                // wait for dV was 2.6 k of a tile's 11.9 k cycles when they came after it.
                 wait_or_fail(sopready, g & 1, failed, status);
                 tc_fence_after();
+                constexpr uint32_t idV = idesc_bf16(64, C::DV, false, true);
                 {
-                    // dV = phi(K) dS ([hi, hi, lo] x [hi, lo, hi]) + C dO (C hi + lo)
-                    constexpr uint32_t idV = idesc_bf16(64, C::DV, false, true);
 #pragma unroll
                     for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
@@ -923,6 +932,10 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                             mma_bf16_ss(tbase + cV, dadd(dPkK, o), dadd(dSlM, so), idV, 1u);
                             mma_bf16_ss(tbase + cV, dadd(dPkK, 2 * T8 + o), dadd(dShM, so), idV, 1u);
                         }
+                }
+                wait_or_fail(mready, g & 1, failed, status);
+                tc_fence_after();
+                {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         mma_bf16_ss(tbase + cV, dadd(dCh, 32 * k), dadd(dOm, 2048 * k), idV, 1u);
@@ -1023,7 +1036,7 @@ __global__ void __launch_bounds__(kCBThreads, 1)
                 tc_fence_after();
                 {
                     uint32_t x[16];
-                    tmem_ld16(tbase + lq + cV + 16 * cg, x);
+                    tmem_ld16(tbase + lq + cC + 16 * cg, x);
                     tmem_wait_ld();
                     float cv[8];
                     half_cols<8>(x, cv, lane);
