@@ -373,7 +373,7 @@ def measure_workload(args, w, dev, world, steps, ch_rms_target=0.0, with_e2e=Tru
 
     # every library kernel of one step, timed live with CUDA events on its launching stream
     kernels = ["phi_prepare", "keystats", "query", "bwd_query", "bwd_key", "grad_sum", "mlp_grads",
-               "causal_out", "causal_bwd_seg", "causal_dq", "causal_dkv"] + L.TC_KERNELS
+               "part_reduce", "causal_out", "causal_bwd_query", "causal_bwd_key"] + L.TC_KERNELS
     if ch_rms_target > 0:
         kernels += ["chrms_stats", "tc_chstats", "chrms_scales", "chrms_scale", "chrms_dstate", "chrms_kappa",
                     "chrms_kterm", "tc_kterm"]
