@@ -62,7 +62,6 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
     const Rows sQ = take_rows(cv, cap, d), sK = take_rows(cv, cap, d), sV = take_rows(cv, cap, dv);
     const Rows sPq = take_rows(cv, cap, D), sPk = take_rows(cv, cap, D), sA = take_rows(cv, cap, cap);
     float *sden = cv.take(cap), *sinv = cv.take(cap);
-    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(8));  // [2 tiles] largest |phi(k)|, |V|
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
     const int len = head_length(a.lengths, bh / a.H, a.n);
@@ -74,30 +73,27 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
     load_phi_tile(s, lay, a.table);
     const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
     __syncthreads();
-    load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv, nullptr);
+    load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv);
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
     const bool vec = vec_store(O, dv);
-    int par = 0;
-    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 4) {
+    for (int t0 = r0; t0 < r1; t0 += cap) {
         const int nr = min(cap, r1 - t0);
-        unsigned *mx = mxs + par;
         __syncthreads();
-        if (threadIdx.x < 4) mxs[(par ^ 4) + threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + 1);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, nullptr);
-        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx);
+        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr);
+        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr);
         __syncthreads();
-        scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int) { return 0.0f; }, [](int, float &, float &) {});
+        scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int, float &, float &) {});
         __syncthreads();
         tile_dens(sPq, nr, D, z, sA, a.eps, sden, sinv);
         __syncthreads();
         // O_r = (phi(q_r) S + sum_{j<=r} A[r][j] v_j) / den_r from the pair of the numerator
-        prod_nn(sPq, nr, S, Dp, dv, sA, sV, [](int) { return 0.0f; },
+        prod_nn(sPq, nr, S, Dp, dv, sA, sV,
                 [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
@@ -111,9 +107,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
                 });
         if (t0 + cap >= r1) break;
         __syncthreads();
-        const float zbound = (float)nr * __uint_as_float(mx[0]);
-        advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base(zbound * __uint_as_float(mx[1])), pair_base(zbound),
-                     nullptr);
+        advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr);
     }
 }
 
@@ -140,8 +134,6 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
     float *sU = cv.take(cap * M);
     int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
     float *sdU = cv.take(cap * du_stride(M));
-    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(16));  // [2 tiles] largest |S|, |z|, |V|, |dO|, |phi(q)|,
-                                                               // |phi(k)|, |dnum|, |dden|
     cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
@@ -163,69 +155,51 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
         load_phi_tile(s, lay, a.table);
         const size_t so = head_state(a, bh) * (a.nseg + 1) + seg;
         __syncthreads();
-        load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv, mxs);
+        load_state(S, z, a.seg_S + so * D * dv, a.seg_z + so * D, D, dv);
     }
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
     const IO *dO = static_cast<const IO *>(a.dO) + head_rows(a, bh) * dv;
-    const Rows none{};
-    int par = 0;
-    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 8) {
+    for (int t0 = r0; t0 < r1; t0 += cap) {
         const int nr = min(cap, r1 - t0);
-        unsigned *mx = mxs + par, *mx_next = mxs + (par ^ 8);
         __syncthreads();
-        if (threadIdx.x < 8) mx_next[threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + 2);
-        block_max(load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap), mx + 3);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
+        load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_rows(lay, s, sQ, nr, cap, sPq, sU, sJ, mx + 4);
-        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr, mx + 5);
+        phi_rows(lay, s, sQ, nr, cap, sPq, sU, sJ);
+        phi_rows(lay, s, sK, nr, cap, sPk, nullptr, nullptr);
         __syncthreads();
-        const float mS = __uint_as_float(mx[0]), mz = __uint_as_float(mx[1]), mV = __uint_as_float(mx[2]);
-        const float mdO = __uint_as_float(mx[3]), mq = __uint_as_float(mx[4]), mk = __uint_as_float(mx[5]);
         // pairs too: o and den are formed from A, and a common rounding error of theirs does not cancel in dphi
-        const float bA = pair_base((float)D * mq * mk);
-        scores_lower<true>(sPq, sPk, nr, Dp, sA, [&](int) { return bA; }, [](int, float &, float &) {});
+        scores_lower<true>(sPq, sPk, nr, Dp, sA, [](int, float &, float &) {});
         __syncthreads();
         row_dots(sPq, nr, D, [&](int, int f) { return z[f]; }, sA, [](int r) { return r + 1; },
                  [&](int r, float h, float l) { rp.set_den(r, h, l, a.eps); });
         __syncthreads();
-        block_max(rp.divide_rows(sdO, nr, dv), mx + 6);  // dnum in place
+        rp.divide_rows(sdO, nr, dv);  // dnum in place
         __syncthreads();
-        const float bnum = pair_base((float)D * mq * fmaf((float)nr * mk, mV, mS));
-        prod_nn(sPq, nr, S, Dp, dv, sA, sV, [&](int) { return bnum; },
-                [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
-                    unit_dots(sdO, sR, nr, q0, c0, h, l, bnum);
-                });
+        prod_nn(sPq, nr, S, Dp, dv, sA, sV, [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
+            unit_dots(sdO, sR, nr, q0, c0, h, l);
+        });
         __syncthreads();
         sum_unit_dots(sR, nr, dvp / 4, [&](int r, float h, float l) {
             rp.set_dden(r, h, l);
-            atomicMax(mx + 7, __float_as_uint(fabsf(rp.gh[r])));
-            // starts of the row's sums: |dP[r][.]| and the terms of dphi(q_r) stay below these bounds
-            const bool live = rp.dh[r] != 0.0f;
-            const float iv = fabsf(rp.inv[r]), gd = fabsf(rp.gh[r]);
-            const float bound_p = fmaf(2.0f * (float)dv * mV * mdO, iv, gd);
-            rp.bp[r] = live ? pair_base(bound_p) : 0.0f;
-            rp.bq[r] = live ? pair_base(fmaf(2.0f * (float)dv * mS * mdO, iv, mz * gd) + (float)nr * mk * bound_p) : 0.0f;
             *reinterpret_cast<float4 *>(a.rowstat + ((size_t)bh * a.n + t0 + r) * 4) =
                 make_float4(rp.dh[r], rp.dl[r], rp.gh[r], rp.gl[r]);
         });
         __syncthreads();
-        scores_lower<true>(sdO, sV, nr, dvp, sA, [&](int r) { return rp.bp[r]; }, [&](int r, float &h, float &l) {
-            pair_mac(h, l, rp.gh[r], 1.0f);
-            l = __fadd_rn(l, rp.gl[r]);
+        scores_lower<true>(sdO, sV, nr, dvp, sA, [&](int r, float &h, float &l) {
+            if (r < nr) { h = rp.gh[r]; l = rp.gl[r]; }
         });
-        acc.add(sPq, D, sdO, dv, rp.gh, rp.gl, nr, pair_base((float)nr * mq * __uint_as_float(mx[6])),
-                pair_base((float)nr * mq * __uint_as_float(mx[7])));
+        acc.add(sPq, D, sdO, dv, rp.gh, rp.gl, nr);
         __syncthreads();
-        prod_nt<kLower>(sdO, nr, S, D, dvp, sA, sPk, nr, [&](int r) { return rp.bq[r]; },
+        prod_nt<kLower>(sdO, nr, S, D, dvp, sA, sPk, nr,
                         [&](int r, int f, float &h, float &l) {
                             if (r < nr) {
-                                l = z[f] * rp.gl[r];
                                 pair_mac(h, l, z[f], rp.gh[r]);
+                                l = __fmaf_rn(z[f], rp.gl[r], l);
                             }
                         },
                         [&](int r, int f, float h, float l) {
@@ -234,9 +208,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
                             if (a.ch_T) atomicAdd(sT + f % a.L, (double)sPq[r][f] * ((double)h + (double)l));
                         });
         __syncthreads();
-        if (t0 + cap < r1)
-            advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr, pair_base((float)nr * mk * mV), pair_base((float)nr * mk),
-                         mx_next);
+        if (t0 + cap < r1) advance_rows(S, z, sPk, D, sV, dv, nullptr, nullptr, nr);
         phi_backward_rows(lay, s, sQ, nr, cap, sPq, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
@@ -275,7 +247,6 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     float *sU = cv.take(cap * M);
     int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
     float *sdU = cv.take(cap * du_stride(M));
-    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(16));  // [2 tiles] largest |G|, |g|, |V|, |dden|, |dnum|, |phi(q)|
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
     double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nseg + seg) % nbuf) * a.gsize;
@@ -291,7 +262,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     load_phi_tile(s, lay, a.table);
     const size_t so = (size_t)bh * a.nseg + seg;
     __syncthreads();
-    load_state(G, gz, a.seg_dS + so * D * dv, a.seg_dz + so * D, D, dv, mxs);
+    load_state(G, gz, a.seg_dS + so * D * dv, a.seg_dz + so * D, D, dv);
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
@@ -299,54 +270,37 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     const bool vec = vec_store(dV, dv);
     GradTile g;
     grad_zero(g);
-    int par = 0;
-    for (int t0 = r0 + ((r1 - 1 - r0) / cap) * cap; t0 >= r0; t0 -= cap, par ^= 8) {
+    for (int t0 = r0 + ((r1 - 1 - r0) / cap) * cap; t0 >= r0; t0 -= cap) {
         const int nr = min(cap, r1 - t0);
-        unsigned *mx = mxs + par, *mx_next = mxs + (par ^ 8);
         __syncthreads();
-        if (threadIdx.x < 8) mx_next[threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + 2);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
         load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
-        float mdd = 0.0f;
         for (int r = threadIdx.x; r < cap; r += blockDim.x) {
             const float4 v = r < nr ? ld4(a.rowstat + ((size_t)bh * a.n + t0 + r) * 4) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             rp.dh[r] = v.x; rp.dl[r] = v.y; rp.inv[r] = 1.0f / v.x;
             rp.gh[r] = v.z; rp.gl[r] = v.w;
-            mdd = fabsf(v.z);
         }
-        block_max(mdd, mx + 3);
         __syncthreads();
-        block_max(rp.divide_rows(sdO, nr, dv), mx + 4);  // dnum in place
-        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr, mx + 5);
-        phi_rows(lay, s, sK, nr, cap, sPk, sU, sJ, nullptr);
+        rp.divide_rows(sdO, nr, dv);  // dnum in place
+        phi_rows(lay, s, sQ, nr, cap, sPq, nullptr, nullptr);
+        phi_rows(lay, s, sK, nr, cap, sPk, sU, sJ);
         __syncthreads();
-        scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int) { return 0.0f; }, [](int, float &, float &) {});
-        const float mG = __uint_as_float(mx[0]), mg = __uint_as_float(mx[1]), mV = __uint_as_float(mx[2]);
-        mdd = __uint_as_float(mx[3]);
-        const float mdn = __uint_as_float(mx[4]), mq = __uint_as_float(mx[5]);
-        const float bound_p = fmaf((float)dv * mdn, mV, mdd), bp = pair_base(bound_p);
-        const float bk = pair_base(fmaf((float)dv * mG, mV, mg) + (float)nr * mq * bound_p);
-        scores_lower<true>(sdO, sV, nr, dvp, sP, [&](int) { return bp; }, [&](int r, float &h, float &l) {
-            pair_mac(h, l, rp.gh[r], 1.0f);
-            l = __fadd_rn(l, rp.gl[r]);
-        });
+        scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int, float &, float &) {});
+        scores_lower<true>(sdO, sV, nr, dvp, sP, [&](int r, float &h, float &l) { h = rp.gh[r]; l = rp.gl[r]; });
         __syncthreads();
         prod_nn_plain(sPk, nr, G, Dp, dv, sA, sdO, nr, [&](int q0, int c0, const float (&h)[2][4]) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
                 if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);
         });
-        prod_nt<kUpper>(sV, nr, G, D, dvp, sP, sPq, nr, [&](int) { return bk; },
-                        [&](int, int f, float &h, float &l) { pair_mac(h, l, gz[f], 1.0f); },
+        prod_nt<kUpper>(sV, nr, G, D, dvp, sP, sPq, nr, [&](int, int f, float &h, float &) { h = gz[f]; },
                         [&](int r, int f, float h, float l) {
                             if (r < nr) sdPhi[r][f] = pair_value(h, l);
                         });
         __syncthreads();
-        if (t0 > r0)
-            advance_rows(G, gz, sPq, D, sdO, dv, rp.gh, rp.gl, nr, pair_base((float)nr * mq * mdn),
-                         pair_base((float)nr * mq * mdd), mx_next);
+        if (t0 > r0) advance_rows(G, gz, sPq, D, sdO, dv, rp.gh, rp.gl, nr);
         phi_backward_rows(lay, s, sK, nr, cap, sPk, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dK + (size_t)t0 * d);
     }
@@ -360,7 +314,7 @@ size_t smem_out(const AttnArgs &a, int cap) {
     take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
     take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv);
     take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, cap);
-    cv.take(cap); cv.take(cap); cv.take(8);
+    cv.take(cap); cv.take(cap);
     return cv.bytes();
 }
 size_t smem_bwd_query(const AttnArgs &a, int cap) {
@@ -370,7 +324,7 @@ size_t smem_bwd_query(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, a.D); take_rows_host(cv, cap, cap);
     cv.take(cap * std::max(row_stride(a.d), std::max(row_stride(a.dv), row_stride(a.D))));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
-    cv.take(16); cv.take(kSlack);
+    cv.take(kSlack);
     return cv.bytes();
 }
 size_t smem_bwd_key(const AttnArgs &a, int cap) {
@@ -381,7 +335,6 @@ size_t smem_bwd_key(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, cap); take_rows_host(cv, cap, cap);
     cv.take(cap * std::max(row_stride(a.d), row_stride(a.D)));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
-    cv.take(16);
     return cv.bytes();
 }
 

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kThreads) k_featmap_var(TableLayout lay, const
         __syncthreads();
         load_tile(sX, X + t0 * lay.d, nr, lay.d, kPhiRows);
         __syncthreads();
-        phi_rows(lay, s, sX, nr, kPhiRows, sPhi, nullptr, nullptr, nullptr);
+        phi_rows(lay, s, sX, nr, kPhiRows, sPhi, nullptr, nullptr);
         __syncthreads();
         for (int e = threadIdx.x; e < nr * lay.D; e += blockDim.x) Phi[t0 * lay.D + e] = sPhi[e / lay.D][e % lay.D];
     }
@@ -89,10 +89,8 @@ __global__ void __launch_bounds__(kThr, 1) k_keystats(AttnArgs a, int cap, int p
     const TableLayout &lay = a.lay;
     SmemPhi s = carve_phi_tile(cv, lay, cap);
     const Rows sK = take_rows(cv, cap, a.d), sV = take_rows(cv, cap, a.dv), sPhi = take_rows(cv, cap, a.D);
-    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(8));  // [2 tiles] largest |phi|, |V|
     cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
-    zero_words(reinterpret_cast<float *>(mxs), 8);
     load_phi_tile(s, lay, a.table);
 
     const int bh = blockIdx.y, split = blockIdx.x;
@@ -103,19 +101,15 @@ __global__ void __launch_bounds__(kThr, 1) k_keystats(AttnArgs a, int cap, int p
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * a.dv;
     OuterAcc<TF, TC> acc;
     acc.zero();
-    int par = 0;
-    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 4) {
+    for (int t0 = r0; t0 < r1; t0 += cap) {
         const int nr = min(cap, r1 - t0);
-        unsigned *mx = mxs + par;
         __syncthreads();
-        if (threadIdx.x < 4) mxs[(par ^ 4) + threadIdx.x] = 0u;
         load_tile(sK, K + (size_t)t0 * a.d, nr, a.d, cap);
-        block_max(load_tile(sV, V + (size_t)t0 * a.dv, nr, a.dv, cap), mx + 1);
+        load_tile(sV, V + (size_t)t0 * a.dv, nr, a.dv, cap);
         __syncthreads();
-        phi_rows(lay, s, sK, nr, cap, sPhi, nullptr, nullptr, mx);
+        phi_rows(lay, s, sK, nr, cap, sPhi, nullptr, nullptr);
         __syncthreads();
-        const float zbound = (float)nr * __uint_as_float(mx[0]);
-        acc.add(sPhi, a.D, sV, a.dv, nullptr, nullptr, nr, pair_base(zbound * __uint_as_float(mx[1])), pair_base(zbound));
+        acc.add(sPhi, a.D, sV, a.dv, nullptr, nullptr, nr);
     }
     const size_t slot = (size_t)bh * a.nsplit + split;
     acc.store(a.D, a.dv, a.S_part, a.z_part, slot, pairs != 0);
@@ -157,7 +151,7 @@ __global__ void __launch_bounds__(kThr, 1) k_query(AttnArgs a, int cap, int rows
     float *sden = cv.take(cap);
     if (!carve_fits(cv, smem)) return;
     load_phi_tile(s, lay, a.table);
-    load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv, nullptr);
+    load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv);
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * a.d;
     const Rows none{};
     const bool vec = vec_store(O, dv);
@@ -167,7 +161,7 @@ __global__ void __launch_bounds__(kThr, 1) k_query(AttnArgs a, int cap, int rows
         __syncthreads();
         load_tile(sQ, Q + (size_t)t0 * a.d, nr, a.d, cap);
         __syncthreads();
-        phi_rows(lay, s, sQ, nr, cap, sPhi, nullptr, nullptr, nullptr);
+        phi_rows(lay, s, sQ, nr, cap, sPhi, nullptr, nullptr);
         __syncthreads();
         row_dots(sPhi, nr, D, [&](int, int f) { return sz[f]; }, none, [](int) { return 0; },
                  [&](int r, float h, float l) {
@@ -210,7 +204,6 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
     float *sU = cv.take(cap * M);
     int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
     float *sdU = cv.take(cap * du_stride(M));
-    unsigned *mxs = reinterpret_cast<unsigned *>(cv.take(12));  // largest |S|, |z|; [2 tiles] |phi|, |dO|, |dnum|, |dden|
     cv.take(kSlack);
     if (!carve_fits(cv, smem)) return;
     zero_words(tiles, (int)(cv.p - tiles));
@@ -220,7 +213,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
     double *gp = reinterpret_cast<double *>(a.gpart) + (slot % nbuf) * a.gsize;
     double *hist = gp + M * d + M;
     __syncthreads();
-    load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv, mxs);
+    load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv);
 
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = split * a.rows_per_split_b;
@@ -236,45 +229,31 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
     acc.zero();
     GradTile g;
     grad_zero(g);
-    int par = 4;
-    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 12) {
+    for (int t0 = r0; t0 < r1; t0 += cap) {
         const int nr = min(cap, r1 - t0);
-        unsigned *mx = mxs + par;
         __syncthreads();
-        if (threadIdx.x < 4) mxs[(par ^ 12) + threadIdx.x] = 0u;
         load_tile(sQ, Q + (size_t)t0 * d, nr, d, cap);
-        block_max(load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap), mx + 1);
+        load_tile(sdO, dO + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_rows(lay, s, sQ, nr, cap, sPhi, sU, sJ, mx);
+        phi_rows(lay, s, sQ, nr, cap, sPhi, sU, sJ);
         __syncthreads();
         row_dots(sPhi, nr, D, [&](int, int f) { return sz[f]; }, none, [](int) { return 0; },
                  [&](int r, float h, float l) { rp.set_den(r, h, l, a.eps); });
         __syncthreads();
-        block_max(rp.divide_rows(sdO, nr, dv), mx + 2);  // dnum in place
+        rp.divide_rows(sdO, nr, dv);  // dnum in place
         __syncthreads();
-        const float mS = __uint_as_float(mxs[0]), mz = __uint_as_float(mxs[1]), mp = __uint_as_float(mx[0]);
-        const float mdO = __uint_as_float(mx[1]);
-        const float bnum = pair_base((float)D * mS * mp);
-        prod_nn(sPhi, nr, sS, Dp, dv, none, none, [&](int) { return bnum; },
-                [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
-                    unit_dots(sdO, sP, nr, q0, c0, h, l, bnum);
-                });
-        __syncthreads();
-        sum_unit_dots(sP, nr, dvp / 4, [&](int r, float h, float l) {
-            rp.set_dden(r, h, l);
-            atomicMax(mx + 3, __float_as_uint(fabsf(rp.gh[r])));
-            rp.bq[r] = rp.dh[r] != 0.0f
-                           ? pair_base(fmaf(2.0f * (float)dv * mS * mdO, fabsf(rp.inv[r]), mz * fabsf(rp.gh[r]))) : 0.0f;
+        prod_nn(sPhi, nr, sS, Dp, dv, none, none, [&](int q0, int c0, const float (&h)[2][4], const float (&l)[2][4]) {
+            unit_dots(sdO, sP, nr, q0, c0, h, l);
         });
         __syncthreads();
-        const float bound = (float)nr * mp;
-        acc.add(sPhi, D, sdO, dv, rp.gh, rp.gl, nr, pair_base(bound * __uint_as_float(mx[2])),
-                pair_base(bound * __uint_as_float(mx[3])));
-        prod_nt<kNone>(sdO, nr, sS, D, dvp, none, none, 0, [&](int r) { return rp.bq[r]; },
+        sum_unit_dots(sP, nr, dvp / 4, [&](int r, float h, float l) { rp.set_dden(r, h, l); });
+        __syncthreads();
+        acc.add(sPhi, D, sdO, dv, rp.gh, rp.gl, nr);
+        prod_nt<kNone>(sdO, nr, sS, D, dvp, none, none, 0,
                        [&](int r, int f, float &h, float &l) {
                            if (r < nr) {
-                               l = sz[f] * rp.gl[r];
                                pair_mac(h, l, sz[f], rp.gh[r]);
+                               l = __fmaf_rn(sz[f], rp.gl[r], l);
                            }
                        },
                        [&](int r, int f, float h, float l) {
@@ -311,7 +290,6 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nb
     float *sU = cv.take(cap * M);
     int *sJ = reinterpret_cast<int *>(cv.take(cap * M));
     float *sdU = cv.take(cap * du_stride(M));
-    unsigned *mx = reinterpret_cast<unsigned *>(cv.take(4));  // largest |dS|, |dz|; [2 tiles] |V|
     if (!carve_fits(cv, smem)) return;
     zero_words(tiles, (int)(cv.p - tiles));
     load_phi_tile(s, lay, a.table);
@@ -319,7 +297,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nb
     double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nsplit_b + split) % nbuf) * a.gsize;
     double *hist = gp + M * d + M;
     __syncthreads();
-    load_state(sdS, sdz, a.dS_fin + (size_t)bh * D * dv, a.dz_fin + (size_t)bh * D, D, dv, mx);
+    load_state(sdS, sdz, a.dS_fin + (size_t)bh * D * dv, a.dz_fin + (size_t)bh * D, D, dv);
 
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = split * a.rows_per_split_b;
@@ -336,25 +314,20 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nb
     const bool vec = vec_store(dV, dv);
     GradTile g;
     grad_zero(g);
-    int par = 2;
-    for (int t0 = r0; t0 < r1; t0 += cap, par ^= 1) {
+    for (int t0 = r0; t0 < r1; t0 += cap) {
         const int nr = min(cap, r1 - t0);
         __syncthreads();
-        if (threadIdx.x == 0) mx[par ^ 1] = 0u;
         load_tile(sK, K + (size_t)t0 * d, nr, d, cap);
-        block_max(load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap), mx + par);
+        load_tile(sV, V + (size_t)t0 * dv, nr, dv, cap);
         __syncthreads();
-        phi_rows(lay, s, sK, nr, cap, sPhi, sU, sJ, nullptr);
+        phi_rows(lay, s, sK, nr, cap, sPhi, sU, sJ);
         __syncthreads();
         prod_nn_plain(sPhi, nr, sdS, Dp, dv, none, none, 0, [&](int q0, int c0, const float (&h)[2][4]) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
                 if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);
         });
-        const float base = pair_base(fmaf((float)dv * __uint_as_float(mx[0]), __uint_as_float(mx[par]),
-                                          __uint_as_float(mx[1])));
-        prod_nt<kNone>(sV, nr, sdS, D, dvp, none, none, 0, [&](int) { return base; },
-                       [&](int, int f, float &h, float &l) { pair_mac(h, l, sdz[f], 1.0f); },
+        prod_nt<kNone>(sV, nr, sdS, D, dvp, none, none, 0, [&](int, int f, float &h, float &) { h = sdz[f]; },
                        [&](int r, int f, float h, float l) {
                            if (r < nr) sdPhi[r][f] = pair_value(h, l);
                        });
@@ -621,7 +594,7 @@ __global__ void __launch_bounds__(128) k_mlp_fc1_sum(TableLayout lay, const doub
 size_t smem_keystats(const AttnArgs &a, int cap) {
     HostCarve cv; carve_phi_tile_host(cv, a.lay, cap);
     take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
-    cv.take(8); cv.take(kSlack);
+    cv.take(kSlack);
     return cv.bytes();
 }
 size_t smem_query(const AttnArgs &a, int cap) {
@@ -636,7 +609,7 @@ size_t smem_bwd_query(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
     cv.take(cap * std::max(row_stride(a.dv), row_stride(a.D)));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
-    cv.take(12); cv.take(kSlack);
+    cv.take(kSlack);
     return cv.bytes();
 }
 size_t smem_bwd_key(const AttnArgs &a, int cap) {
@@ -644,7 +617,7 @@ size_t smem_bwd_key(const AttnArgs &a, int cap) {
     take_rows_host(cv, r4(a.D), a.dv); cv.take(r4(a.D));
     take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
     take_rows_host(cv, cap, a.D);
-    cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M)); cv.take(4);
+    cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
     return cv.bytes();
 }
 

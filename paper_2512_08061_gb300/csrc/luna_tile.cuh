@@ -4,8 +4,8 @@
 // What bounds these kernels is arithmetic.  The parameter gradients are sums of terms that cancel by factors
 // of hundreds, so the statistics, the row normalisers, the outputs and dphi have to be formed to more than
 // fp32 and rounded once.  fp64 does that at 2 multiply-adds per cycle and SM on this part (measured through
-// the fp64 form of these kernels: 0.6 T/s); the pair form below does it with four fp32 operations at 128 per
-// cycle and SM, 16 times the rate, and keeps about 46 bits.
+// the fp64 form of these kernels: 0.6 T/s); the pair form below does it with five fp32 operations at 128 per
+// cycle and SM, and keeps about 46 bits of sum_k |a_k b_k| (pair_base).
 #pragma once
 
 #include <algorithm>
@@ -66,7 +66,8 @@ inline int grad_buffers(int64_t blocks, int64_t room) {
 // Sums as pairs h + l.
 
 // (h, l) += a b with the rounding error of h's update carried in l.  The product is exact (fma).  The error is
-// exact where |h| >= |a b|; elsewhere up to half an ulp of a b is lost, which `pair_base` rules out.
+// exact where |h| >= |a b| and the sum does not cancel; elsewhere up to half an ulp of a b is lost.  A start value
+// from `pair_base` rules both out.
 __device__ __forceinline__ void pair_mac(float &h, float &l, float a, float b) {
     const float t = __fmaf_rn(a, b, h);
     const float q = __fsub_rn(t, h);
@@ -102,9 +103,12 @@ __device__ __forceinline__ double pair_double(float h, float l) {
     return fabsf(h) < INFINITY ? (double)h + (double)l : (double)h;
 }
 
-// Start value of a sum whose partial sums stay below `bound`: 1.5 times a power of two at least twice the
-// bound.  h then never leaves one binade, so every update of pair_mac is exact to 2^-24 of the start value's
-// ulp, also where the terms cancel.  0 (an ordinary start) for a bound that is not finite.
+// Start value of a sum whose terms' sizes add up to `bound`: 1.5 times a power of two at least twice the bound.
+// h then never leaves one binade, so every update of pair_mac is exact to 2^-24 of the start value's ulp, also
+// where the terms cancel.  The bound is the sum's own, sum_k |a_k b_k|, formed in a pass of its own before it (one
+// operation more per product, and its loads again): with one bound for a whole tile (rows x largest |a| x largest
+// |b|) a column of values 1e-4 of the largest was summed no better than in fp32, and an outlier in one row cost
+// every other sum of its tile its low half.  0 (an ordinary start) for a bound that is not finite or above 1e37.
 __device__ __forceinline__ float pair_base(float bound) {
     if (!(bound < 1e37f)) return 0.0f;
     const int e = (__float_as_int(bound) >> 23) & 0xff;
@@ -143,58 +147,37 @@ __device__ __forceinline__ bool vec_rows(const void *p, int w) {
     return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (w * sizeof(IO)) % 16 == 0;
 }
 
-__device__ __forceinline__ float max4(const float4 &v, float m) {
-    if (v.x != v.x || v.y != v.y || v.z != v.z || v.w != v.w) return INFINITY;
-    return fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fmaxf(fabsf(v.y), fabsf(v.z))), fabsf(v.w));
+__device__ __forceinline__ void put16(float *dst, const float *, const uint4 &v) {
+    st4(dst, make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w)));
 }
-__device__ __forceinline__ float put16(float *dst, const float *, const uint4 &v, float m) {
-    const float4 a = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
-    st4(dst, a);
-    return max4(a, m);
-}
-__device__ __forceinline__ float put16(float *dst, const __nv_bfloat16 *, const uint4 &v, float m) {
-    const float4 a = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
-                                 __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
-    const float4 b = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
-                                 __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
-    st4(dst, a);
-    st4(dst + 4, b);
-    return max4(b, max4(a, m));
+__device__ __forceinline__ void put16(float *dst, const __nv_bfloat16 *, const uint4 &v) {
+    st4(dst, make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                         __uint_as_float(v.y & 0xffff0000u)));
+    st4(dst + 4, make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u), __uint_as_float(v.w << 16),
+                             __uint_as_float(v.w & 0xffff0000u)));
 }
 
-// nr contiguous rows of w elements into the tile (cap rows); the pad columns and the rows from nr on are 0.  Returns
-// the largest |value| this thread has read (infinity with a NaN), for block_max.
+// nr contiguous rows of w elements into the tile (cap rows); the pad columns and the rows from nr on are 0.
 template <typename IO>
-__device__ float load_tile(const Rows &t, const IO *src, int nr, int w, int cap) {
+__device__ void load_tile(const Rows &t, const IO *src, int nr, int w, int cap) {
     constexpr int VE = 16 / sizeof(IO);
-    float m = 0.0f;
     if (vec_rows<IO>(src, w)) {
         const Div wv(w / VE);
 #pragma unroll 2
         for (int e = threadIdx.x; e < nr * wv.n; e += blockDim.x) {
             const int r = wv(e), c = (e - r * wv.n) * VE;
-            m = put16(t[r] + c, src, *reinterpret_cast<const uint4 *>(src + (size_t)e * VE), m);
+            put16(t[r] + c, src, *reinterpret_cast<const uint4 *>(src + (size_t)e * VE));
         }
     } else {
         for (int e = threadIdx.x; e < nr * w; e += blockDim.x) {
             const int r = e / w, c = e - r * w;
-            const float v = io_load(src + e);
-            t[r][c] = v;
-            m = v == v ? fmaxf(m, fabsf(v)) : INFINITY;
+            t[r][c] = io_load(src + e);
         }
         const int wp = (w + 3) & ~3;
         if (wp != w)
             for (int e = threadIdx.x; e < nr * (wp - w); e += blockDim.x) t[e / (wp - w)][w + e % (wp - w)] = 0.0f;
     }
     for (int e = threadIdx.x; e < (cap - nr) * t.ld; e += blockDim.x) t[nr][e] = 0.0f;
-    return m;
-}
-
-// The largest of the threads' values m >= 0 into *slot, as the bits of a float (zeroed before, in an earlier phase).
-__device__ __forceinline__ void block_max(float m, unsigned *slot) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(slot, __float_as_uint(m));
 }
 
 // ---------------------------------------------------------------------------
@@ -265,10 +248,9 @@ __device__ void load_phi_tile(const SmemPhi &s, const TableLayout &lay, const ch
 // phi of rows [0, nr) of X into Phi, zeros in its other rows (cap in all) and pad columns; with sU also the
 // projections u[r * M + i] and their intervals.  The projection is one fma chain over the columns in order, as
 // in every generic kernel: which side of a kink a row falls on does not depend on the kernel.  Called by every
-// thread of the block; synchronises it first if the map has a gate or coefficients.  slot (or null): the largest
-// |phi|, as for block_max.
+// thread of the block; synchronises it first if the map has a gate or coefficients.
 __device__ void phi_rows(const TableLayout &lay, const SmemPhi &s, const Rows &X, int nr, int cap, const Rows &Phi,
-                         float *sU, int *sJ, unsigned *slot) {
+                         float *sU, int *sJ) {
     const int M = lay.M, L = lay.L, d = lay.d, D = lay.D, ldw = row_stride(d), dp = (d + 3) & ~3;
     const float fl = channel_floor(lay);
     const bool ev = lay.env || lay.coef;
@@ -280,7 +262,6 @@ __device__ void phi_rows(const TableLayout &lay, const SmemPhi &s, const Rows &X
     const float sc = phi_scale(lay);
     const unsigned short *sB = reinterpret_cast<const unsigned short *>(s.T + kSearchT);
     const Div byM(M);
-    float mx = 0.0f;
     for (int e = threadIdx.x; e < cap * M; e += blockDim.x) {
         const int r = byM(e), i = e - r * M;
         float *out = Phi[r] + i * L;
@@ -310,40 +291,49 @@ __device__ void phi_rows(const TableLayout &lay, const SmemPhi &s, const Rows &X
                 for (int l = 0; l < 8; ++l) {
                     const float2 p = ab_pair(ab, l);
                     y[l] = fmaxf(fmaf(p.x, u, p.y), fl);
-                    mx = fmaxf(mx, fabsf(y[l]));
                 }
                 st4(out, make_float4(y[0], y[1], y[2], y[3]));
                 st4(out + 4, make_float4(y[4], y[5], y[6], y[7]));
             } else {
                 for (int l = 0; l < L; ++l) {
                     const float2 p = ab_pair(ab, l);
-                    const float v = fmaxf(fmaf(p.x, u, p.y), fl);
-                    out[l] = v;
-                    mx = fmaxf(mx, fabsf(v));
+                    out[l] = fmaxf(fmaf(p.x, u, p.y), fl);
                 }
             }
         } else {
-            for (int l = 0; l < L; ++l) {
-                const float v = fmaxf(sc * channel_direct(lay, s, l, u, nullptr), fl);
-                out[l] = v;
-                mx = fmaxf(mx, fabsf(v));
-            }
+            for (int l = 0; l < L; ++l) out[l] = fmaxf(sc * channel_direct(lay, s, l, u, nullptr), fl);
         }
         if (ev)
-            for (int l = 0; l < L; ++l) {
-                const float v = out[l] * s.E[r * L + l];
-                out[l] = v;
-                mx = fmaxf(mx, fabsf(v));
-            }
+            for (int l = 0; l < L; ++l) out[l] *= s.E[r * L + l];
         if (sU) { sU[e] = u; sJ[e] = j; }
     }
-    if (slot) block_max(mx, slot);
 }
 
 // ---------------------------------------------------------------------------
 // Products.  A unit is 2 rows x 4 columns of the result per thread: six 16-byte shared loads for 32 products
-// (128 operations in pair form), so the loads take a small part of the issue slots and of the shared-memory
-// bandwidth, and the eight chains of a unit hide the fma latency with four warps per scheduler.
+// (160 operations in pair form with the bounds), so the loads take a small part of the issue slots and of the
+// shared-memory bandwidth, and the eight chains of a unit hide the fma latency with four warps per scheduler.
+
+__device__ __forceinline__ void abs_mac(float &s, float a, float b) { s = fmaf(fabsf(a), fabsf(b), s); }
+
+// The start values of a unit's sums from their bounds, in place; h starts there.
+__device__ __forceinline__ void unit_base(float (&b)[2][4], float (&h)[2][4], float (&l)[2][4]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            b[i][m] = pair_base(b[i][m]);
+            h[i][m] = b[i][m];
+            l[i][m] = 0.0f;
+        }
+}
+// The sums without their start values (exact).
+__device__ __forceinline__ void unit_unbase(float (&h)[2][4], const float (&b)[2][4]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) h[i][m] = __fsub_rn(h[i][m], b[i][m]);
+}
 
 // One step of a unit's sums over four k: rows x0, x1 of A (k .. k + 3) and the four B rows at b.
 __device__ __forceinline__ void unit_nn(float (&h)[2][4], float (&l)[2][4], const float4 &x0, const float4 &x1,
@@ -355,6 +345,18 @@ __device__ __forceinline__ void unit_nn(float (&h)[2][4], float (&l)[2][4], cons
         for (int m = 0; m < 4; ++m) {
             pair_mac(h[0][m], l[0][m], at(x0, kk), at(v, m));
             pair_mac(h[1][m], l[1][m], at(x1, kk), at(v, m));
+        }
+    }
+}
+// The step's share of the bounds.
+__device__ __forceinline__ void unit_abs_nn(float (&s)[2][4], const float4 &x0, const float4 &x1, const float *b, int ldb) {
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+        const float4 v = ld4(b + kk * ldb);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            abs_mac(s[0][m], at(x0, kk), at(v, m));
+            abs_mac(s[1][m], at(x1, kk), at(v, m));
         }
     }
 }
@@ -371,22 +373,31 @@ __device__ __forceinline__ void unit_nn(float (&h)[2][4], const float4 &x0, cons
 }
 
 // out(r, c) = sum_{k < K} A[r][k] B[k][c] + sum_{k <= r} T[r][k] B2[k][c] (K rounded up to a multiple of 4; T null:
-// the first sum alone): a unit's rows r0, r0 + 1 and columns c0 .. c0 + 3 go to done(r0, c0, h, l).  The sums start
-// at base(r).  The triangle ends exactly at the diagonal: a later row's infinity must not meet a zero of T.
-template <typename Base, typename Done>
+// the first sum alone): a unit's rows r0, r0 + 1 and columns c0 .. c0 + 3 go to done(r0, c0, h, l) as pairs.  The
+// triangle ends exactly at the diagonal: a later row's infinity must not meet a zero of T.
+template <typename Done>
 __device__ __forceinline__ void prod_nn(const Rows &A, int rows, const Rows &B, int K, int cols, const Rows &T,
-                                        const Rows &B2, Base base, Done done) {
+                                        const Rows &B2, Done done) {
     const int ng = (cols + 3) / 4, nu = ((rows + 1) / 2) * ng;
     const Div by(ng);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
         const int g = by(u), r0 = 2 * g, c0 = 4 * (u - g * ng);
-        float h[2][4], l[2][4];
+        float h[2][4], l[2][4], b[2][4] = {};
+        for (int k = 0; k < K; k += 4) unit_abs_nn(b, ld4(A[r0] + k), ld4(A[r0 + 1] + k), B[k] + c0, B.ld);
+        if (T.p) {
+            int k = 0;
+            for (; k + 4 <= r0 + 1; k += 4) unit_abs_nn(b, ld4(T[r0] + k), ld4(T[r0 + 1] + k), B2[k] + c0, B2.ld);
+            for (; k <= r0 + 1; ++k) {
+                const float4 v = ld4(B2[k] + c0);
+                const float x0 = T[r0][k], x1 = T[r0 + 1][k];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const float s = base(r0 + i);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) { h[i][m] = s; l[i][m] = 0.0f; }
+                for (int m = 0; m < 4; ++m) {
+                    if (k <= r0) abs_mac(b[0][m], x0, at(v, m));
+                    abs_mac(b[1][m], x1, at(v, m));
+                }
+            }
         }
+        unit_base(b, h, l);
         for (int k = 0; k < K; k += 4) unit_nn(h, l, ld4(A[r0] + k), ld4(A[r0 + 1] + k), B[k] + c0, B.ld);
         if (T.p) {
             int k = 0;
@@ -401,6 +412,7 @@ __device__ __forceinline__ void prod_nn(const Rows &A, int rows, const Rows &B, 
                 }
             }
         }
+        unit_unbase(h, b);
         done(r0, c0, h, l);
     }
 }
@@ -433,30 +445,66 @@ __device__ __forceinline__ void prod_nn_plain(const Rows &A, int rows, const Row
 // out(r, f) = init(r, f) + sum_{k < K} A[r][k] B[f][k] + (second sum) for f < F: a unit is rows r0, r0 + 1 and the
 // four f of f0, f0 + F4, f0 + 2 F4, f0 + 3 F4 (F4 = ceil(F / 4)), so that consecutive lanes read consecutive rows
 // of B.  The second sum runs over the rows k of B2: of A2[r][k] B2[k][f] for k <= r (Lower), or of
-// A2[k][r] B2[k][f] for r <= k < k2 (Upper), with A2 lower triangular.  Row r's sums start at base(r);
-// init(r, f, h, l) adds to them, and done(r, f, h, l) gets them without the start, for f < F.
+// A2[k][r] B2[k][f] for r <= k < k2 (Upper), with A2 lower triangular.  init(r, f, h, l) sets a pair (0 before);
+// done(r, f, h, l) gets the sums, for f < F.
 enum Second { kNone, kLower, kUpper };
-template <Second MODE, typename Base, typename Init, typename Done>
+template <Second MODE, typename Init, typename Done>
 __device__ __forceinline__ void prod_nt(const Rows &A, int rows, const Rows &B, int F, int K, const Rows &A2,
-                                        const Rows &B2, int k2, Base base, Init init, Done done) {
+                                        const Rows &B2, int k2, Init init, Done done) {
     const int F4 = (F + 3) / 4, nu = ((rows + 1) / 2) * F4;
     const Div by(F4);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
         const int g = by(u), r0 = 2 * g, f0 = u - g * F4;
-        float h[2][4], l[2][4];
-        const float start[2] = {base(r0), base(r0 + 1)};
         int f[4];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            f[m] = min(f0 + m * F4, F - 1);
+        for (int m = 0; m < 4; ++m) f[m] = min(f0 + m * F4, F - 1);
+        const float *a0 = A[r0], *a1 = A[r0 + 1];
+        float h[2][4], l[2][4], b[2][4] = {};
+        for (int k = 0; k < K; k += 4) {
+            const float4 x0 = ld4(a0 + k), x1 = ld4(a1 + k);
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                h[i][m] = start[i];
-                l[i][m] = 0.0f;
-                init(r0 + i, f[m], h[i][m], l[i][m]);
+            for (int m = 0; m < 4; ++m) {
+                const float4 v = ld4(B[f[m]] + k);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    abs_mac(b[0][m], at(x0, kk), at(v, kk));
+                    abs_mac(b[1][m], at(x1, kk), at(v, kk));
+                }
             }
         }
-        const float *a0 = A[r0], *a1 = A[r0 + 1];
+        if (MODE == kLower) {
+            for (int k = 0; k <= r0 + 1 && k < k2; ++k) {
+                const float x0 = A2[r0][k], x1 = A2[r0 + 1][k];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float v = B2[k][f[m]];
+                    if (k <= r0) abs_mac(b[0][m], x0, v);
+                    abs_mac(b[1][m], x1, v);
+                }
+            }
+        }
+        if (MODE == kUpper) {
+            for (int k = r0; k < k2; ++k) {
+                const float2 x = *reinterpret_cast<const float2 *>(A2[k] + r0);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float v = B2[k][f[m]];
+                    abs_mac(b[0][m], x.x, v);
+                    if (k > r0) abs_mac(b[1][m], x.y, v);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                float ih = 0.0f, il = 0.0f;
+                init(r0 + i, f[m], ih, il);
+                b[i][m] = pair_base(b[i][m] + fabsf(ih));
+                h[i][m] = b[i][m];
+                l[i][m] = il;
+                pair_mac(h[i][m], l[i][m], ih, 1.0f);
+            }
         for (int k = 0; k < K; k += 4) {
             const float4 x0 = ld4(a0 + k), x1 = ld4(a1 + k);
 #pragma unroll
@@ -491,34 +539,56 @@ __device__ __forceinline__ void prod_nt(const Rows &A, int rows, const Rows &B, 
                 }
             }
         }
+        unit_unbase(h, b);
 #pragma unroll
         for (int m = 0; m < 4; ++m)
 #pragma unroll
             for (int i = 0; i < 2; ++i)
-                if (f0 + m * F4 < F) done(r0 + i, f[m], __fsub_rn(h[i][m], start[i]), l[i][m]);
+                if (f0 + m * F4 < F) done(r0 + i, f[m], h[i][m], l[i][m]);
     }
 }
 
 // Lower triangle of A B^T for the rows of a tile: S[r][j] for j <= r < rows, 0 above the diagonal, in row `rows`
-// of an odd count and in the columns up to a multiple of 4.  PAIR: as pairs from base(r), changed by add(r, h, l),
-// rounded once; else one plain fma chain over k in order.
-template <bool PAIR, typename Base, typename Add>
-__device__ __forceinline__ void scores_lower(const Rows &A, const Rows &B, int rows, int K, const Rows &S, Base base,
-                                             Add add) {
+// of an odd count and in the columns up to a multiple of 4.  PAIR: as pairs from init(r, h, l), rounded once; else
+// one plain fma chain over k in order.
+template <bool PAIR, typename Init>
+__device__ __forceinline__ void scores_lower(const Rows &A, const Rows &B, int rows, int K, const Rows &S, Init init) {
     const int F4 = (rows + 3) / 4, nu = ((rows + 1) / 2) * F4;
     const Div by(F4);
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
         const int g = by(u), r0 = 2 * g, f0 = u - g * F4;
-        float h[2][4], l[2][4], start[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            start[i] = PAIR ? base(r0 + i) : 0.0f;
-#pragma unroll
-            for (int m = 0; m < 4; ++m) { h[i][m] = start[i]; l[i][m] = 0.0f; }
-        }
+        float h[2][4] = {}, l[2][4] = {}, b[2][4] = {};
         const int nm = f0 <= r0 + 1 ? min(4, (r0 + 1 - f0) / F4 + 1) : 0;  // columns at or below the diagonal
+        const float *a0 = A[r0], *a1 = A[r0 + 1];
+        if (PAIR && nm) {
+            for (int k = 0; k < K; k += 4) {
+                const float4 x0 = ld4(a0 + k), x1 = ld4(a1 + k);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    if (m < nm) {
+                        const float4 v = ld4(B[f0 + m * F4] + k);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            abs_mac(b[0][m], at(x0, kk), at(v, kk));
+                            abs_mac(b[1][m], at(x1, kk), at(v, kk));
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float ih = 0.0f, il = 0.0f;
+                init(r0 + i, ih, il);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    b[i][m] = pair_base(b[i][m] + fabsf(ih));
+                    h[i][m] = b[i][m];
+                    l[i][m] = il;
+                    pair_mac(h[i][m], l[i][m], ih, 1.0f);
+                }
+            }
+        }
         if (nm) {
-            const float *a0 = A[r0], *a1 = A[r0 + 1];
             for (int k = 0; k < K; k += 4) {
                 const float4 x0 = ld4(a0 + k), x1 = ld4(a1 + k);
 #pragma unroll
@@ -546,51 +616,62 @@ __device__ __forceinline__ void scores_lower(const Rows &A, const Rows &B, int r
             for (int i = 0; i < 2; ++i) {
                 const int r = r0 + i;
                 float v = 0.0f;
-                if (j <= r && r < rows) {
-                    if (PAIR) {
-                        add(r, h[i][m], l[i][m]);
-                        v = pair_value(h[i][m] - start[i], l[i][m]);
-                    } else {
-                        v = h[i][m];
-                    }
-                }
+                if (j <= r && r < rows) v = PAIR ? pair_value(__fsub_rn(h[i][m], b[i][m]), l[i][m]) : h[i][m];
                 S[r][j] = v;
             }
         }
     }
 }
 
-// Rows r of A (TF values at a) times rows r of B (TC values at b) over a tile, added to the pairs h, l.
-template <int TF, int TC>
-__device__ __forceinline__ void outer_rows(float (&h)[TF][TC], float (&l)[TF][TC], const float *a, int lda,
-                                           const float *b, int ldb, int nr) {
+// sum_{r < nr} A[r][f] B[r][c] of two f (values at a, row stride lda) and four c (at b) as pairs.
+__device__ __forceinline__ void outer_rows(float (&h)[2][4], float (&l)[2][4], const float *a, int lda, const float *b,
+                                           int ldb, int nr) {
+    float s[2][4] = {};
+#pragma unroll 4
+    for (int r = 0; r < nr; ++r) {
+        const float2 x = *reinterpret_cast<const float2 *>(a + r * lda);
+        const float4 y = ld4(b + r * ldb);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            abs_mac(s[0][m], x.x, at(y, m));
+            abs_mac(s[1][m], x.y, at(y, m));
+        }
+    }
+    unit_base(s, h, l);
 #pragma unroll 2
     for (int r = 0; r < nr; ++r) {
-        float x[TF], y[TC];
-        if constexpr (TF == 2) {
-            const float2 v = *reinterpret_cast<const float2 *>(a + r * lda);
-            x[0] = v.x; x[1] = v.y;
-        } else {
-            const float4 v = ld4(a + r * lda);
+        const float2 x = *reinterpret_cast<const float2 *>(a + r * lda);
+        const float4 y = ld4(b + r * ldb);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = at(v, i);
+        for (int m = 0; m < 4; ++m) {
+            pair_mac(h[0][m], l[0][m], x.x, at(y, m));
+            pair_mac(h[1][m], l[1][m], x.y, at(y, m));
         }
-#pragma unroll
-        for (int q = 0; q < TC / 4; ++q) {
-            const float4 v = ld4(b + r * ldb + 4 * q);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) y[4 * q + m] = at(v, m);
-        }
-#pragma unroll
-        for (int i = 0; i < TF; ++i)
-#pragma unroll
-            for (int m = 0; m < TC; ++m) pair_mac(h[i][m], l[i][m], x[i], y[m]);
     }
+    unit_unbase(h, s);
+}
+
+// (h, l) = sum_{r < nr} A[r][f] (w, wl)[r] (w null: 1) for the column at a.
+__device__ __forceinline__ void column_sum(float &h, float &l, const float *a, int lda, const float *w, const float *wl,
+                                           int nr) {
+    float s = 0.0f;
+#pragma unroll 4
+    for (int r = 0; r < nr; ++r) abs_mac(s, a[r * lda], w ? w[r] : 1.0f);
+    s = pair_base(s);
+    h = s;
+    l = 0.0f;
+#pragma unroll 4
+    for (int r = 0; r < nr; ++r) {
+        const float x = a[r * lda];
+        pair_mac(h, l, x, w ? w[r] : 1.0f);
+        if (w) l = __fmaf_rn(x, wl[r], l);
+    }
+    h = __fsub_rn(h, s);
 }
 
 // Register accumulator of sum_r A[r][f] B[r][c] over every tile of a block: a thread owns TF x TC elements, the
-// smallest of 2 x 4, 4 x 4, 4 x 8 that covers D x dv with 512 threads.  A tile's sums start at base (z: zbase;
-// bounds of nr products) and are folded into the running pairs after it, so that no update loses its error.
+// smallest of 2 x 4, 4 x 4, 4 x 8 that covers D x dv with 512 threads, and forms them 2 x 4 at a time: the tile's
+// pairs and start values beside all the running ones.
 template <int TF, int TC>
 struct OuterAcc {
     float H[TF][TC], L[TF][TC];
@@ -604,34 +685,26 @@ struct OuterAcc {
     }
     // rows [0, nr); w, wl: weights of z as pairs (null: 1)
     __device__ __forceinline__ void add(const Rows &A, int D, const Rows &B, int dv, const float *w, const float *wl,
-                                        int nr, float base, float zbase) {
+                                        int nr) {
         const int nc = (dv + TC - 1) / TC;
         const int tf = threadIdx.x / nc, tc = threadIdx.x - tf * nc;
         if (tf * TF < D) {
 #pragma unroll
-            for (int q = 0; q < TC; q += 4) {  // four columns at a time: the tile's pairs beside all the running ones
-                float h[TF][4], l[TF][4];
+            for (int i = 0; i < TF; i += 2)
 #pragma unroll
-                for (int i = 0; i < TF; ++i)
+                for (int q = 0; q < TC; q += 4) {
+                    float h[2][4], l[2][4];
+                    outer_rows(h, l, A.p + tf * TF + i, A.ld, B.p + tc * TC + q, B.ld, nr);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) { h[i][m] = base; l[i][m] = 0.0f; }
-                outer_rows<TF, 4>(h, l, A.p + tf * TF, A.ld, B.p + tc * TC + q, B.ld, nr);
+                    for (int k = 0; k < 2; ++k)
 #pragma unroll
-                for (int i = 0; i < TF; ++i)
-#pragma unroll
-                    for (int m = 0; m < 4; ++m)
-                        pair_add(H[i][q + m], L[i][q + m], __fsub_rn(h[i][m], base), l[i][m]);
-            }
+                        for (int m = 0; m < 4; ++m) pair_add(H[i + k][q + m], L[i + k][q + m], h[k][m], l[k][m]);
+                }
         }
         if ((int)threadIdx.x < D) {
-            float h = zbase, l = 0.0f;
-#pragma unroll 4
-            for (int r = 0; r < nr; ++r) {
-                const float x = A[r][threadIdx.x];
-                pair_mac(h, l, x, w ? w[r] : 1.0f);
-                if (w) l = __fmaf_rn(x, wl[r], l);
-            }
-            pair_add(zh, zl, __fsub_rn(h, zbase), l);
+            float h, l;
+            column_sum(h, l, A.p + threadIdx.x, A.ld, w, wl, nr);
+            pair_add(zh, zl, h, l);
         }
     }
     // The sums of partial `slot` at S [slot][D][dv], z [slot][D], rounded; with `pairs`, high and low parts at
@@ -658,20 +731,14 @@ struct OuterAcc {
 };
 
 // S[f][c] += sum_{r < nr} A[r][f] B[r][c] and z[f] += sum_r A[r][f] (w, wl)[r] (null: 1) in shared memory, each rounded
-// once; the tile's sums start at base and zbase as in OuterAcc.  The running state loses half an ulp per tile.
-// slots (or null): the largest |S| and |z| after it, as for block_max.
+// once.  The running state loses half an ulp per tile.
 __device__ void advance_rows(const Rows &S, float *z, const Rows &A, int D, const Rows &B, int dv, const float *w,
-                             const float *wl, int nr, float base, float zbase, unsigned *slots) {
-    float mS = 0.0f, mz = 0.0f;
+                             const float *wl, int nr) {
     const int ng = (dv + 3) / 4, nu = ((D + 1) / 2) * ng;
     for (int u = threadIdx.x; u < nu; u += blockDim.x) {
         const int g = u / ng, f0 = 2 * g, c0 = 4 * (u - g * ng);
         float h[2][4], l[2][4];
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int m = 0; m < 4; ++m) { h[i][m] = base; l[i][m] = 0.0f; }
-        outer_rows<2, 4>(h, l, A.p + f0, A.ld, B.p + c0, B.ld, nr);
+        outer_rows(h, l, A.p + f0, A.ld, B.p + c0, B.ld, nr);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const float4 v = ld4(S[f0 + i] + c0);
@@ -679,29 +746,17 @@ __device__ void advance_rows(const Rows &S, float *z, const Rows &A, int D, cons
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 float H = at(v, m), L = 0.0f;
-                pair_add(H, L, __fsub_rn(h[i][m], base), l[i][m]);
+                pair_add(H, L, h[i][m], l[i][m]);
                 o[m] = pair_value(H, L);
             }
-            const float4 nv = make_float4(o[0], o[1], o[2], o[3]);
-            st4(S[f0 + i] + c0, nv);
-            mS = max4(nv, mS);
+            st4(S[f0 + i] + c0, make_float4(o[0], o[1], o[2], o[3]));
         }
     }
     if ((int)threadIdx.x < D) {
-        float h = zbase, l = 0.0f, H = z[threadIdx.x], L = 0.0f;
-#pragma unroll 4
-        for (int r = 0; r < nr; ++r) {
-            const float x = A[r][threadIdx.x];
-            pair_mac(h, l, x, w ? w[r] : 1.0f);
-            if (w) l = __fmaf_rn(x, wl[r], l);
-        }
-        pair_add(H, L, __fsub_rn(h, zbase), l);
-        mz = pair_value(H, L);
-        z[threadIdx.x] = mz;
-    }
-    if (slots) {
-        block_max(mS, slots);
-        block_max(fabsf(mz), slots + 1);
+        float h, l, H = z[threadIdx.x], L = 0.0f;
+        column_sum(h, l, A.p + threadIdx.x, A.ld, w, wl, nr);
+        pair_add(H, L, h, l);
+        z[threadIdx.x] = pair_value(H, L);
     }
 }
 
@@ -745,7 +800,6 @@ __device__ __forceinline__ void pair_quot(float h, float l, float dh, float dl, 
 struct RowPairs {
     float *dh, *dl, *inv;  // den (and 1 / dh)
     float *gh, *gl;        // dden
-    float *bp, *bq;        // starts of the row's sums of dP and dphi
     __device__ __forceinline__ void set_den(int r, float h, float l, float eps) const {
         pair_mac_any(h, l, eps, 1.0f);
         const float v = pair_value(h, l);
@@ -763,10 +817,9 @@ struct RowPairs {
         gh[r] = v;
         gl[r] = fabsf(v) < INFINITY ? __fadd_rn(__fsub_rn(qh, v), ql) : 0.0f;
     }
-    // rows [0, nr) of dO divided by den, each element rounded once, in place; returns this thread's largest |value|
-    __device__ __forceinline__ float divide_rows(const Rows &dO, int nr, int cols) const {
+    // rows [0, nr) of dO divided by den, each element rounded once, in place
+    __device__ __forceinline__ void divide_rows(const Rows &dO, int nr, int cols) const {
         const Div by((cols + 3) / 4);
-        float m = 0.0f;
 #pragma unroll 2
         for (int e = threadIdx.x; e < nr * by.n; e += blockDim.x) {
             const int r = by(e);
@@ -781,23 +834,20 @@ struct RowPairs {
                 x[k] = den != 0.0f ? pair_value(qh, ql) : 0.0f;
             }
             st4(p, v);
-            m = max4(v, m);
         }
-        return m;
     }
 };
 __device__ RowPairs take_row_pairs(Carve &cv, int cap) {
     RowPairs p;
     p.dh = cv.take(cap); p.dl = cv.take(cap); p.inv = cv.take(cap); p.gh = cv.take(cap); p.gl = cv.take(cap);
-    p.bp = cv.take(cap); p.bq = cv.take(cap);
     return p;
 }
-void take_row_pairs_host(HostCarve &cv, int cap) { for (int k = 0; k < 7; ++k) cv.take(cap); }
+void take_row_pairs_host(HostCarve &cv, int cap) { for (int k = 0; k < 5; ++k) cv.take(cap); }
 
-// A unit's share of sum_c dnum_c num_c of its two rows (num: the sums of prod_nn, which started at base) as pairs at
-// P[r][2 g], P[r][2 g + 1], g the unit's column group; rows < nr.
+// A unit's share of sum_c dnum_c num_c of its two rows (num: the sums of prod_nn) as pairs at P[r][2 g],
+// P[r][2 g + 1], g the unit's column group; rows < nr.
 __device__ __forceinline__ void unit_dots(const Rows &dnum, const Rows &P, int nr, int r0, int c0, const float (&h)[2][4],
-                                          const float (&l)[2][4], float base) {
+                                          const float (&l)[2][4]) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         if (r0 + i >= nr) continue;
@@ -805,7 +855,7 @@ __device__ __forceinline__ void unit_dots(const Rows &dnum, const Rows &P, int n
         float ph = 0.0f, pl = 0.0f;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            pair_mac_any(ph, pl, at(g, m), __fsub_rn(h[i][m], base));
+            pair_mac_any(ph, pl, at(g, m), h[i][m]);
             pl = __fmaf_rn(at(g, m), l[i][m], pl);
         }
         *reinterpret_cast<float2 *>(P[r0 + i] + c0 / 2) = make_float2(ph, pl);
@@ -875,38 +925,25 @@ __device__ void zero_words(float *p, int n) {
     for (int e = threadIdx.x; e < n; e += blockDim.x) p[e] = 0.0f;
 }
 
-// The fp32 state [D][dv] into rows of shared memory (zeros in the pads), z beside it.  slots (or null): the largest
-// |S| and |z|, as for block_max.
-__device__ void load_state(const Rows &S, float *z, const float *gS, const float *gz, int D, int dv, unsigned *slots) {
+// The fp32 state [D][dv] into rows of shared memory (zeros in the pads), z beside it.
+__device__ void load_state(const Rows &S, float *z, const float *gS, const float *gz, int D, int dv) {
     const int Dp = (D + 3) & ~3;
-    float mS = 0.0f, mz = 0.0f;
     if (dv % 4 == 0 && (reinterpret_cast<uintptr_t>(gS) & 15) == 0) {
         const Div q(dv / 4);
 #pragma unroll 4
         for (int e = threadIdx.x; e < D * q.n; e += blockDim.x) {
             const int f = q(e), c = 4 * (e - f * q.n);
-            const float4 v = ld4(gS + 4 * e);
-            st4(S[f] + c, v);
-            mS = max4(v, mS);
+            st4(S[f] + c, ld4(gS + 4 * e));
         }
     } else {
         const int wp = (dv + 3) & ~3;
         for (int e = threadIdx.x; e < D * wp; e += blockDim.x) {
             const int f = e / wp, c = e - f * wp;
-            const float v = c < dv ? gS[f * dv + c] : 0.0f;
-            S[f][c] = v;
-            mS = v == v ? fmaxf(mS, fabsf(v)) : INFINITY;
+            S[f][c] = c < dv ? gS[f * dv + c] : 0.0f;
         }
     }
     for (int e = threadIdx.x; e < (Dp - D) * S.ld; e += blockDim.x) S[D][e] = 0.0f;
-    for (int f = threadIdx.x; f < D; f += blockDim.x) {
-        z[f] = gz[f];
-        mz = fmaxf(mz, fabsf(gz[f]));
-    }
-    if (slots) {
-        block_max(mS, slots);
-        block_max(mz, slots + 1);
-    }
+    for (int f = threadIdx.x; f < D; f += blockDim.x) z[f] = gz[f];
 }
 
 // ---------------------------------------------------------------------------

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kThr, 2) k_weights(AttnArgs a, int causal, int
     if (!teacher) load_phi_tile(s, lay, a.table + (size_t)(bh % a.H) * tstride);  // this head's table
     load_tile(teacher ? sQ : sX, Qh + (size_t)i_lo * d, nq, d, kW);
     __syncthreads();
-    if (!teacher) phi_rows(lay, s, sX, nq, kW, sQ, nullptr, nullptr, nullptr);
+    if (!teacher) phi_rows(lay, s, sX, nq, kW, sQ, nullptr, nullptr);
     // thread: rows 2g, 2g + 1, columns f0 + 16 m of every key tile
     const int r0 = 2 * (threadIdx.x / 16), f0 = threadIdx.x % 16, K = ((teacher ? d : D) + 3) & ~3;
     const int jend = causal ? min(i_lo + nq, len) : len;  // keys the block needs
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kThr, 2) k_weights(AttnArgs a, int causal, int
             load_tile(sX, Kh + (size_t)j0 * d, nk, d, kW);
             __syncthreads();
             if (!teacher) {
-                phi_rows(lay, s, sX, nk, kW, sP, nullptr, nullptr, nullptr);
+                phi_rows(lay, s, sX, nk, kW, sP, nullptr, nullptr);
                 __syncthreads();
             }
             const float *q0 = sQ[r0], *q1 = sQ[r0 + 1], *p = sP[f0];

@@ -1,0 +1,47 @@
+"""GPU: the sums of the CUDA-core kernels are as good at every scale of their operands.
+
+The statistics, normalisers and feature gradients are sums of cancelling terms, carried as pairs of floats and
+rounded once.  How many bits such a sum keeps must depend on its own terms alone, not on what else its tile holds.
+"""
+import math
+
+import numpy as np
+import pytest
+
+from cases import Case, to_device, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2512_08061_gb300 import build
+    build.build()
+
+
+def _case(n, d, dv, M, L, causal, seed):
+    return Case(1, 2, n, d, M, L, "f32", causal, seed=seed, qkv_scale=1.0 / math.sqrt(d), dv=dv, with_grad=True)
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("n,d,dv,M,L", [(150, 32, 32, 8, 8), (200, 64, 96, 8, 8), (70, 20, 33, 3, 5)])
+def test_sums_do_not_depend_on_other_columns(n, d, dv, M, L, causal):
+    """Columns of V scaled by 2^-18 and 2^-6 with the columns of dO scaled by the inverse: every product of a column
+    of V and one of dO, and every power of two, stays exact, so dQ and dK keep their bits, and so do O and dV
+    after their own scale."""
+    case = _case(n, d, dv, M, L, causal, 211)
+    lu = case.luna()
+    O, g = case.run_fwd(lu), case.run_bwd(lu)
+    plain = {"O": to_host(O), **{k: to_host(g[k]) for k in ("dQ", "dK", "dV")}}
+    import torch
+    scale = torch.tensor([2.0 ** (-18, 0, -6)[c % 3] for c in range(dv)], dtype=torch.float32, device="cuda")
+    case.dev["V"] = case.dev["V"] * scale
+    case.dev["dO"] = case.dev["dO"] / scale
+    O, g = case.run_fwd(lu), case.run_bwd(lu)
+    s = to_host(scale)
+    got = {"O": to_host(O) / s, "dQ": to_host(g["dQ"]), "dK": to_host(g["dK"]), "dV": to_host(g["dV"]) * s}
+    for k, v in plain.items():
+        assert np.array_equal(got[k], v), (k, int((got[k] != v).sum()))
