@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
         scores_lower<false>(sPq, sPk, nr, Dp, sA, [](int, float &, float &) {});
         scores_lower<true>(sdO, sV, nr, dvp, sP, [&](int r, float &h, float &l) { h = rp.gh[r]; l = rp.gl[r]; });
         __syncthreads();
-        prod_nn_plain(sPk, nr, G, Dp, dv, sA, sdO, nr, [&](int q0, int c0, const float (&h)[2][4]) {
+        prod_nn_chains(sPk, nr, G, Dp, dv, sA, sdO, nr, [&](int q0, int c0, const float (&h)[2][4]) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
                 if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);

@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kThr, 1) k_query(AttnArgs a, int cap, int rows
                      sden[r] = pair_value(h, l);
                  });
         __syncthreads();
-        prod_nn_plain(sPhi, nr, sS, Dp, dv, none, none, 0, [&](int r0, int c0, const float (&h)[2][4]) {
+        prod_nn_plain(sPhi, nr, sS, Dp, dv, [&](int r0, int c0, const float (&h)[2][4]) {
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 if (r0 + i >= nr) continue;
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nb
         __syncthreads();
         phi_rows(lay, s, sK, nr, cap, sPhi, sU, sJ);
         __syncthreads();
-        prod_nn_plain(sPhi, nr, sdS, Dp, dv, none, none, 0, [&](int q0, int c0, const float (&h)[2][4]) {
+        prod_nn_plain(sPhi, nr, sdS, Dp, dv, [&](int q0, int c0, const float (&h)[2][4]) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
                 if (q0 + i < nr) store4(dV + (size_t)(t0 + q0 + i) * dv + c0, h[i], dv - c0, vec);
