@@ -991,7 +991,8 @@ __device__ void load_state(const Rows &S, float *z, const float *gS, const float
 // Backward through phi for a tile.
 
 // dW of a block: a thread owns rows i0, i0 + 1 and columns c0 .. c0 + 3 of the M x d matrix, over every G-th row
-// of the tiles (G = 512 / tiles of 2 x 4).
+// of the tiles (G = 512 / tiles of 2 x 4).  The sums cancel and run from zero over the whole block, so every
+// product is added exactly whatever its size: with pair_mac they kept 40 bits of sum |dU x| and not 46.
 struct GradTile {
     float h[2][4], l[2][4];
     float bh, bl;  // thread i < M: db
@@ -1197,8 +1198,8 @@ __device__ void phi_backward_rows(const TableLayout &lay, const SmemPhi &s, cons
             const float4 x = ld4(X[r] + c0);
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                pair_mac(g.h[0][m], g.l[0][m], a.x, at(x, m));
-                pair_mac(g.h[1][m], g.l[1][m], a.y, at(x, m));
+                pair_mac_any(g.h[0][m], g.l[0][m], a.x, at(x, m));
+                pair_mac_any(g.h[1][m], g.l[1][m], a.y, at(x, m));
             }
         }
     }

@@ -60,3 +60,25 @@ def test_streaming_outputs_are_no_further_off_than_fp64_sums():
         for k in err:
             err[k].append(math.sqrt(np.mean((got[k] - ref[k]) ** 2) / np.mean(ref[k] ** 2)))
     assert np.mean(err["O"]) < 6.8e-8 and np.mean(err["dV"]) < 1.27e-7, err
+
+
+@pytest.mark.parametrize("causal", [False, True])
+def test_projection_gradients_are_the_sums_of_their_rows(causal):
+    """With W the identity, dX = dU W returns each row's dU, so dW = sum_rows dU x^T and db = sum_rows dU over Q and K
+    can be formed on the host in 64 bits from the call's own dQ and dK.  Half an ulp for the result's rounding, and
+    2^-42 of the terms' sizes for the pairs: their low parts are sums of at most 500 roundings of 2^-25, rounded at
+    2^-25 in turn (sqrt(500) 2^-50 of the sizes if these are independent), and a margin of eight."""
+    import synth
+    d, n = 8, 500
+    params = synth.phi_params(227, d, d, 8, 64)
+    params["W"], params["b"] = np.eye(d, dtype=np.float32), np.zeros(d, np.float32)
+    case = Case(2, 2, n, d, d, 8, "f32", causal, seed=227, params=params, with_grad=True)
+    lu = case.luna()
+    case.run_fwd(lu)
+    g = {k: to_host(v) for k, v in case.run_bwd(lu).items()}
+    x = {k: case.inp[k].value.reshape(-1, d) for k in ("Q", "K")}
+    du = {k: g["d" + k].reshape(-1, d) for k in ("Q", "K")}
+    for key, ref, size in (("dW", sum(du[k].T @ x[k] for k in x), sum(abs(du[k]).T @ abs(x[k]) for k in x)),
+                           ("db", sum(du[k].sum(0) for k in x), sum(abs(du[k]).sum(0) for k in x))):
+        half_ulp = np.spacing(abs(g[key]).astype(np.float32)).astype(np.float64) / 2
+        assert (abs(g[key] - ref) <= half_ulp + 2.0 ** -42 * size).all(), key
