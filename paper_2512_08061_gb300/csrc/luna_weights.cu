@@ -15,7 +15,8 @@
 // writes the raw scores (the kernel values, or the scaled dot products) and
 // accumulates each row's sum (LUNA, as a pair of floats) or its running maximum
 // and rescaled exponential sum (teacher); pass 2 rereads the thread's own
-// entries, from L2, and normalises them.  No scratch memory.  Measured at 48
+// entries, from L2, and normalises them.  A NaN score of the teacher makes the
+// row's sum NaN and its scale 0, whichever tile holds it.  No scratch memory.  Measured at 48
 // heads of 512 x 512, d = D = 64: kernel weights 1590 -> 158 us, teacher 1202 ->
 // 114 us against one score per thread from scalar shared loads.
 #include <math.h>
@@ -108,13 +109,14 @@ __global__ void __launch_bounds__(kThr, 2) k_weights(AttnArgs a, int causal, int
                 } else if (teacher) {
                     h[i][m] *= qscale;
                     if (h[i][m] > m2) m2 = h[i][m];
+                    if (h[i][m] != h[i][m]) es[i] = h[i][m];  // a NaN score: the row's sum is NaN from here on
                 } else {
                     pair_mac_any(sh[i], sl[i], h[i][m], 1.0f);
                 }
                 if (j < n) Ar[(size_t)i * n + j] = h[i][m];
             }
             if (teacher && m2 > -INFINITY) {
-                float e = es[i] > 0.0f ? es[i] * expf(mx[i] - m2) : 0.0f;
+                float e = es[i] * expf(mx[i] - m2);
 #pragma unroll
                 for (int m = 0; m < 4; ++m)
                     if (j0 + f0 + 16 * m < jmax[i]) e += expf(h[i][m] - m2);
@@ -132,7 +134,8 @@ __global__ void __launch_bounds__(kThr, 2) k_weights(AttnArgs a, int causal, int
             if (teacher) {
                 const float m2 = __shfl_xor_sync(0xffffffffu, mx[i], o), e2 = __shfl_xor_sync(0xffffffffu, es[i], o);
                 const float m = fmaxf(mx[i], m2);
-                es[i] = (m == -INFINITY) ? 0.0f : es[i] * expf(mx[i] - m) + e2 * expf(m2 - m);
+                // (no maximum yet: both sums are 0, or NaN)
+                es[i] = (m == -INFINITY) ? es[i] + e2 : es[i] * expf(mx[i] - m) + e2 * expf(m2 - m);
                 mx[i] = m;
             } else {
                 const float h2 = __shfl_xor_sync(0xffffffffu, sh[i], o), l2 = __shfl_xor_sync(0xffffffffu, sl[i], o);
