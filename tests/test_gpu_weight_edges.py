@@ -47,3 +47,17 @@ def test_nan_score_reaches_its_row(key, causal):
     assert (np.delete(got[sees], key, axis=1) == 0).all()
     if not sees.all():
         assert relerr(got[~sees], ref[0, 0][~sees]) < TOL["f32"]
+
+
+@pytest.mark.parametrize("n,d,M,L,io,causal,row0,rows", [
+    (1, 64, 8, 8, "f32", False, 0, 1), (4, 20, 3, 5, "f32", True, 1, 3), (31, 64, 8, 8, "bf16", True, 0, 31),
+    (32, 33, 2, 8, "f32", False, 0, 32), (32, 128, 16, 8, "bf16", False, 30, 2), (33, 64, 8, 8, "f32", True, 0, 33)])
+@pytest.mark.parametrize("teacher", [False, True])
+def test_short_sequences(n, d, M, L, io, causal, row0, rows, teacher):
+    """Sequences of one small tile: at, below and above the size where the tile changes."""
+    case = Case(3, 2, n, d, M, L, io, causal, seed=233, qkv_scale=1.0 / math.sqrt(d), lengths=[n, max(1, n // 2), 1])
+    ref = oracle.attn_weights(case.params, case.inp["Q"].value, case.inp["K"].value, case.lengths, causal, case.eps,
+                              row0, rows, teacher)
+    got = _weights(case, case.luna(), teacher, row0, rows)
+    assert ((got == 0) == (ref == 0)).all()
+    assert relerr(got, ref) < TOL[io]
