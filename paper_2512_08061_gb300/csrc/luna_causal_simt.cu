@@ -405,7 +405,7 @@ cudaError_t causal_bwd_impl(const AttnArgs &a0, bool have_state, cudaStream_t s)
 }  // namespace
 
 size_t causal_max_smem(const AttnArgs &a) {
-    return std::max(smem_out(a, kMinC), std::max(smem_bwd_query(a, kMinC), smem_bwd_key(a, kMinC)));
+    return std::max(smem_out(a, kMinC), std::max(smem_bwd_query(a, kMinC), smem_bwd_key(a, kMinC))) + kStaticSmem;
 }
 
 cudaError_t launch_causal_fwd(const AttnArgs &a, luna_dtype io, bool, cudaStream_t s) {

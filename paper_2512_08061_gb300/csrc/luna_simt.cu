@@ -741,7 +741,7 @@ size_t simt_max_smem(const AttnArgs &a) {
     size_t m = smem_keystats(a, kMinC);
     m = std::max(m, smem_query(a, kMinC));
     m = std::max(m, smem_bwd_query(a, kMinC));
-    return std::max(m, smem_bwd_key(a, kMinC));
+    return std::max(m, smem_bwd_key(a, kMinC)) + kStaticSmem;
 }
 
 cudaError_t launch_grad_reduce(const AttnArgs &a, int nparts, cudaStream_t s) {

@@ -22,7 +22,11 @@ constexpr int kMaxC = 64;   // rows per tile at most
 constexpr int kMinC = 8;    // and at least (every tile is a multiple of 8 rows)
 constexpr int kSlack = 8;   // floats after the last tile: an 8-column read of its last row may pass its end
 constexpr int kSMs = 152;
-constexpr size_t kSmemLimit = 227 * 1024;
+// Shared memory of a block for the arrays of a tile: 227 KB less what the kernels hold statically (last_arrival's flag,
+// the 128 bytes of channel sums of k_causal_bwd_query).  A launch whose static and dynamic parts exceed 227 KB is
+// refused, so tiles are chosen, and shapes accepted, by this limit.
+constexpr size_t kStaticSmem = 256;
+constexpr size_t kSmemLimit = 227 * 1024 - kStaticSmem;
 
 // Row stride in floats of a tile of x columns: whole 16-byte words, an odd number of them, so that eight lanes
 // reading 16 bytes each from consecutive rows touch all 32 banks.
