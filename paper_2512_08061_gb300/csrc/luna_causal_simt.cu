@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_out(AttnArgs a, int cap) {
 //   dphi(q_i) = S_{before tile} dnum_i + z dden_i + sum_{j<=i in tile} dP_ij phi(k_j),  dP_ij = dnum_i . v_j + dden_i
 // den_i, dnum_i . num_i and dden_i are pairs (RowPairs); dP and dphi are pairs rounded once.
 template <typename IO, int TF, int TC>
-__global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int cap, int nbuf, int finish) {
+__global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int cap, int finish) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
@@ -140,8 +140,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
     __shared__ double sT[kMaxL];  // channel normalisation: the block's sums of phi . dphi per channel
     if ((int)threadIdx.x < kMaxL) sT[threadIdx.x] = 0.0;
     const size_t slot = (size_t)bh * a.nseg + seg;
-    double *gp = reinterpret_cast<double *>(a.gpart) + (slot % nbuf) * a.gsize;
-    double *hist = gp + M * d + M;
+    double *hist = a.gh + (slot % a.gh_n) * (a.gsize - M * d - M);
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = seg * a.seg_len, rend = min(a.n, r0 + a.seg_len), r1 = min(len, rend);
     IO *dQ = static_cast<IO *>(a.dQ) + head_rows(a, bh) * d;
@@ -212,9 +211,8 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
         phi_backward_rows(lay, s, sQ, nr, cap, sPq, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
-    __syncthreads();
     acc.store(D, dv, a.dS_part, a.dz_part, slot, false);
-    if (r0 < r1) add_grad_tile(lay, g, gp);
+    store_grad_tile(lay, g, smem, a.gw + slot * (M * d + M));
     if (a.ch_T && (int)threadIdx.x < a.L) a.ch_T[slot * a.L + threadIdx.x] = sT[threadIdx.x];
     if (finish && last_arrival(a.counters + a.B * a.H + bh, a.nseg)) {
         exclusive_scan(a.dS_part + (size_t)bh * a.nseg * D * dv, a.nseg, D * dv, a.seg_dS + (size_t)bh * a.nseg * D * dv,
@@ -228,7 +226,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_query(AttnArgs a, int ca
 //   dv_j = G^T phi(k_j) + sum_{i>=j in tile} A_ij dnum_i
 //   dphi(k_j) = G v_j + g + sum_{i>=j in tile} dP_ij phi(q_i)
 template <typename IO>
-__global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap, int nbuf) {
+__global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
@@ -249,20 +247,22 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
     float *sdU = cv.take(cap * du_stride(M));
     if (!carve_fits(cv, smem)) return;
     const int bh = blockIdx.y, seg = blockIdx.x;
-    double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nseg + seg) % nbuf) * a.gsize;
-    double *hist = gp + M * d + M;
+    const size_t slot = (size_t)bh * a.nseg + seg;
+    double *hist = a.gh + (slot % a.gh_n) * (a.gsize - M * d - M), *gw = a.gw + (a.gw_n / 2 + slot) * (M * d + M);
     const int len = head_length(a.lengths, bh / a.H, a.n);
     const int r0 = seg * a.seg_len, rend = min(a.n, r0 + a.seg_len), r1 = min(len, rend);
     IO *dK = static_cast<IO *>(a.dK) + head_rows(a, bh) * d;
     IO *dV = static_cast<IO *>(a.dV) + head_rows(a, bh) * dv;
     zero_rows(dK, max(r0, len), rend, d);
     zero_rows(dV, max(r0, len), rend, dv);
-    if (r1 <= r0) return;
+    if (r1 <= r0) {
+        for (int e = threadIdx.x; e < M * d + M; e += blockDim.x) gw[e] = 0.0;
+        return;
+    }
     zero_words(tiles, (int)(cv.p - tiles));
     load_phi_tile(s, lay, a.table);
-    const size_t so = (size_t)bh * a.nseg + seg;
     __syncthreads();
-    load_state(G, gz, a.seg_dS + so * D * dv, a.seg_dz + so * D, D, dv);
+    load_state(G, gz, a.seg_dS + slot * D * dv, a.seg_dz + slot * D, D, dv);
     const IO *Q = static_cast<const IO *>(a.Q) + head_rows(a, bh) * d;
     const IO *K = static_cast<const IO *>(a.K) + head_rows(a, bh) * d;
     const IO *V = static_cast<const IO *>(a.V) + head_rows(a, bh) * dv;
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kThr, 1) k_causal_bwd_key(AttnArgs a, int cap,
         phi_backward_rows(lay, s, sK, nr, cap, sPk, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dK + (size_t)t0 * d);
     }
-    add_grad_tile(lay, g, gp);
+    store_grad_tile(lay, g, smem, gw);
 }
 
 // ---------------------------------------------------------------------------
@@ -325,6 +325,7 @@ size_t smem_bwd_query(const AttnArgs &a, int cap) {
     cv.take(cap * std::max(row_stride(a.d), std::max(row_stride(a.dv), row_stride(a.D))));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
     cv.take(kSlack);
+    cv.at_least(kGradScratch);
     return cv.bytes();
 }
 size_t smem_bwd_key(const AttnArgs &a, int cap) {
@@ -335,6 +336,7 @@ size_t smem_bwd_key(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, cap); take_rows_host(cv, cap, cap);
     cv.take(cap * std::max(row_stride(a.d), row_stride(a.D)));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
+    cv.at_least(kGradScratch);
     return cv.bytes();
 }
 
@@ -366,19 +368,16 @@ cudaError_t causal_fwd_impl(const AttnArgs &a, cudaStream_t s) {
 template <typename IO>
 cudaError_t causal_bwd_impl(const AttnArgs &a0, bool have_state, cudaStream_t s) {
     AttnArgs a = a0;
-    a.gpart64 = 1;  // the generic kernels write fp64 parameter-gradient sums
     cudaError_t e;
     if (!have_state && (e = seg_stats<IO>(a, s)) != cudaSuccess) return e;
-    const int64_t blocks = (int64_t)a.B * a.H * a.nseg;
-    const int nbuf = grad_buffers(blocks, 2 * blocks);
-    if ((e = cudaMemsetAsync(a.gpart, 0, (size_t)nbuf * a.gsize * sizeof(double), s)) != cudaSuccess) return e;
+    if ((e = place_grads(a, (int64_t)a.B * a.H * a.nseg, s)) != cudaSuccess) return e;
     const dim3 grid(a.nseg, a.B * a.H);
     int cap = seg_cap(a, [&](int c) { return smem_bwd_query(a, c); });
     size_t sm = smem_bwd_query(a, cap);
     outer_dispatch(a.D, a.dv, [&](auto tf, auto tc) {
         auto k = k_causal_bwd_query<IO, decltype(tf)::value, decltype(tc)::value>;
         if ((e = set_smem(k, sm)) != cudaSuccess) return;
-        LUNA_LAUNCH("causal_bwd_query", k, grid, kThr, sm, s, a, cap, nbuf, a.nseg <= kFinishParts);
+        LUNA_LAUNCH("causal_bwd_query", k, grid, kThr, sm, s, a, cap, a.nseg <= kFinishParts);
         e = cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
@@ -392,9 +391,9 @@ cudaError_t causal_bwd_impl(const AttnArgs &a0, bool have_state, cudaStream_t s)
     cap = seg_cap(a, [&](int c) { return smem_bwd_key(a, c); });
     sm = smem_bwd_key(a, cap);
     if ((e = set_smem(k_causal_bwd_key<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("causal_bwd_key", k_causal_bwd_key<IO>, grid, kThr, sm, s, a, cap, nbuf);
+    LUNA_LAUNCH("causal_bwd_key", k_causal_bwd_key<IO>, grid, kThr, sm, s, a, cap);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int nparts = nbuf;
+    int nparts = 0;
     if (a.ch_sigma) {  // the scale term of the channel normalisation (kappa from the queries' T rows)
         a.ch_T_rows = a.B * a.H * a.nseg;
         if ((e = launch_chrms_backward(a, nparts, &nparts, s)) != cudaSuccess) return e;

@@ -5,8 +5,9 @@
 // does not specialise.  A block owns a range of rows of one head and walks it
 // in tiles of up to 64 rows (luna_tile.cuh); the statistics, normalisers and
 // feature gradients are pairs of floats rounded once.  Every cross-block sum of
-// S, z, dS, dz runs in a fixed order; the parameter gradients are fp64 sums by
-// L2 reductions, whose order varies in the last bits of the fp64 sum.
+// S, z, dS, dz, dW and db runs in a fixed order; the channel MLPs' gradients come
+// from fp64 histograms filled by L2 reductions, whose order varies in the last
+// bits of the fp64 sums.
 //
 // Measured at 8 x 12 heads of 512 fp32 rows, d = D = 64 (us; before: fp64 sums in
 // tiles of 16 or 32 rows, 64 of 256 threads in the outer products):
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(kThr, 1) k_query(AttnArgs a, int cap, int rows
 //   dphi(q_i) = S dnum_i + z dden_i,  dS += phi(q_i) dnum_i^T,  dz += phi(q_i) dden_i
 // den, the sum dnum_i . num_i and dden are pairs (RowPairs), dphi is a pair rounded once.
 template <typename IO, int TF, int TC>
-__global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int nbuf, int finish) {
+__global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int finish) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
@@ -210,8 +211,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
     load_phi_tile(s, lay, a.table);
     const int bh = blockIdx.y, split = blockIdx.x;
     const size_t slot = (size_t)bh * a.nsplit_b + split;
-    double *gp = reinterpret_cast<double *>(a.gpart) + (slot % nbuf) * a.gsize;
-    double *hist = gp + M * d + M;
+    double *hist = a.gh + (slot % a.gh_n) * (a.gsize - M * d - M);
     __syncthreads();
     load_state(sS, sz, a.S_fin + head_state(a, bh) * D * dv, a.z_fin + head_state(a, bh) * D, D, dv);
 
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
         store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
     acc.store(D, dv, a.dS_part, a.dz_part, slot, true);
-    add_grad_tile(lay, g, gp);
+    store_grad_tile(lay, g, smem, a.gw + slot * (M * d + M));
     if (finish && last_arrival(a.counters + a.B * a.H + bh, a.nsplit_b)) {
         const int np = 2 * a.nsplit_b;
         ordered_sum(a.dS_part + (size_t)bh * np * D * dv, np, D * dv, a.dS_fin + (size_t)bh * D * dv);
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
 // key side of the backward pass (non-causal):
 //   dv_j = dS^T phi(k_j),  dphi(k_j) = dS v_j + dz
 template <typename IO>
-__global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nbuf) {
+__global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nb
     zero_words(tiles, (int)(cv.p - tiles));
     load_phi_tile(s, lay, a.table);
     const int bh = blockIdx.y, split = blockIdx.x;
-    double *gp = reinterpret_cast<double *>(a.gpart) + (((size_t)bh * a.nsplit_b + split) % nbuf) * a.gsize;
-    double *hist = gp + M * d + M;
+    const size_t slot = (size_t)bh * a.nsplit_b + split;
+    double *hist = a.gh + (slot % a.gh_n) * (a.gsize - M * d - M);
     __syncthreads();
     load_state(sdS, sdz, a.dS_fin + (size_t)bh * D * dv, a.dz_fin + (size_t)bh * D, D, dv);
 
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_key(AttnArgs a, int cap, int nb
         phi_backward_rows(lay, s, sK, nr, cap, sPhi, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dK + (size_t)t0 * d);
     }
-    add_grad_tile(lay, g, gp);
+    store_grad_tile(lay, g, smem, a.gw + (a.gw_n / 2 + slot) * (M * d + M));
 }
 
 // ---------------------------------------------------------------------------
@@ -391,48 +391,30 @@ struct CompSum {
     }
 };
 
-// Sum of the per-block parameter-gradient partials, in the fixed order p = 0..nparts-1
+// Sum of the per-block parameter-gradient partials of the tensor-core kernels, in the fixed order p = 0..nparts-1
 // per element: 64 elements per block, each summed by 8 threads over consecutive
-// eighths of the partials (8 loads in flight; fp32 partials in compensated fp32,
-// fp64 partials in fp64), then the eight parts combined in order in fp64.
+// eighths of the partials (8 loads in flight, compensated fp32), then the eight parts combined in order in fp64.
 constexpr int kSumElems = 64, kSumSplit = 8;
-template <typename P>
-__global__ void __launch_bounds__(kSumElems * kSumSplit) k_grad_sum(const P *gpart, int nparts, int gsize,
+__global__ void __launch_bounds__(kSumElems * kSumSplit) k_grad_sum(const float *gpart, int nparts, int gsize,
                                                                     double *out) {
     __shared__ double part[kSumSplit][kSumElems];
     grid_dependency_sync();
     const int el = threadIdx.x % kSumElems, q = threadIdx.x / kSumElems;
     const int e = blockIdx.x * kSumElems + el;
     const int p0 = (int)((long long)q * nparts / kSumSplit), p1 = (int)((long long)(q + 1) * nparts / kSumSplit);
-    if constexpr (sizeof(P) == 4) {
-        CompSum cs;
-        if (e < gsize) {
-            int p = p0;
-            for (; p + 8 <= p1; p += 8) {
-                float v[8];
+    CompSum cs;
+    if (e < gsize) {
+        int p = p0;
+        for (; p + 8 <= p1; p += 8) {
+            float v[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = __ldcg(gpart + (size_t)(p + k) * gsize + e);
+            for (int k = 0; k < 8; ++k) v[k] = __ldcg(gpart + (size_t)(p + k) * gsize + e);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) cs.add(v[k]);
-            }
-            for (; p < p1; ++p) cs.add(__ldcg(gpart + (size_t)p * gsize + e));
+            for (int k = 0; k < 8; ++k) cs.add(v[k]);
         }
-        part[q][el] = (double)cs.s + (double)cs.c;
-    } else {
-        double t = 0.0;
-        if (e < gsize) {
-            int p = p0;
-            for (; p + 8 <= p1; p += 8) {
-                double v[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = __ldcg(gpart + (size_t)(p + k) * gsize + e);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) t += v[k];
-            }
-            for (; p < p1; ++p) t += __ldcg(gpart + (size_t)p * gsize + e);
-        }
-        part[q][el] = t;
+        for (; p < p1; ++p) cs.add(__ldcg(gpart + (size_t)p * gsize + e));
     }
+    part[q][el] = (double)cs.s + (double)cs.c;
     __syncthreads();
     if (q == 0 && e < gsize) {
         double t = part[0][el];
@@ -440,6 +422,42 @@ __global__ void __launch_bounds__(kSumElems * kSumSplit) k_grad_sum(const P *gpa
         for (int k = 1; k < kSumSplit; ++k) t += part[k][el];
         out[e] = t;
     }
+}
+
+// Sums of the generic kernels' fp64 parameter gradients, in a fixed order: element e < nw over the gw_n slots, the
+// others over the gh_n histograms, and both over the `np` partials of the channel normalisation.  16 elements per
+// block, each by 32 threads over consecutive shares (there are up to 1216 slots, more with more heads).
+constexpr int kSum64Elems = 16, kSum64Split = 32;
+__global__ void __launch_bounds__(kSum64Elems * kSum64Split)
+    k_grad_sum64(const double *gw, int gw_n, const double *gh, int gh_n, const double *gpart, int np, int nw, int gsize,
+                 double *out) {
+    __shared__ double part[kSum64Split][kSum64Elems];
+    grid_dependency_sync();
+    const int el = threadIdx.x % kSum64Elems, q = threadIdx.x / kSum64Elems;
+    const int e = blockIdx.x * kSum64Elems + el;
+    double t = 0.0;
+    auto sum = [&](const double *x, int n, int step) {
+        const int p1 = (int)((long long)(q + 1) * n / kSum64Split);
+        int p = (int)((long long)q * n / kSum64Split);
+        for (; p + 8 <= p1; p += 8) {
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = __ldcg(x + (size_t)(p + k) * step);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) t += v[k];
+        }
+        for (; p < p1; ++p) t += __ldcg(x + (size_t)p * step);
+    };
+    if (e < nw) sum(gw + e, gw_n, nw);
+    else if (e < gsize) sum(gh + (e - nw), gh_n, gsize - nw);
+    if (e < gsize) sum(gpart + e, np, gsize);
+    part[q][el] = t;
+#pragma unroll
+    for (int o = kSum64Split / 2; o >= 1; o /= 2) {
+        __syncthreads();
+        if (q < o) part[q][el] += part[q + o][el];
+    }
+    if (q == 0 && e < gsize) out[e] = part[0][el];
 }
 
 // Inclusive scan of x[0..n) into y (forward: prefix sums; backward: suffix sums), accumulated in fp64,
@@ -610,6 +628,7 @@ size_t smem_bwd_query(const AttnArgs &a, int cap) {
     cv.take(cap * std::max(row_stride(a.dv), row_stride(a.D)));
     take_row_pairs_host(cv, cap); cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
     cv.take(kSlack);
+    cv.at_least(kGradScratch);
     return cv.bytes();
 }
 size_t smem_bwd_key(const AttnArgs &a, int cap) {
@@ -618,6 +637,7 @@ size_t smem_bwd_key(const AttnArgs &a, int cap) {
     take_rows_host(cv, cap, a.d); take_rows_host(cv, cap, a.dv); take_rows_host(cv, cap, a.D);
     take_rows_host(cv, cap, a.D);
     cv.take(cap * a.M); cv.take(cap * a.M); cv.take(cap * du_stride(a.M));
+    cv.at_least(kGradScratch);
     return cv.bytes();
 }
 
@@ -691,22 +711,19 @@ cudaError_t fwd_impl(const AttnArgs &a, cudaStream_t s) {
 template <typename IO>
 cudaError_t bwd_impl(const AttnArgs &a0, bool have_stats, cudaStream_t s) {
     AttnArgs a = a0;
-    a.gpart64 = 1;  // the generic kernels write fp64 parameter-gradient sums
     cudaError_t e;
     if (!have_stats && (e = stats_impl<IO>(a, s)) != cudaSuccess) return e;
     const int BH = a.B * a.H;
     const int cap = pick_cap(BH, a.n, [&](int c) { return std::max(smem_bwd_query(a, c), smem_bwd_key(a, c)); });
     const Range r = split_rows(BH, a.n, cap, a.nsplit_b);
-    const int64_t slots = 2 * (int64_t)BH * a.nsplit_b;
     a.nsplit_b = r.splits;
     a.rows_per_split_b = r.rows;
-    const int nbuf = grad_buffers(BH * (int64_t)r.splits, slots);
-    if ((e = cudaMemsetAsync(a.gpart, 0, (size_t)nbuf * a.gsize * sizeof(double), s)) != cudaSuccess) return e;
+    if ((e = place_grads(a, BH * (int64_t)r.splits, s)) != cudaSuccess) return e;
     size_t sm = smem_bwd_query(a, cap);
     outer_dispatch(a.D, a.dv, [&](auto tf, auto tc) {
         auto k = k_bwd_query<IO, decltype(tf)::value, decltype(tc)::value>;
         if ((e = set_smem(k, sm)) != cudaSuccess) return;
-        LUNA_LAUNCH("bwd_query", k, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, nbuf, a.nsplit_b <= kFinishParts);
+        LUNA_LAUNCH("bwd_query", k, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, a.nsplit_b <= kFinishParts);
         e = cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
@@ -720,10 +737,10 @@ cudaError_t bwd_impl(const AttnArgs &a0, bool have_stats, cudaStream_t s) {
     if ((e = launch_chrms_dstate(a, s)) != cudaSuccess) return e;
     sm = smem_bwd_key(a, cap);
     if ((e = set_smem(k_bwd_key<IO>, sm)) != cudaSuccess) return e;
-    LUNA_LAUNCH("bwd_key", k_bwd_key<IO>, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, nbuf);
+    LUNA_LAUNCH("bwd_key", k_bwd_key<IO>, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     int nparts = 0;
-    if ((e = launch_chrms_backward(a, nbuf, &nparts, s)) != cudaSuccess) return e;
+    if ((e = launch_chrms_backward(a, 0, &nparts, s)) != cudaSuccess) return e;
     return launch_grad_reduce(a, nparts, s);
 }
 
@@ -748,16 +765,18 @@ cudaError_t launch_grad_reduce(const AttnArgs &a, int nparts, cudaStream_t s) {
     const int nb = (a.gsize + kSumElems - 1) / kSumElems;
     const bool dep = !a.ch_sigma;
     if (a.gpart64)
-        LUNA_LAUNCH_DEP("grad_sum", dep, k_grad_sum<double>, nb, kSumElems * kSumSplit, 0, s,
-                        reinterpret_cast<const double *>(a.gpart), nparts, a.gsize, a.hist);
+        LUNA_LAUNCH_DEP("grad_sum", dep, k_grad_sum64, (a.gsize + kSum64Elems - 1) / kSum64Elems,
+                        kSum64Elems * kSum64Split, 0, s, static_cast<const double *>(a.gw), a.gw_n,
+                        static_cast<const double *>(a.gh), a.gh_n, reinterpret_cast<const double *>(a.gpart), nparts,
+                        a.M * a.d + a.M, a.gsize, a.hist);
     else
-        LUNA_LAUNCH_DEP("grad_sum", dep, k_grad_sum<float>, nb, kSumElems * kSumSplit, 0, s,
+        LUNA_LAUNCH_DEP("grad_sum", dep, k_grad_sum, nb, kSumElems * kSumSplit, 0, s,
                         static_cast<const float *>(a.gpart), nparts, a.gsize, a.hist);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if ((e = launch_chrms_hist(a, s)) != cudaSuccess) return e;
     // the partials have been summed: their buffer holds the shared MLP's per-channel fc1 terms
-    double *fc1_part = reinterpret_cast<double *>(a.gpart);
+    double *fc1_part = a.gpart64 ? a.gw : reinterpret_cast<double *>(a.gpart);
     LUNA_LAUNCH_DEP("mlp_grads", dep, k_mlp_grads, a.lay.L + 1, 128, 0, s, a.lay, a.table,
                     static_cast<const double *>(a.hist), a.grads, fc1_part);
     if ((e = cudaGetLastError()) != cudaSuccess || !a.lay.shared || a.lay.act) return e;

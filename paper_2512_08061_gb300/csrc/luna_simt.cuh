@@ -21,9 +21,11 @@ struct AttnArgs {
     // backward
     int nsplit_b, rows_per_split_b;
     float *dS_part, *dz_part, *dS_fin, *dz_fin;
-    float *gpart;                      // [2 * BH * nsplit_b][gsize] parameter-gradient partials (fp32, or
-                                       // fp64 when gpart64: the generic kernels)
+    float *gpart;                      // [2 * BH * nsplit_b][gsize] parameter-gradient partials (fp32; fp64 when
+                                       // gpart64: the channel normalisation's beside the generic kernels')
     int gpart64;                       // 1: the partials are doubles
+    double *gw, *gh;                   // generic kernels: dW, db of every block [gw_n][M*d + M], in a fixed place each,
+    int gw_n, gh_n;                    // and gh_n histograms (with the variants' sums) that the blocks share
     int gsize;                         // M*d + M + nint*L*2
     double *hist;                      // [gsize] the partials' sum: dW, db, then the histogram [nint][L][2]
     luna_phi_grads grads;

@@ -33,6 +33,7 @@ __device__ __forceinline__ bool carve_fits(const Carve &cv, const float *base) {
 struct HostCarve {
     int n = 0;
     void take(int k) { n += r4(k); }
+    void at_least(int k) { n = n > k ? n : k; }
     size_t bytes() const { return (size_t)n * 4; }
 };
 

@@ -59,11 +59,20 @@ void outer_dispatch(int D, int dv, F f) {
     else f(std::integral_constant<int, 4>{}, std::integral_constant<int, 8>{});
 }
 
-// Parameter-gradient sums (fp64, zeroed by the caller) that the blocks of a backward pass share, block b adding
-// to buffer b mod count: one per SM keeps the reductions of concurrent blocks apart, and their zeroing and final
-// sum at 152 x 70 KB instead of a buffer per block.
-inline int grad_buffers(int64_t blocks, int64_t room) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(blocks, kSMs), room));
+// Parameter gradients of the generic backward kernels, in the partials' buffer of 2 * blocks * gsize doubles
+// (`blocks`: of one of the two kernels at most): dW and db of every block of both in a slot of its own, so that
+// they are summed in a fixed order, and before the channel normalisation's partials (a.gpart from here on) the
+// histograms.  These are the large part and are added to by L2 reductions: the blocks share one per SM, which
+// keeps the reductions of concurrent blocks apart and their zeroing and sum at 152 x 70 KB instead of one per block.
+inline cudaError_t place_grads(AttnArgs &a, int64_t blocks, cudaStream_t s) {
+    const int nw = a.M * a.d + a.M, nh = a.gsize - nw;
+    a.gpart64 = 1;
+    a.gw = reinterpret_cast<double *>(a.gpart);
+    a.gw_n = (int)(2 * blocks);
+    a.gh = a.gw + (size_t)a.gw_n * nw;
+    a.gh_n = (int)std::min<int64_t>(blocks, kSMs);
+    a.gpart = reinterpret_cast<float *>(a.gh + (size_t)a.gh_n * nh);
+    return cudaMemsetAsync(a.gh, 0, (size_t)a.gh_n * nh * sizeof(double), s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1235,19 +1244,36 @@ __device__ void store_dx_rows(const TableLayout &lay, const SmemPhi &s, const fl
     }
 }
 
-// Adds dW and db to the fp64 sums gp = [dW | db | histogram].
-__device__ void add_grad_tile(const TableLayout &lay, const GradTile &g, double *gp) {
+// dW and db of the block into its slot [dW | db]: the groups' pairs, added in a tree of fixed shape in `scratch`
+// (kGradScratch floats of shared memory that nothing else uses any more).  Called by every thread.
+constexpr int kGradScratch = 2 * 8 * kThr;
+__device__ void store_grad_tile(const TableLayout &lay, GradTile &g, float *scratch, double *slot) {
     const int M = lay.M, d = lay.d, nc = (d + 3) / 4, nt = ((M + 1) / 2) * nc;
     const int G = kThr / nt, grp = threadIdx.x / nt, t = threadIdx.x - grp * nt;
-    if (grp < G) {
+    float2 *sc = reinterpret_cast<float2 *>(scratch);
+    __syncthreads();
+    int s = 1;
+    while (s < G) s *= 2;
+    for (s /= 2; s >= 1; s /= 2) {  // groups s .. 2 s - 1 hand their pairs to groups 0 .. s - 1
+        if (grp >= s && grp < 2 * s)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sc[k * kThr + threadIdx.x] = make_float2(g.h[k / 4][k % 4], g.l[k / 4][k % 4]);
+        __syncthreads();
+        if (grp < s && grp + s < G)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float2 v = sc[k * kThr + threadIdx.x + s * nt];
+                pair_add(g.h[k / 4][k % 4], g.l[k / 4][k % 4], v.x, v.y);
+            }
+    }
+    if (grp == 0) {
         const int i0 = 2 * (t / nc), c0 = 4 * (t % nc);
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int m = 0; m < 4; ++m)
-                if (i0 + i < M && c0 + m < d) atomicAdd(gp + (i0 + i) * d + c0 + m, pair_double(g.h[i][m], g.l[i][m]));
+        for (int k = 0; k < 8; ++k)
+            if (i0 + k / 4 < M && c0 + k % 4 < d)
+                slot[(i0 + k / 4) * d + c0 + k % 4] = pair_double(g.h[k / 4][k % 4], g.l[k / 4][k % 4]);
     }
-    if ((int)threadIdx.x < M) atomicAdd(gp + M * d + threadIdx.x, pair_double(g.bh, g.bl));
+    if ((int)threadIdx.x < M) slot[M * d + threadIdx.x] = pair_double(g.bh, g.bl);
 }
 
 }  // namespace
