@@ -124,6 +124,7 @@ luna_status make_plan(const luna_attn_desc *ad, const luna_phi_desc *pd, Plan &p
     }
     const size_t f = sizeof(float);
     const size_t SD = (size_t)D * dv;
+    p.tc = tc_plan(*ad, p.lay);
     Bump w;
     p.o_status = w.take(sizeof(int));  // offset 0: device status word of the last call
     p.o_counters = w.take(2 * (size_t)BH * sizeof(int));
@@ -175,14 +176,15 @@ luna_status make_plan(const luna_attn_desc *ad, const luna_phi_desc *pd, Plan &p
         p.o_dzpart = w.take((size_t)BH * ns * D * f);
         p.o_segdS = w.take((size_t)BH * ns * SD * f);
         p.o_segdz = w.take((size_t)BH * ns * D * f);
-        p.o_rowstat = w.take((size_t)BH * n * 4 * f);
+        // den and dden of every row: floats (tensor cores) or pairs (generic kernels; in a plan for the tensor
+        // cores, whose inputs turn out not to be aligned, these lie in dphi's place)
+        p.o_rowstat = w.take((size_t)BH * n * (p.tc.causal_bwd ? 2 : 4) * f);
         p.o_gpart = w.take((2 * (size_t)BH * ns + (p.ch_target > 0.0f ? 2 * kChKBlocks : 0)) * p.gsize *
                            sizeof(double));
         p.o_hist = w.take((size_t)p.gsize * sizeof(double));
         p.ws_bwd = w.n;
         p.state_bytes = (size_t)BH * (ns + 1) * (SD + D) * f;
     }
-    p.tc = tc_plan(*ad, p.lay);
     if (p.tc.eligible) {
         p.ws_fwd = std::max(p.ws_fwd, p.tc.ws_fwd);
         p.ws_bwd = std::max(p.ws_bwd, p.tc.ws_bwd);
@@ -479,13 +481,15 @@ luna_status luna_attn_bwd(const luna_attn_desc *ad, const luna_phi_desc *pd, con
     }
     const int nsub = pd->param_head_stride ? ad->H : 1;  // per-head parameters: one sub-problem per head index
     for (int h = 0; h < nsub; ++h) {
-        const AttnArgs b = pd->param_head_stride ? head_args(a, ad, pd, p, h) : a;
+        AttnArgs b = pd->param_head_stride ? head_args(a, ad, pd, p, h) : a;
         if (ad->causal) {
             if (p.tc.causal_bwd && tc_inputs_ok(TcPlan{true}, b.Q, b.K, b.V, b.dO) &&
-                tc_inputs_ok(TcPlan{true}, b.dQ, b.dK, b.dV, nullptr))
+                tc_inputs_ok(TcPlan{true}, b.dQ, b.dK, b.dV, nullptr)) {
                 e = launch_tc_causal_bwd(b, state != nullptr, s);
-            else
+            } else {
+                if (p.tc.causal_bwd) b.rowstat = b.dphi;
                 e = launch_causal_bwd(b, ad->io, state != nullptr, s);
+            }
         } else if (p.tc.eligible && tc_inputs_ok(p.tc, b.Q, b.K, b.V, b.dO) &&
                    tc_inputs_ok(p.tc, b.dQ, b.dK, b.dV, nullptr)) {
             e = launch_tc_bwd(p.tc, b, w, state != nullptr, s);

@@ -34,7 +34,7 @@ struct AttnArgs {
     float *seg_S, *seg_z;              // [BH][nseg+1][D][dv], [BH][nseg+1][D]: prefix at each segment start, total last
     float *seg_dS, *seg_dz;            // [BH][nseg][D][dv], [BH][nseg][D]: suffix after segment end
     float *rowstat;                    // backward pass, per row: [BH][n][4] den_i and dden_i as pairs
-                                       // (tensor cores: [BH][n][2])
+                                       // (tensor cores: [BH][n][2] floats)
     // streaming-form backward on tensor cores
     float *dphi;                       // [BH][n][D] fp32: dLoss/dphi of Q, then of K
     void *phik, *pq2;                  // [BH][n][2D] bf16 phi(k), phi(q)/den, each as (hi | lo)
