@@ -281,11 +281,17 @@ class Luna:
         self.ws = alloc_bytes(max(luna_workspace_size(self.ad, self.pd, False),
                                   luna_workspace_size(self.ad, self.pd, True)), self.device)
         self.state = alloc_bytes(luna_state_size(self.ad, self.pd), self.device)
-        self._final = None
-        if causal and self.state.data_ptr() and B and H and n:  # where the final S, z lie in any state buffer
+        self._final = (None, None)  # descriptors (by value), place of the final S, z in a state buffer
+
+    def _final_state(self) -> tuple[int, int, int, int]:
+        """luna_state_final of this object's state buffer.  The place of S and z depends on the descriptors alone: it is
+        kept with their bytes (0.3 us to compare, the call takes 2) and looked up again when either has changed."""
+        key, at = bytes(self.ad) + bytes(self.pd), self.state.data_ptr()
+        if key != self._final[0] or not at:
             S, Ss, z, zs = luna_state_final(self.ad, self.pd, self.state)
-            at = self.state.data_ptr()
-            self._final = (S - at, Ss, z - at, zs)
+            self._final = (key, (S - at, Ss, z - at, zs))
+        S, Ss, z, zs = self._final[1]
+        return at + S, Ss, at + z, zs
 
     def prepare(self, params: dict, stream=None):
         """params: W, b, w1, b1, w2, b2 device tensors (with a leading head axis for per-head parameters),
@@ -328,11 +334,6 @@ class Luna:
         (saved with save_state=True), which it advances in place.  q, k: (B, H, d); v: (B, H, dv)."""
         if o is None:
             o = torch.empty(q.shape[:-1] + (self.ad.dv,), dtype=q.dtype, device=q.device)
-        if self._final is None:
-            S, Ss, z, zs = luna_state_final(self.ad, self.pd, self.state)
-        else:
-            at = self.state.data_ptr()
-            S, Ss, z, zs = self._final
-            S, z = at + S, at + z
+        S, Ss, z, zs = self._final_state()
         luna_attn_decode(self.ad, self.pd, self.table, q, k, v, o, S, Ss, z, zs, stream)
         return o
