@@ -143,8 +143,8 @@ luna_status make_plan(const luna_attn_desc *ad, const luna_phi_desc *pd, Plan &p
         }
         p.ws_fwd = w.n;
         // per-head partial slots: generic splits, or (tensor-core path) runs of work items, never more
-        // than the forward split count; the generic kernels' partials are pairs
-        const size_t nslot = (size_t)std::max(p.nsplit, 2 * p.nsplit_b);
+        // than the forward split count; the generic kernels' partials are pairs where a head has several
+        const size_t nslot = (size_t)std::max(p.nsplit, p.nsplit_b > 1 ? 2 * p.nsplit_b : 1);
         p.o_dSpart = w.take((size_t)BH * nslot * SD * f);
         p.o_dzpart = w.take((size_t)BH * nslot * D * f);
         p.o_dSfin = w.take((size_t)BH * SD * f);

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kThr, 1) k_query(AttnArgs a, int cap, int rows
 //   dphi(q_i) = S dnum_i + z dden_i,  dS += phi(q_i) dnum_i^T,  dz += phi(q_i) dden_i
 // den, the sum dnum_i . num_i and dden are pairs (RowPairs), dphi is a pair rounded once.
 template <typename IO, int TF, int TC>
-__global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int finish) {
+__global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int pairs, int finish) {
     extern __shared__ __align__(16) float smem[];
     Carve cv{smem};
     const TableLayout &lay = a.lay;
@@ -263,10 +263,10 @@ __global__ void __launch_bounds__(kThr, 1) k_bwd_query(AttnArgs a, int cap, int 
         phi_backward_rows(lay, s, sQ, nr, cap, sPhi, sdPhi, sU, sJ, sdU, hist, hist + mlp_words(lay), g);
         store_dx_rows(lay, s, sdU, nr, dQ + (size_t)t0 * d);
     }
-    acc.store(D, dv, a.dS_part, a.dz_part, slot, true);
+    acc.store(D, dv, a.dS_part, a.dz_part, slot, pairs != 0);
     store_grad_tile(lay, g, smem, a.gw + slot * (M * d + M));
     if (finish && last_arrival(a.counters + a.B * a.H + bh, a.nsplit_b)) {
-        const int np = 2 * a.nsplit_b;
+        const int np = pairs ? 2 * a.nsplit_b : a.nsplit_b;
         ordered_sum(a.dS_part + (size_t)bh * np * D * dv, np, D * dv, a.dS_fin + (size_t)bh * D * dv);
         ordered_sum(a.dz_part + (size_t)bh * np * D, np, D, a.dz_fin + (size_t)bh * D);
         if (threadIdx.x == 0) a.counters[a.B * a.H + bh] = 0;
@@ -720,10 +720,11 @@ cudaError_t bwd_impl(const AttnArgs &a0, bool have_stats, cudaStream_t s) {
     a.rows_per_split_b = r.rows;
     if ((e = place_grads(a, BH * (int64_t)r.splits, s)) != cudaSuccess) return e;
     size_t sm = smem_bwd_query(a, cap);
+    const int pairs = a.nsplit_b > 1;  // a single partial is the sum itself, rounded once either way
     outer_dispatch(a.D, a.dv, [&](auto tf, auto tc) {
         auto k = k_bwd_query<IO, decltype(tf)::value, decltype(tc)::value>;
         if ((e = set_smem(k, sm)) != cudaSuccess) return;
-        LUNA_LAUNCH("bwd_query", k, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, a.nsplit_b <= kFinishParts);
+        LUNA_LAUNCH("bwd_query", k, dim3(a.nsplit_b, BH), kThr, sm, s, a, cap, pairs, a.nsplit_b <= kFinishParts);
         e = cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
