@@ -282,6 +282,8 @@ class Luna:
                                   luna_workspace_size(self.ad, self.pd, True)), self.device)
         self.state = alloc_bytes(luna_state_size(self.ad, self.pd), self.device)
         self._final = (None, None)  # descriptors (by value), place of the final S, z in a state buffer
+        if causal and B and H and n and self.state.data_ptr():
+            self._final_state()  # not left to the first decode step
 
     def _final_state(self) -> tuple[int, int, int, int]:
         """luna_state_final of this object's state buffer.  The place of S and z depends on the descriptors alone: it is

@@ -40,3 +40,10 @@ def test_decode_follows_changed_descriptors(L, monkeypatch):
     with pytest.raises(L.LunaError) as e:
         check()
     assert e.value.status == 1
+
+
+def test_first_decode_looks_nothing_up(L, monkeypatch):
+    """The place of the state is found with the object, not by its first decode step."""
+    lu = L.Luna(1, 2, 100, 16, 16, 4, 4, 8, True, 1e-6, device="cpu")
+    monkeypatch.setattr(L, "luna_state_final", lambda *a: pytest.fail("looked up in the decode call"))
+    _decoded(L, lu, monkeypatch)
