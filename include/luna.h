@@ -166,8 +166,8 @@ typedef struct {
  * causal = 1 selects the streaming form (sums over j <= i).  chunk (0, or
  * 16..128 in steps of 16, else LUNA_ERR_INVALID_ARG) is accepted for the
  * interface and otherwise not used: the kernels choose their own tiles (128
- * rows in the tensor-core streaming forward, 64 in its backward, 16 in the
- * generic kernels), and results do not depend on it beyond rounding order.
+ * rows in the tensor-core streaming forward, 64 in its backward, 8 to 64 in
+ * the generic kernels), and results do not depend on it beyond rounding order.
  * eps >= 0 guards the row normaliser: O_i = num_i / (den_i + eps); a row
  * whose guarded normaliser is exactly 0 produces O_i = 0 and zero gradients. */
 typedef struct {
@@ -259,9 +259,9 @@ luna_status luna_attn_bwd(const luna_attn_desc *ad, const luna_phi_desc *pd, con
  * ignored); A: fp32 device array (B, H, rows, n), every entry written.
  * 0 <= row0, 0 <= rows, row0 + rows <= n, else LUNA_ERR_INVALID_ARG;
  * pd->ch_rms_target > 0 gives LUNA_ERR_UNSUPPORTED.  No workspace: each block
- * of 32 rows writes its raw scores and normalises them in a second pass over
- * its own rows.  The feature map is fp32 for both io types; each row's sum
- * is accumulated in fp64. */
+ * writes the raw scores of its rows and normalises them in a second pass.  The
+ * feature map is fp32 for both io types; each row's sum of kernel values is
+ * accumulated as a pair of floats. */
 luna_status luna_attn_weights(const luna_attn_desc *ad, const luna_phi_desc *pd, const void *table, const void *Q,
                               const void *K, const int32_t *lengths, int row0, int rows, int teacher, float *A,
                               void *stream);

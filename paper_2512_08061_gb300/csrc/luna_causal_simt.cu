@@ -28,8 +28,8 @@ namespace {
 using namespace simt;
 
 // Measured at 8 x 12 heads of 1024 bf16 rows, d = D = 64 (us; before: fp64 sums, tiles of 16 rows, and separate
-// sweeps for the segment sums and dQ): outputs 5918 -> 326, backward queries 16081 -> 937, backward keys
-// 6861 -> 606, with the key statistics 2715 -> 177.
+// sweeps for the segment sums and dQ): outputs 5918 -> 389, backward queries 16081 -> 1123, backward keys
+// 6861 -> 743, with the key statistics 2715 -> 211.
 //
 // Each kernel walks its segment in tiles of `cap` rows (luna_tile.cuh).  The running state is held in fp32 in
 // shared memory and advances once per tile from pairs of floats, so a tile of 64 rows rounds it a quarter as

@@ -11,9 +11,9 @@
 //
 // Measured at 8 x 12 heads of 512 fp32 rows, d = D = 64 (us; before: fp64 sums in
 // tiles of 16 or 32 rows, 64 of 256 threads in the outer products):
-//   key statistics 1402 -> 121, queries 161 -> 54, backward queries 3848 -> 300,
-//   backward keys 1451 -> 151, gradient sum 30 -> 8.
-// The fma pipe is 30 to 35 % busy and the issue slots about half: what is left is
+//   key statistics 1402 -> 135, queries 161 -> 53, backward queries 3848 -> 336,
+//   backward keys 1451 -> 162, gradient sum 30 -> 14.
+// The fma pipe is 33 to 38 % busy and the issue slots half: what is left is
 // barriers between a tile's phases, the feature map's gathers and the histogram.
 #include <math.h>
 

@@ -44,8 +44,8 @@ struct SmemPhi {
     float *T, *AB, *W, *b;
     float *w1, *b1, *w2, *b2;  // channel MLPs (non-ReLU activation)
     float *We, *be, *coef;     // envelope gate, Bank+Coef coefficients
-    float *E, *H, *dE;         // [kPhiRows][L] per row: e_l = h_l c_l, the gate h_l, dLoss/de_l (then the gate's
-                               // pre-activation gradient)
+    float *E, *H, *dE;         // [cap][L], a row for each of the kernel's tile: e_l = h_l c_l, the gate h_l, dLoss/de_l
+                               // (then the gate's pre-activation gradient)
 };
 
 // The (alpha, beta) table into shared memory at ab_stride(lay) words per interval.

@@ -197,7 +197,8 @@ __device__ void load_tile(const Rows &t, const IO *src, int nr, int w, int cap) 
 // The feature map over a tile.
 
 // Shared memory of the feature map (the generic SmemPhi, with the projection rows padded and the bucketed
-// search block in place of the kinks alone).
+// search block in place of the kinks alone).  cap: the rows that phi_rows is called with, for the gate's and the
+// coefficients' factors of each; 0 only where the map has neither.
 __device__ SmemPhi carve_phi_tile(Carve &cv, const TableLayout &lay, int cap) {
     SmemPhi s = {};
     if (!lay.act) {
